@@ -258,10 +258,11 @@ int dm_sp2_bsr(tb_ctx* ctx, const double* H, int n, double nocc, const tb_sp2_op
                size_t ws_bytes, tb_sp2_report* rep, cudaStream_t s);
 
 // Encode a 2D row-major tensor map over an ld x ld operand array (gemm_tc.cu):
-// boxes of box_rows (64 or 128) rows of row_bytes (64 or 128) bytes, swizzled
+// boxes of box_rows (32, 64 or 128) rows of row_bytes (64 or 128) bytes, swizzled
 // to the row width.  The projection and Fermi-product kernels read 128-row
-// boxes of sp2_tc_row_bytes(); the emulated-FP64 product reads 128-byte rows,
-// in 64-row boxes for the B operand of its CTA-pair form.
+// boxes of sp2_tc_row_bytes(), and the single-launch forms B boxes of their unit
+// width; the emulated-FP64 product reads 128-byte rows, in 64-row boxes for the B
+// operand of its CTA-pair form.
 int sp2_tc_make_map(tb_ctx* ctx, int precision, const void* base, int ld, CUtensorMap* map, int row_bytes = 128,
                     int box_rows = 128);
 int sp2_tc_row_bytes();

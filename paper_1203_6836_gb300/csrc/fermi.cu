@@ -51,7 +51,7 @@
 // dTr D/dmu = beta Tr[D(I - D)] inside a bisection bracket, one full
 // expansion per step; every decision is taken on the device.
 
-#include "common.cuh"
+#include "foe.cuh"
 
 #include <algorithm>
 #include <math.h>
@@ -59,39 +59,11 @@
 namespace {
 
 constexpr int kTile = 128;
-constexpr int kMaxMu = 40;
-constexpr int kMaxM = 40;   // doubling steps issued at most
+constexpr int kMaxMu = kFoeMaxMu;
+constexpr int kMaxM = kFoeMaxM;  // doubling steps issued at most
 constexpr int kMinM = 8;    // doubling steps used at least
-constexpr int kMats = 7;    // E0/E1 (the iterate, alternating), A, Z, T, Y, W
-// Canonical shift: the last expansion is accepted and shifted by u = beta dmu
-// to second order,
-//   D(mu + dmu) = D + u D(I - D) + u^2/2 D(I - D)(I - 2D) + R,
-// with D(I - D) = W/4 and D(I - D)(I - 2D) = -E W/2, W = (I - 2E)(I + 2E) (two
-// products, W and E W, after every expansion), u the root of the trace condition
-// Tr D + u Tr[D(I-D)] + u^2/2 Tr[D(I-D)(I-2D)] = N_occ near -(Tr D - N)/Tr[D(I-D)].
-// The remainder involves the third derivative beta^3 f(1-f)(1-6f+6f^2), whose
-// last factor is at most 1 in magnitude, so ||R||_F <= |u|^3/6 Tr[D(I - D)]
-// (D(I - D) is positive semi-definite with eigenvalues <= 1/4).  The shift
-// replaces another expansion when that bound is below kCorrFro sqrt(n) and
-// |u| <= kCorrMax.
-constexpr double kCorrFro = 1e-7;
-constexpr double kCorrMax = 0.1;
-
+constexpr int kMats = kFoeMats;  // E0/E1 (the iterate, alternating), A, Z, T, Y, W
 inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
-
-struct FoeState {
-  double mu, lo, hi;
-  double emin, emax;
-  int done, iters, capped, err;
-  int ran;     // 1: the last k_foe_mu evaluated an expansion (it was not skipped)
-  int nocorr;  // 0: apply the canonical shift u to the last expansion
-  double dmu;  // u / beta
-  double u;
-  double c;    // start scale beta / 2^{meff+2}
-  int meff;    // doubling steps used
-  int skipd[kMaxM];  // 1: doubling step k returns at once (k < m_max - meff, or done)
-  double tr[kMaxMu + 1], trdd[kMaxMu + 1], mus[kMaxMu + 1];
-};
 
 struct Mat {
   float* m;
@@ -177,44 +149,7 @@ __global__ void k_foe_mu(FoeState* st, const double* parts, const double* partsw
   y = warp_sum(y);  // Tr W
   z = warp_sum(z);  // Tr E W
   if (threadIdx.x != 0) return;
-  const int it = st->iters;
-  const double mu = st->mu;
-  const double trd = 0.5 * n + x;
-  const double t1 = 0.25 * y;    // Tr D(I - D)
-  const double t2 = -0.5 * z;    // Tr D(I - D)(I - 2D)
-  st->tr[it] = trd;
-  st->trdd[it] = t1;
-  st->mus[it] = mu;
-  st->iters = it + 1;
-  st->ran = 1;
-  const double dev = trd - nocc;
-  const double step = t1 > 1e-12 ? -dev / (beta * t1) : NAN;  // Newton step on mu
-  double u = beta * step;
-  for (int k = 0; k < 3 && isfinite(u); ++k) {  // root of dev + t1 u + t2 u^2/2 near the Newton step
-    const double g = dev + u * (t1 + 0.5 * t2 * u), gp = t1 + t2 * u;
-    if (!(gp > 0.0)) break;
-    u -= g / gp;
-  }
-  const bool shift = isfinite(u) && fabs(u) <= kCorrMax &&
-                     fabs(u) * u * u / 6.0 * t1 <= kCorrFro * sqrt((double)max(n, 1));
-  if (shift) {
-    // accept this expansion with the second-order shift to mu + u / beta
-    st->done = 1;
-    st->nocorr = 0;
-    st->u = u;
-    st->dmu = u / beta;
-    st->tr[it] = trd + u * (t1 + 0.5 * t2 * u);
-    st->mus[it] = mu + u / beta;
-  } else if (fabs(dev) <= tol) {
-    st->done = 1;
-  } else if (it + 1 >= max_it) {
-    st->done = 1;
-    st->capped = 1;
-  } else {
-    if (dev < 0.0) st->lo = mu;
-    else st->hi = mu;
-    st->mu = foe_next_mu(mu, dev, t1, beta, tol, st->lo, st->hi);
-  }
+  foe_mu_step(st, x, y, z, n, nocc, beta, tol, max_it);
   if (st->done)
     for (int k = 0; k < kMaxM; ++k) st->skipd[k] = 1;
   if (cond && st->done) cudaGraphSetConditional(handle, 0);
@@ -268,15 +203,12 @@ __global__ void __launch_bounds__(256) k_foe_keep(const FoeState* st, size_t cou
 __global__ void __launch_bounds__(256) k_foe_correct(const FoeState* st, int n, int ld, const float* __restrict__ T,
                                                      const float* __restrict__ U, float* __restrict__ E) {
   if (st->nocorr) return;
-  const float u = (float)st->u, h = 0.5f * u * u;
+  const float u = (float)st->u;
   const size_t total = (size_t)n * n;
   for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
     const int r = (int)(e / n), col = (int)(e % n);
     const size_t i = (size_t)r * ld + col;
-    const float x = E[i];
-    const float first = 0.25f * T[i];
-    const float second = -0.5f * U[i];
-    E[i] = fmaf(h, second, fmaf(u, first, x));
+    E[i] = foe_shifted(E[i], T[i], U[i], u);
   }
 }
 
@@ -288,22 +220,7 @@ __global__ void __launch_bounds__(256) k_foe_finalize(const FoeState* st, int n,
     const int r = (int)(e / n), c = (int)(e % n);
     D[e] = (double)X[(size_t)r * ld + c] + (r == c ? 0.5 : 0.0);
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    const int it = st->iters > 0 ? st->iters - 1 : 0;
-    const double mu = st->mus[it];
-    if (mu_out) *mu_out = mu;
-    if (rep) {
-      rep->status = st->err ? st->err : (fabs(st->tr[it] - nocc) <= tol ? TB_OK : TB_ERR_NOT_CONVERGED);
-      rep->mu_iters = st->iters;
-      rep->m = st->meff;
-      rep->n = n;
-      rep->mu = mu;
-      rep->trace = st->tr[it];
-      rep->trace_dd = st->trdd[it];
-      rep->eps_min = st->emin;
-      rep->eps_max = st->emax;
-    }
-  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) foe_report(st, st->err, n, nocc, tol, mu_out, rep);
 }
 
 struct FoeLayout {
@@ -374,14 +291,6 @@ extern "C" int dm_fermi(tb_ctx* ctx, const double* H, int n, double nocc, double
     M[i].m = reinterpret_cast<float*>(base + L.off_mat[i][0]);
     M[i].hi = base + L.off_mat[i][1];
     M[i].lo = L.off_mat[i][2] ? base + L.off_mat[i][2] : nullptr;
-    int rc = sp2_tc_make_map(ctx, o->precision, M[i].hi, L.ld, &M[i].mh, sp2_tc_row_bytes());
-    if (rc) return rc;
-    if (M[i].lo) {
-      rc = sp2_tc_make_map(ctx, o->precision, M[i].lo, L.ld, &M[i].ml, sp2_tc_row_bytes());
-      if (rc) return rc;
-    } else {
-      M[i].ml = M[i].mh;
-    }
   }
   const double beta = 1.0 / kT;
   // at most m doubling steps (m = 14: beta (hi - lo) <= 32768); the device uses
@@ -403,8 +312,42 @@ extern "C" int dm_fermi(tb_ctx* ctx, const double* H, int n, double nocc, double
   k_foe_bounds<<<1, 32, 0, s>>>(bparts, (n + 7) / 8, st, mu, kT, m);
   TB_LAUNCH_CHECK(ctx);
 
-  // the chemical-potential loop: a while graph node under capture, else
-  // mu_iters unrolled rounds that return at once after the stop decision
+  // tf32 and tf32x3: the whole expansion loop in one launch; a captured call whose matrix is too
+  // large for one cluster instead takes the launched form below, whose
+  // chemical-potential loop is a while graph node
+  {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    TB_CUDA_TRY(ctx, cudaStreamIsCapturing(s, &cs));
+    FoeRunArgs a{};
+    a.H = H;
+    a.D = D;
+    a.mu_out = mu;
+    a.rep = rep;
+    a.st = st;
+    for (int i = 0; i < kMats; ++i) {
+      a.m[i] = M[i].m;
+      a.hi[i] = M[i].hi;
+      a.lo[i] = M[i].lo;
+    }
+    a.parts = parts;
+    a.partsw = partsw;
+    a.parts3 = parts3;
+    a.n = n;
+    a.ld = L.ld;
+    a.ns = ns;
+    a.max_it = o->mu_iters;
+    a.nocc = nocc;
+    a.beta = beta;
+    a.tol = tol;
+    a.wait_ns = ctx->wait_ns;
+    int ran = 0;
+    if ((rc = foe_run(ctx, o->precision, a, cs != cudaStreamCaptureStatusNone, &ran, s)) || ran) return rc;
+  }
+  for (int i = 0; i < kMats; ++i) {
+    if ((rc = sp2_tc_make_map(ctx, o->precision, M[i].hi, L.ld, &M[i].mh, sp2_tc_row_bytes()))) return rc;
+    M[i].ml = M[i].mh;
+    if (M[i].lo && (rc = sp2_tc_make_map(ctx, o->precision, M[i].lo, L.ld, &M[i].ml, sp2_tc_row_bytes()))) return rc;
+  }
   DevLoop loop;
   if ((rc = tb_loop_begin(ctx, s, &loop))) return rc;
   cudaStream_t ls = loop.body_stream;

@@ -753,7 +753,7 @@ int sp2_tc_make_map(tb_ctx* ctx, int precision, const void* base, int ld, CUtens
                     int box_rows) {
   if (!ctx->encode_tiled) return tb_fail(ctx, TB_ERR_UNSUPPORTED, "cuTensorMapEncodeTiled unavailable");
   if (row_bytes != 64 && row_bytes != 128) return tb_fail(ctx, TB_ERR_ARG, "tile row of %d bytes", row_bytes);
-  if (box_rows != 64 && box_rows != 128) return tb_fail(ctx, TB_ERR_ARG, "tile of %d rows", box_rows);
+  if (box_rows != 32 && box_rows != 64 && box_rows != 128) return tb_fail(ctx, TB_ERR_ARG, "tile of %d rows", box_rows);
   const bool tf = precision == TB_PREC_TF32 || precision == TB_PREC_TF32X3;
   const size_t eb = tf ? 4 : 2;
   const cuuint64_t dims[2] = {(cuuint64_t)ld, (cuuint64_t)ld};

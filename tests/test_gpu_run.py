@@ -1,0 +1,77 @@
+"""The single-launch form of dm_fermi: tile
+edges, every unit width, cut last rounds, one cluster and a cooperative grid."""
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import density
+from paper_1203_6836_gb300 import tbmd
+from paper_1203_6836_gb300.device import FermiSolver, fermi_opts, fermi_report_to_dict
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = tbmd.Context()
+    yield c
+    c.close()
+
+
+def _banded(n, seed):
+    """A symmetric matrix with a 2 eV gap in its middle and a spectral width of ~14 eV."""
+    rng = np.random.default_rng(seed)
+    H = np.diag(np.where(np.arange(n) < n // 2, -4.0, 4.0) + rng.uniform(-1, 1, n))
+    for k in (1, 2, 5):
+        if k < n:
+            H += np.diag(rng.uniform(-0.3, 0.3, n - k), k) + 0.0
+    return np.triu(H) + np.triu(H, 1).T
+
+
+# n: one CTA; a ragged tile; the cluster's edges (ld 640 / 768); 32-, 64- and 128-column
+# units on the whole chip; grid limits that give several rounds, and last rounds cut in 2 and 4
+@pytest.mark.parametrize("n,limit", [(1, 0), (2, 0), (31, 0), (128, 0), (129, 0), (300, 0), (640, 0), (641, 0),
+                                     (1100, 0), (1600, 0), (300, 1), (300, 5), (400, 8), (513, 12)])
+def test_fermi_single_launch(ctx, n, limit):
+    H = _banded(n, n)
+    nocc, kT = 0.5 * n - (0.25 if n < 3 else 0.0), 0.15
+    Ht = torch.as_tensor(H, device="cuda")
+    D = torch.full_like(Ht, float("nan"))
+    s = FermiSolver(ctx, n, fermi_opts())
+    tbmd.tb_ctx_set_grid_limit(ctx, limit)
+    try:
+        s(Ht, nocc, kT, D)
+        torch.cuda.synchronize()
+    finally:
+        tbmd.tb_ctx_set_grid_limit(ctx, 0)
+    rep = fermi_report_to_dict(s.report)
+    assert rep["status"] == tbmd.TB_OK
+    Dn = D.cpu().numpy()
+    assert np.array_equal(Dn, Dn.T)
+    # dm_fermi's bound: FP32-level products whose errors add up over the doubling steps
+    assert np.linalg.norm(Dn - density.density_fermi(H, nocc, kT).D) / np.sqrt(n) < 2e-6
+
+
+def test_two_streams_at_once(ctx):
+    """Calls on two streams with workspaces of their own do not disturb each other."""
+    sizes, res = (900, 1000), []
+    Hs = [torch.as_tensor(_banded(n, n), device="cuda") for n in sizes]
+    sol = [FermiSolver(ctx, n, fermi_opts()) for n in sizes]
+    Ds = [torch.empty_like(H) for H in Hs]
+    for s, H, D, n in zip(sol, Hs, Ds, sizes):
+        s(H, 0.5 * n, 0.2, D)
+        torch.cuda.synchronize()
+        res.append(D.clone())
+        s.mu.fill_(float("nan"))
+    streams = [torch.cuda.Stream() for _ in sizes]
+    torch.cuda.synchronize()
+    for _ in range(3):
+        for s, H, D, n, st in zip(sol, Hs, Ds, sizes, streams):
+            with torch.cuda.stream(st):
+                s.mu.fill_(float("nan"))
+            s(H, 0.5 * n, 0.2, D, stream=st)
+    torch.cuda.synchronize()
+    for s, D, R in zip(sol, Ds, res):
+        assert fermi_report_to_dict(s.report)["status"] == tbmd.TB_OK
+        assert torch.equal(D, R)
