@@ -159,6 +159,7 @@ struct SP2State {
   unsigned long long rbranch;
   unsigned long long block_products;  // block-sparse path: executed 128^3 block products
   int kc[2];                     // main-phase projection index inside a while graph node
+  unsigned bar;                  // arrivals at the grid barriers of the single-launch form
 };
 
 // Parameters of a purification step shared by the FP64 and tensor-core kernels.
@@ -309,18 +310,15 @@ __device__ __forceinline__ void warp_reduce_partials(const double* parts, int np
 // takes it from there.  A rise of Tr X - Tr X^2 alone is no stop signal:
 // on small-gap spectra the HOMO or LUMO eigenvalue of X climbs from near 0
 // across the middle over several projections, doubling it each time.
-__device__ __forceinline__ int sp2_decide(const SP2StepArgs& a, double t1, double t2,
-                                          const double* hist_t1, const double* hist_t2,
-                                          bool tc_phase, int* branch, int* capped) {
+// e1, e2, e3: Tr X - Tr X^2 of the three projections before (tensor-core phase, k >= 3).
+__device__ __forceinline__ int sp2_decide_e(const SP2StepArgs& a, double t1, double t2, double e1, double e2,
+                                            double e3, bool tc_phase, int* branch, int* capped) {
   const double e = t1 - t2;
   *capped = 0;
   if (tc_phase) {
     if (e <= a.floor) return 1;
-    if (a.k >= 3) {
-      bool flat = e <= 4.0 * a.floor;
-      for (int j = 1; j <= 3; ++j) flat = flat && (hist_t1[a.k - j] - hist_t2[a.k - j] <= 4.0 * a.floor);
-      if (flat) return 1;
-    }
+    const double flat = 4.0 * a.floor;
+    if (a.k >= 3 && e <= flat && e1 <= flat && e2 <= flat && e3 <= flat) return 1;
   } else if (fabs(e) <= a.tol) {
     return 1;
   }
@@ -333,6 +331,15 @@ __device__ __forceinline__ int sp2_decide(const SP2StepArgs& a, double t1, doubl
   else
     *branch = (t1 > a.nocc) ? 0 : 1;
   return 0;
+}
+// The same with the history of the phase's traces.
+__device__ __forceinline__ int sp2_decide(const SP2StepArgs& a, double t1, double t2,
+                                          const double* hist_t1, const double* hist_t2,
+                                          bool tc_phase, int* branch, int* capped) {
+  double e[3] = {0.0, 0.0, 0.0};
+  if (tc_phase && a.k >= 3)
+    for (int j = 1; j <= 3; ++j) e[j - 1] = hist_t1[a.k - j] - hist_t2[a.k - j];
+  return sp2_decide_e(a, t1, t2, e[0], e[1], e[2], tc_phase, branch, capped);
 }
 
 // Next chemical potential of the Fermi expansion after an expansion at mu

@@ -1,4 +1,4 @@
-"""The single-launch form of dm_fermi: tile
+"""The single-launch forms of dm_fermi and of dm_sp2's tensor-core phase: tile
 edges, every unit width, cut last rounds, one cluster and a cooperative grid."""
 
 import numpy as np
@@ -7,7 +7,9 @@ import torch
 
 from oracle import density
 from paper_1203_6836_gb300 import tbmd
-from paper_1203_6836_gb300.device import FermiSolver, fermi_opts, fermi_report_to_dict
+from paper_1203_6836_gb300.device import (DensitySolver, FermiSolver, fermi_opts, fermi_report_to_dict,
+                                          report_to_dict, sp2_opts)
+from workloads import random_gapped_matrix
 
 pytestmark = pytest.mark.gpu
 
@@ -51,6 +53,55 @@ def test_fermi_single_launch(ctx, n, limit):
     assert np.array_equal(Dn, Dn.T)
     # dm_fermi's bound: FP32-level products whose errors add up over the doubling steps
     assert np.linalg.norm(Dn - density.density_fermi(H, nocc, kT).D) / np.sqrt(n) < 2e-6
+
+
+@pytest.mark.parametrize("n", [1, 127, 130, 300, 640, 700, 1300, 1700])
+@pytest.mark.parametrize("prec", ["tf32", "tf32x3"])
+def test_sp2_single_launch_is_the_launched_form(ctx, n, prec):
+    """Same products, same order: the same D to the last bit, eagerly and captured (launch
+    timing selects the launched form)."""
+    H = _banded(n, n + 1)
+    nocc = float(n // 2)
+    Ht = torch.as_tensor(H, device="cuda")
+    s = DensitySolver(ctx, n, sp2_opts(prec, refine=0 if n > 1500 else 2))
+    out = []
+    for form in ("launched", "single", "captured"):
+        D = torch.full_like(Ht, float("nan"))
+        tbmd.tb_ctx_set_profiling(ctx, form == "launched")
+        if form == "captured":
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, capture_error_mode="thread_local"):
+                s(Ht, nocc, D)
+            for _ in range(2):
+                g.replay()
+        else:
+            s(Ht, nocc, D)
+        torch.cuda.synchronize()
+        out.append((D, report_to_dict(s.report)))
+    tbmd.tb_ctx_set_profiling(ctx, False)
+    (D0, r0), rest = out[0], out[1:]
+    for D, r in rest:
+        assert torch.equal(D, D0)
+        for k in ("status", "iters", "refine_iters", "branches", "refine_branches", "eps_min", "eps_max"):
+            assert r[k] == r0[k]
+        assert abs(r["trace"] - r0["trace"]) <= 1e-12 * max(1.0, n)
+
+
+@pytest.mark.parametrize("limit", [1, 4, 7, 24])
+def test_sp2_single_launch_on_few_ctas(ctx, limit):
+    H, _ = random_gapped_matrix(600, 250, gap=4.0, width=20.0, seed=3)
+    Ht = torch.as_tensor(H, device="cuda")
+    s = DensitySolver(ctx, 600, sp2_opts("tf32x3", refine=0))
+    D0, D = torch.empty_like(Ht), torch.empty_like(Ht)
+    s(Ht, 250.0, D0)
+    tbmd.tb_ctx_set_grid_limit(ctx, limit)
+    try:
+        s(Ht, 250.0, D)
+        torch.cuda.synchronize()
+    finally:
+        tbmd.tb_ctx_set_grid_limit(ctx, 0)
+    assert torch.equal(D, D0)
+    assert report_to_dict(s.report)["status"] == tbmd.TB_OK
 
 
 def test_two_streams_at_once(ctx):
