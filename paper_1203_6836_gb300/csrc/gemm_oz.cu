@@ -74,59 +74,102 @@ __device__ __forceinline__ void pair_of(int p, int* s, int* t) {
   *t = rem + 1;
 }
 
-// One warp per row: e_i from the row maximum, then the kS signed 7-bit
-// digits of every entry of the row.  r = x 2^{-e} (|r| < 1/2) is scaled
-// exactly and rounded once to the integer R = rint(r 2^{7 kS}) (|R| <= 2^41);
-// the digits are R's balanced base-128 digits, peeled off from the least
-// significant end in int64 arithmetic: d in [-64, 63] for s >= 2 and
-// |d_1| <= 64 (2^41 + 2^34 < 64.5 2^35), all exact in bf16.  Four consecutive
-// entries per lane per pass.
-__global__ void __launch_bounds__(256) k_oz_split(const SP2State* st, const double* __restrict__ X, int ld,
-                                                  __nv_bfloat16* __restrict__ slices, int* __restrict__ exps) {
+// One block per row (256 threads, 8 or 16 entries each, read once): e_i from the
+// row maximum, then the kS signed 7-bit digits of every entry of the row.
+// r = x 2^{-e} (|r| < 1/2) is rounded once to the integer R = rint(r 2^{7 kS})
+// (|R| <= 2^41); the digits are R's balanced base-128 digits: d in [-64, 63] for
+// s >= 2 and |d_1| <= 64 (2^41 + 2^34 < 64.5 2^35), all exact in bf16.
+// Integer throughout: the FP64 pipe (2 results per clock and SM) and the I2F
+// conversions bound the form before this one (a scaled FP64 multiplication, an FP64 to
+// int64 conversion and six int64 to FP32 conversions per entry, each row read twice):
+// 0.31 ms at ld = 4096, where reading 8 and writing 12 bytes per entry takes 0.05.
+// R comes from the entry's bits by a rounding shift, its digits from R + sum 64 128^k
+// as unsigned bit fields, and a digit's bf16 is the high half of an FP32 obtained by
+// an addition (1.5 2^23 + d) - 1.5 2^23.
+constexpr int kSplitThreads = 256;
+
+// rint(x 2^{kBeta kS - e}) for a finite x with |x| < 2^{e-1} (else the integer that an
+// FP64 to int64 conversion gives: the smallest)
+__device__ __forceinline__ long long oz_fixed(double x, int e) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int ef = (int)(b >> 52) & 0x7ff;
+  unsigned long long m = b & 0xfffffffffffffull;
+  if (ef) m |= 1ull << 52;
+  // x = m 2^{max(ef, 1) - 1075}; the shift is at least 12 as the row maximum sets e
+  int sh = 1075 - kBeta * kS + e - (ef ? ef : 1);
+  sh = min(sh, 60);  // below half a unit either way: rounds to 0
+  m = (m + (1ull << (sh - 1)) - 1 + ((m >> sh) & 1)) >> sh;  // nearest, ties to even
+  const long long r = (long long)b < 0 ? -(long long)m : (long long)m;
+  return ef == 0x7ff ? (long long)0x8000000000000000ull : r;
+}
+
+__global__ void __launch_bounds__(kSplitThreads) k_oz_split(const SP2State* st, const double* __restrict__ X, int ld,
+                                                            __nv_bfloat16* __restrict__ slices,
+                                                            int* __restrict__ exps) {
+  __shared__ unsigned long long s_mx[kSplitThreads / 32];
   if (st->rdone || st->err) return;
-  const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (row >= ld) return;
+  const int row = blockIdx.x, lane = threadIdx.x & 31;
   const double* xr = X + (size_t)row * ld;
-  double mx = 0.0;
-  for (int j = 4 * lane; j < ld; j += 128) {
-    const double2 u = *reinterpret_cast<const double2*>(xr + j);
-    const double2 w = *reinterpret_cast<const double2*>(xr + j + 2);
-    mx = fmax(mx, fmax(fmax(fabs(u.x), fabs(u.y)), fmax(fabs(w.x), fabs(w.y))));
+  constexpr int kStep = 8 * kSplitThreads;  // entries per pass: ld <= 4096 takes two at most
+  double x[2][8];
+  unsigned long long mx = 0;  // largest magnitude as bits, which order alike; NaN left out
+#pragma unroll
+  for (int p = 0; p < 2; ++p) {
+    const int j = p * kStep + 8 * threadIdx.x;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      double2 u = make_double2(0.0, 0.0);
+      if (j < ld) u = *reinterpret_cast<const double2*>(xr + j + 2 * q);
+      x[p][2 * q] = u.x;
+      x[p][2 * q + 1] = u.y;
+    }
   }
-  mx = warp_max(mx);
+#pragma unroll
+  for (int p = 0; p < 2; ++p)
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const unsigned long long b = (unsigned long long)__double_as_longlong(x[p][q]) & 0x7fffffffffffffffull;
+      if (b <= 0x7ff0000000000000ull && b > mx) mx = b;
+    }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long v = __shfl_xor_sync(0xffffffffu, mx, o);
+    mx = v > mx ? v : mx;
+  }
+  if (lane == 0) s_mx[threadIdx.x >> 5] = mx;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kSplitThreads / 32; ++w) mx = s_mx[w] > mx ? s_mx[w] : mx;
+  // mx = f 2^{e-1} with f in [0.5, 1): |x| / 2^e < 1/2; not below -960: such rows are
+  // below every digit (subnormal maxima too)
   int e = 0;
-  if (mx > 0.0) {
-    frexp(mx, &e);  // mx = f 2^e, f in [0.5, 1): |x| / 2^{e+1} < 1/2
-    e = max(e + 1, -960);  // keeps 2^{42 - e} finite; such rows are below every digit
-  }
-  if (lane == 0) exps[row] = e;
+  if (mx) e = max((int)(mx >> 52) - 1021, -960);
+  if (threadIdx.x == 0) exps[row] = e;
   const size_t plane = (size_t)ld * ld;
-  const double scale = ldexp(1.0, kBeta * kS - e);  // exact power of two
-  for (int j = 4 * lane; j < ld; j += 128) {
-    const double2 u = *reinterpret_cast<const double2*>(xr + j);
-    const double2 w = *reinterpret_cast<const double2*>(xr + j + 2);
-    long long R[4] = {__double2ll_rn(u.x * scale), __double2ll_rn(u.y * scale), __double2ll_rn(w.x * scale),
-                      __double2ll_rn(w.y * scale)};
-    unsigned short dg[kS][4];
 #pragma unroll
-    for (int s = kS - 1; s >= 1; --s) {
+  for (int p = 0; p < 2; ++p) {
+    const int j = p * kStep + 8 * threadIdx.x;
+    if (j >= ld) continue;
+    uint32_t w[kS][4];
 #pragma unroll
-      for (int e4 = 0; e4 < 4; ++e4) {
-        const long long d = ((R[e4] + 64) & 127) - 64;  // balanced remainder in [-64, 63]
-        R[e4] = (R[e4] - d) >> kBeta;                   // exact division by 128
-        dg[s][e4] = __bfloat16_as_ushort(__float2bfloat16_rn((float)d));
+    for (int q = 0; q < 4; ++q) {
+      float f[2][kS];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        // digits d_k + 64 of kBeta bits, k = 0 (least) .. kS - 2, below the leading one
+        const long long B = oz_fixed(x[p][2 * q + h], e) + 0x408102040ll;
+#pragma unroll
+        for (int k = 0; k < kS - 1; ++k)
+          f[h][kS - 1 - k] = __int_as_float(0x4b400000 + (int)((B >> (kBeta * k)) & 127) - 64) - 12582912.0f;
+        f[h][0] = (float)(int)(B >> (kBeta * (kS - 1)));
       }
+#pragma unroll
+      for (int s = 0; s < kS; ++s)
+        w[s][q] = __byte_perm(__float_as_uint(f[0][s]), __float_as_uint(f[1][s]), 0x7632);
     }
 #pragma unroll
-    for (int e4 = 0; e4 < 4; ++e4) dg[0][e4] = __bfloat16_as_ushort(__float2bfloat16_rn((float)R[e4]));
-#pragma unroll
-    for (int s = 0; s < kS; ++s) {
-      uint2 pk;
-      pk.x = (uint32_t)dg[s][0] | ((uint32_t)dg[s][1] << 16);
-      pk.y = (uint32_t)dg[s][2] | ((uint32_t)dg[s][3] << 16);
-      *reinterpret_cast<uint2*>(slices + s * plane + (size_t)row * ld + j) = pk;
-    }
+    for (int s = 0; s < kS; ++s)
+      *reinterpret_cast<uint4*>(slices + s * plane + (size_t)row * ld + j) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
   }
 }
 
@@ -300,7 +343,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         uint32_t v[16];
         tmem_ld16(tmem + (static_cast<uint32_t>(32 * q) << 16) + acc * kTile + 64 * h + 16 * c, v);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) acc64[16 * c + j] += __float2ll_rn(__uint_as_float(v[j]) * fs) << lsh;
+        for (int j = 0; j < 16; ++j) acc64[16 * c + j] += (long long)__float2int_rn(__uint_as_float(v[j]) * fs) << lsh;
       }
       tc_fence_before();
       __syncwarp();
@@ -595,7 +638,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             uint32_t v[16];
             tmem_ld16(tmem + (static_cast<uint32_t>(32 * q) << 16) + (2 * set + p) * kTile + 64 * h + 16 * c, v);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) acc64[16 * c + j] += __float2ll_rn(__uint_as_float(v[j]) * fs) << lsh;
+            for (int j = 0; j < 16; ++j) acc64[16 * c + j] += (long long)__float2int_rn(__uint_as_float(v[j]) * fs) << lsh;
           }
         }
         tc_fence_before();
@@ -713,7 +756,7 @@ int sp2_oz_step(tb_ctx* ctx, const SP2StepArgs& a, const double* Xin, double* Xo
   if (a.ld > 4096 || a.ld % kTile) return tb_fail(ctx, TB_ERR_UNSUPPORTED, "emulated FP64 needs ld <= 4096");
   static unsigned long long attr_done = 0;
   if (int rc_attr = tb_smem_attr(ctx, k_sp2_step_oz, kSmem, &attr_done)) return rc_attr;
-  k_oz_split<<<(a.ld * 32 + 255) / 256, 256, 0, s>>>(a.st, Xin, a.ld, static_cast<__nv_bfloat16*>(slices), exps);
+  k_oz_split<<<a.ld, kSplitThreads, 0, s>>>(a.st, Xin, a.ld, static_cast<__nv_bfloat16*>(slices), exps);
   TB_LAUNCH_CHECK(ctx);
   const size_t plane = (size_t)a.ld * a.ld * sizeof(__nv_bfloat16);
   const int pairs = oz_pairs(ctx, a.ld);

@@ -329,22 +329,26 @@ void launch_f64(dim3 g, const SP2StepArgs& a, const double* X, double* Y, cudaSt
   else k_sp2_step_f64<kF64Tile><<<g, 256, 0, s>>>(a, X, Y);
 }
 
-// FP32 master (buffer chosen by the main phase's iteration count) -> FP64,
-// with trace partials: the start of the FP64 refinement.
+// FP32 master (buffer chosen by the main phase's iteration count) -> FP64: the
+// start of the FP64 refinement.  Its traces are those of the main phase's last
+// iterate (FP64 sums over the same FP32 values), so none are summed again: with them
+// the pass took as long on the FP64 pipe (two results per clock and SM) as on memory.
 __global__ void __launch_bounds__(256) k_to_f64(const SP2State* st, const float* __restrict__ M0,
-                                                const float* __restrict__ M1, int ld,
+                                                const float* __restrict__ M1, size_t quads,
                                                 double* __restrict__ F, double* __restrict__ parts) {
-  const float* M = (st->iters & 1) ? M1 : M0;
-  const int r0 = blockIdx.y * kInitTile, c0 = blockIdx.x * kInitTile;
-  double t1 = 0.0, t2 = 0.0;
-  for (int e = threadIdx.x; e < kInitTile * kInitTile; e += blockDim.x) {
-    const int r = r0 + e / kInitTile, c = c0 + e % kInitTile;
-    const double x = (double)M[(size_t)r * ld + c];
-    F[(size_t)r * ld + c] = x;
-    if (r == c) t1 += x;
-    t2 += x * x;
+  const float4* M = reinterpret_cast<const float4*>((st->iters & 1) ? M1 : M0);
+  const size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i0 == 0) {
+    parts[0] = st->t1[st->iters];
+    parts[1] = st->t2[st->iters];
+    parts[2] = 0.0;
   }
-  block_sum3(t1, t2, 0.0, parts + 3 * (blockIdx.y * gridDim.x + blockIdx.x));
+  for (size_t i = i0; i < quads; i += (size_t)gridDim.x * blockDim.x) {
+    const float4 x = M[i];
+    double2* o = reinterpret_cast<double2*>(F + 4 * i);
+    o[0] = make_double2((double)x.x, (double)x.y);
+    o[1] = make_double2((double)x.z, (double)x.w);
+  }
 }
 
 // Copy the final iterate into D (n x n) and fill the report.
@@ -356,17 +360,21 @@ __global__ void __launch_bounds__(256) k_finalize(SP2State* st, int n, int ld, i
                                                   double* __restrict__ D, double nocc,
                                                   tb_sp2_report* rep) {
   // mode 0: FP64 main phase; 1: FP64 refinement; 2: FP32 master, no refinement
-  const size_t total = (size_t)n * n;
+  // (a row per block and pass: no division per element)
   const int sel = mode == 1 ? (st->riters & 1) : (st->iters & 1);
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (size_t)gridDim.x * blockDim.x) {
-    const int r = (int)(e / n), c = (int)(e % n);
-    double x;
-    if (mode == 2)
-      x = (double)(sel ? M1 : M0)[(size_t)r * ld + c];
-    else
-      x = (sel ? F1 : F0)[(size_t)r * ld + c];
-    D[e] = x;
+  const double* F = sel ? F1 : F0;
+  const float* M = sel ? M1 : M0;
+  for (int r = blockIdx.x; r < n; r += gridDim.x) {
+    double* d = D + (size_t)r * n;
+    if (mode == 2) {
+      const float* m = M + (size_t)r * ld;
+#pragma unroll 4
+      for (int c = threadIdx.x; c < n; c += blockDim.x) d[c] = (double)m[c];
+    } else {
+      const double* f = F + (size_t)r * ld;
+#pragma unroll 4
+      for (int c = threadIdx.x; c < n; c += blockDim.x) d[c] = f[c];
+    }
   }
   if (blockIdx.x == 0 && threadIdx.x == 0 && rep) {
     double t1, t2;
@@ -556,7 +564,7 @@ extern "C" int dm_sp2(tb_ctx* ctx, const double* H, int n, double nocc, const tb
       return TB_OK;
     });
     if (rc) return rc;
-    const int fb = std::min(1184, (int)(((size_t)n * n + 255) / 256));
+    const int fb = std::min(1216, n);
     k_finalize<<<fb, 256, 0, s>>>(st, n, ld, 0, F0, F1, nullptr, nullptr, D, nocc, rep);
     TB_LAUNCH_CHECK(ctx);
     return TB_OK;
@@ -619,15 +627,15 @@ extern "C" int dm_sp2(tb_ctx* ctx, const double* H, int n, double nocc, const tb
   }
   a.kc = nullptr;
   a.cond = 0;
-  const int fb = std::min(1184, (int)(((size_t)n * n + 255) / 256));
+  const int fb = std::min(1216, n);
   if (refine == 0) {
     k_finalize<<<fb, 256, 0, s>>>(st, n, ld, 2, nullptr, nullptr, M[0], M[1], D, nocc, rep);
     TB_LAUNCH_CHECK(ctx);
     return TB_OK;
   }
   // FP64 refinement
-  const dim3 gc(ld / kInitTile, ld / kInitTile);
-  k_to_f64<<<gc, 256, 0, s>>>(st, M[0], M[1], ld, F0, slot[0]);
+  const size_t quads = (size_t)ld * ld / 4;
+  k_to_f64<<<(int)std::min<size_t>(2432, (quads + 255) / 256), 256, 0, s>>>(st, M[0], M[1], quads, F0, slot[0]);
   TB_LAUNCH_CHECK(ctx);
   SP2StepArgs r = a;
   r.phase = 1;
@@ -638,7 +646,7 @@ extern "C" int dm_sp2(tb_ctx* ctx, const double* H, int n, double nocc, const tb
   tb_prof_mark(ctx, 1, 0, s);
   for (int k = 0; k <= refine; ++k) {
     r.k = k;
-    r.nparts_in = k == 0 ? (int)(gc.x * gc.y) : np_ref;
+    r.nparts_in = k == 0 ? 1 : np_ref;
     r.parts_in = slot[k & 1];
     r.parts_out = slot[(k + 1) & 1];
     double* Fin = (k & 1) ? F1 : F0;
