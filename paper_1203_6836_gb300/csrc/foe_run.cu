@@ -425,7 +425,7 @@ int launch(tb_ctx* ctx, const FoeRunArgs& a, int cluster, int grid, int* ran, cu
   static unsigned long long attr_done = 0;
   if (int rc = tb_smem_attr(ctx, k_foe_run<P, BN>, Q::smem, &attr_done)) return rc;
   static RunFits fits;
-  return tb_run_launch(ctx, k_foe_run<P, BN>, &fits, Q::smem, cluster, grid, ran, s, a, mp);
+  return tb_run_launch(ctx, k_foe_run<P, BN>, &fits, kRunThreads, Q::smem, cluster, grid, ran, s, a, mp);
 }
 
 template <int P>

@@ -354,11 +354,11 @@ int tb_run_maps(tb_ctx* ctx, float* m, void* hi, void* lo, int ld, CUtensorMap (
 
 // Launches it; *ran stays 0 where no cluster of this size fits the device.
 template <typename K, typename... A>
-int tb_run_launch(tb_ctx* ctx, K kernel, RunFits* fits, int smem, int cluster, int grid, int* ran, cudaStream_t s,
+int tb_run_launch(tb_ctx* ctx, K kernel, RunFits* fits, int threads, int smem, int cluster, int grid, int* ran, cudaStream_t s,
                   const A&... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(tcx::kRunThreads);
+  cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute at{};

@@ -277,6 +277,15 @@ __global__ void __launch_bounds__(256) k_sp2_step_f64(const SP2StepArgs a_in, co
   if (stop) return;
 
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  // upper-triangle tiles only, mirrored: X is symmetric (the FP64 pipe bounds this
+  // kernel, so the half that is left out is half its time)
+  double* const part = a.parts_out + 3 * (blockIdx.y * gridDim.x + blockIdx.x);
+  if (blockIdx.x < blockIdx.y) {
+    if (threadIdx.x < 3) part[threadIdx.x] = 0.0;
+    return;
+  }
+  const bool mirror = blockIdx.x != blockIdx.y;
+  const double w = mirror ? 2.0 : 1.0;  // the transposed tile counts too
   const int row0 = blockIdx.y * T, col0 = blockIdx.x * T;
   const int ld = a.ld;
   double acc[R][R];
@@ -317,11 +326,12 @@ __global__ void __launch_bounds__(256) k_sp2_step_f64(const SP2StepArgs a_in, co
       const double cxx = acc[i][j];
       const double y = br ? 2.0 * x - cxx : cxx;
       Y[(size_t)r * ld + c] = y;
+      if (mirror) Y[(size_t)c * ld + r] = y;
       if (r == c) t1 += y;
       t2 += y * y;
       t3 += (cxx - x) * (cxx - x);
     }
-  block_sum3(t1, t2, t3, a.parts_out + 3 * (blockIdx.y * gridDim.x + blockIdx.x));
+  block_sum3(t1, w * t2, w * t3, part);
 }
 
 void launch_f64(dim3 g, const SP2StepArgs& a, const double* X, double* Y, cudaStream_t s) {
@@ -376,39 +386,7 @@ __global__ void __launch_bounds__(256) k_finalize(SP2State* st, int n, int ld, i
       for (int c = threadIdx.x; c < n; c += blockDim.x) d[c] = f[c];
     }
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0 && rep) {
-    double t1, t2;
-    if (mode == 1) {
-      t1 = st->rt1[st->riters];
-      t2 = st->rt2[st->riters];
-    } else {
-      t1 = st->t1[st->iters];
-      t2 = st->t2[st->iters];
-    }
-    // status: device error; an FP64 phase that hit its cap without reaching
-    // |Tr X - Tr X^2| <= 1e-6 max(1, N_occ); a trace that missed N_occ
-    // (no gap at the occupation)
-    int status = TB_OK;
-    const double e = t1 - t2;
-    const bool capped = mode == 1 ? st->rcapped : (mode == 0 ? st->capped : 0);
-    if (st->err) status = st->err;
-    else if (capped && fabs(e) > 1e-6 * fmax(1.0, nocc)) status = TB_ERR_NOT_CONVERGED;
-    else if (fabs(t1 - nocc) > 0.25) status = TB_ERR_GAP;
-    rep->status = status;
-    rep->iters = st->iters;
-    rep->refine_iters = mode == 1 ? st->riters : 0;
-    rep->n = n;
-    rep->eps_min = st->emin;
-    rep->eps_max = st->emax;
-    rep->trace = t1;
-    rep->idem_trace = e;
-    rep->idem_fro = mode == 1 && st->riters > 0 ? st->idem_fro : -1.0;
-    rep->branch_bits[0] = st->branch[0];
-    rep->branch_bits[1] = st->branch[1];
-    rep->refine_bits = st->rbranch;
-    rep->block_products = 0;
-    rep->blocks = 0;
-  }
+  if (blockIdx.x == 0 && threadIdx.x == 0 && rep) sp2_fill_report(st, mode, n, nocc, rep);
 }
 
 }  // namespace
@@ -553,6 +531,24 @@ extern "C" int dm_sp2(tb_ctx* ctx, const double* H, int n, double nocc, const tb
   a.tol = o->tol;
   a.max_iter = o->max_iter;
   a.phase = 0;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  TB_CUDA_TRY(ctx, cudaStreamIsCapturing(s, &cs));
+  const int captured = cs != cudaStreamCaptureStatusNone;
+  if (!tc && n <= kSp2Run64Max && !ctx->prof_on) {
+    Sp2Run64Args g{};
+    g.a = a;
+    g.H = H;
+    g.bparts = bparts;
+    g.nbparts = nb;
+    g.F[0] = F0;
+    g.F[1] = F1;
+    g.parts[0] = slot[0];
+    g.parts[1] = slot[1];
+    g.bar = &st->bar;
+    g.D = D;
+    g.rep = rep;
+    return sp2_run64(ctx, g, captured, s);
+  }
   if (!tc) {
     k_init_x<<<g_init, 256, 0, s>>>(H, n, ld, bparts, nb, st, F0, nullptr, slot[0]);
     TB_LAUNCH_CHECK(ctx);
@@ -581,8 +577,6 @@ extern "C" int dm_sp2(tb_ctx* ctx, const double* H, int n, double nocc, const tb
   // timing on, the launched form: it has the launches that are timed)
   int ran = 0;
   if (!ctx->prof_on) {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    TB_CUDA_TRY(ctx, cudaStreamIsCapturing(s, &cs));
     Sp2RunArgs g{};
     g.a = a;
     g.H = H;
@@ -595,7 +589,7 @@ extern "C" int dm_sp2(tb_ctx* ctx, const double* H, int n, double nocc, const tb
       g.parts[b] = slot[b];
     }
     g.bar = &st->bar;
-    const int rc = sp2_run(ctx, o->precision, g, cs != cudaStreamCaptureStatusNone, &ran, s);
+    const int rc = sp2_run(ctx, o->precision, g, captured, &ran, s);
     if (rc) return rc;
   }
   if (!ran) {

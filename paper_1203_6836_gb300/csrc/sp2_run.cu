@@ -344,7 +344,7 @@ int launch(tb_ctx* ctx, const Sp2RunArgs& g, const RunShape& r, int* ran, cudaSt
   static unsigned long long attr_done = 0;
   if (int rc = tb_smem_attr(ctx, k_sp2_run<P, BN>, Q::smem, &attr_done)) return rc;
   static RunFits fits;
-  return tb_run_launch(ctx, k_sp2_run<P, BN>, &fits, Q::smem, r.cluster, r.grid, ran, s, g, mp);
+  return tb_run_launch(ctx, k_sp2_run<P, BN>, &fits, kRunThreads, Q::smem, r.cluster, r.grid, ran, s, g, mp);
 }
 
 template <int P>

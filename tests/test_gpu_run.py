@@ -126,3 +126,41 @@ def test_two_streams_at_once(ctx):
     for s, D, R in zip(sol, Ds, res):
         assert fermi_report_to_dict(s.report)["status"] == tbmd.TB_OK
         assert torch.equal(D, R)
+
+
+# units of 8 x 8 (to n = 136) and 16 x 16; one cluster, one unit per SM, several; grid limits
+@pytest.mark.parametrize("n,limit", [(1, 0), (7, 0), (8, 0), (40, 0), (48, 0), (48, 3), (136, 0), (137, 0), (200, 16),
+                                     (300, 0), (512, 0), (513, 0)])
+def test_fp64_single_launch(ctx, n, limit):
+    """The FP64 recursion against the eigenvalue projector and against the launched form (same
+    branches; sums over K in another order: a rounding of 1e-16 n per product, which the
+    projections of converged eigenvalues contract)."""
+    H = _banded(n, n + 2)
+    nocc = float(n // 2)
+    Ht = torch.as_tensor(H, device="cuda")
+    s = DensitySolver(ctx, n, sp2_opts("fp64", tol=1e-11))
+    D0, D = torch.empty_like(Ht), torch.full_like(Ht, float("nan"))
+    tbmd.tb_ctx_set_profiling(ctx, True)  # selects the launched form
+    s(Ht, nocc, D0)
+    torch.cuda.synchronize()
+    r0 = report_to_dict(s.report)
+    tbmd.tb_ctx_set_profiling(ctx, False)
+    tbmd.tb_ctx_set_grid_limit(ctx, limit)
+    try:
+        s(Ht, nocc, D)
+        g = torch.cuda.CUDAGraph()
+        Dg = torch.empty_like(D)
+        torch.cuda.synchronize()
+        r = report_to_dict(s.report)
+        with torch.cuda.graph(g, capture_error_mode="thread_local"):
+            s(Ht, nocc, Dg)
+        g.replay()
+        torch.cuda.synchronize()
+    finally:
+        tbmd.tb_ctx_set_grid_limit(ctx, 0)
+    assert r["status"] == r0["status"] == tbmd.TB_OK
+    assert r["iters"] == r0["iters"] and r["branches"] == r0["branches"]
+    assert torch.equal(Dg, D)
+    assert (D - D0).abs().max().item() < 1e-12
+    if 1 < n:
+        assert np.linalg.norm(D.cpu().numpy() - density.density_T0(H, int(nocc)).D) / np.sqrt(n) < 1e-9
