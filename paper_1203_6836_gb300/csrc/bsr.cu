@@ -172,6 +172,12 @@ __device__ __forceinline__ double x0_val(const double* H, int n, int r, int c, d
   return ((r == c ? emax : 0.0) - H[(size_t)r * n + c]) * inv;
 }
 
+// Whether any lane's value is not zero (an integer test and a vote: a few cycles,
+// where an FP64 instruction of a warp takes 19).
+__device__ __forceinline__ bool any_nonzero(double x) {
+  return __any_sync(0xffffffffu, (__double_as_longlong(x) << 1) != 0);
+}
+
 // Per-lane partial sums of squares of the 16 32 x 32 sub-blocks of a 128 x 128
 // block x(r, c) (256 threads: warp w takes rows w + 8k, lane l the columns
 // 32 c + l, so every row segment is one coalesced load; row w + 8k lies in
@@ -182,13 +188,17 @@ __device__ __forceinline__ void block_partials(X x, double (&acc)[16]) {
 #pragma unroll
   for (int s = 0; s < 16; ++s) acc[s] = 0.0;
 #pragma unroll
-  for (int k = 0; k < 16; ++k) {
-    const int r = warp + 8 * k;
+  for (int kb = 0; kb < 4; ++kb) {  // the rows of one sub-block row: 16 loads in flight
+    double v[4][4];
 #pragma unroll
-    for (int cc = 0; cc < 4; ++cc) {
-      const double v = x(r, 32 * cc + lane);
-      acc[(k >> 2) * 4 + cc] = fma(v, v, acc[(k >> 2) * 4 + cc]);
-    }
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int cc = 0; cc < 4; ++cc) v[k][cc] = x(warp + 32 * kb + 8 * k, 32 * cc + lane);
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int cc = 0; cc < 4; ++cc)
+        if (any_nonzero(v[k][cc])) acc[kb * 4 + cc] = fma(v[k][cc], v[k][cc], acc[kb * 4 + cc]);
   }
 }
 
@@ -359,40 +369,49 @@ __device__ __forceinline__ int bsr_find(const int* __restrict__ row_ptr, const i
   return -1;
 }
 
-// Gershgorin partials of block row I (one block of 256 threads): warp w
-// takes rows w + 8k of every block of the row, lane l the columns 32 c + l, so
-// each block is read as 64 independent coalesced loads a lane, and the row
-// sums stay in registers until one warp sum per row; min(H_ii - r_i) and
-// max(H_ii + r_i) over the rows go into bparts[2 I].
+// Gershgorin partials of block row I (kBndSplit blocks of 256 threads, 32 rows
+// each): warp w takes rows w + 8k, lane l the columns 32 c + l, so each block is read
+// as 16 independent coalesced loads a lane, and the row sums stay in registers until
+// one warp sum per row; min(H_ii - r_i) and max(H_ii + r_i) over the rows go into
+// bparts[2 (I kBndSplit + y)].  The FP64 pipe would bound this kernel (1.1 ms for the
+// 1.2 GB of a 16 383-atom H): pieces of rows that are all zero, most of a block of a
+// molecular H, are skipped.
+constexpr int kBndSplit = 4;
 __global__ void __launch_bounds__(256) k_bsr_bounds_in(tb_bsr H, double* __restrict__ bparts) {
   __shared__ double smin[8], smax[8];
+  constexpr int kRows = 16 / kBndSplit;  // rows per warp
   const int I = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int r0 = blockIdx.y * (SB / kBndSplit) + warp;
+  bparts += 2 * (I * kBndSplit + blockIdx.y);
   if (*H.status != TB_OK) {  // an incomplete H (k_bsr_status_in fails the call)
-    if (threadIdx.x == 0) bparts[2 * I] = bparts[2 * I + 1] = 0.0;
+    if (threadIdx.x == 0) bparts[0] = bparts[1] = 0.0;
     return;
   }
-  double rad[16], dia[16];
+  double rad[kRows], dia[kRows];
 #pragma unroll
-  for (int k = 0; k < 16; ++k) rad[k] = dia[k] = 0.0;
+  for (int k = 0; k < kRows; ++k) rad[k] = dia[k] = 0.0;
   for (int o = H.row_ptr[I]; o < H.row_ptr[I + 1]; ++o) {
     const double* blk = H.val + (size_t)o * kTiles;
     const bool dblk = H.col[o] == I;
+    double x[kRows][4];
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      const int r = warp + 8 * k;
+    for (int k = 0; k < kRows; ++k)
+#pragma unroll
+      for (int cc = 0; cc < 4; ++cc) x[k][cc] = blk[(size_t)(r0 + 8 * k) * SB + 32 * cc + lane];
+#pragma unroll
+    for (int k = 0; k < kRows; ++k)
 #pragma unroll
       for (int cc = 0; cc < 4; ++cc) {
-        const double x = blk[(size_t)r * SB + 32 * cc + lane];
-        if (dblk && 32 * cc + lane == r) dia[k] += x;
-        else rad[k] += fabs(x);
+        if (!any_nonzero(x[k][cc])) continue;
+        if (dblk && 32 * cc + lane == r0 + 8 * k) dia[k] += x[k][cc];
+        else rad[k] += fabs(x[k][cc]);
       }
-    }
   }
   double lo = INFINITY, hi = -INFINITY;
 #pragma unroll
-  for (int k = 0; k < 16; ++k) {
+  for (int k = 0; k < kRows; ++k) {
     const double rs = warp_sum(rad[k]), c = warp_sum(dia[k]);  // one lane holds the diagonal element
-    if (I * SB + warp + 8 * k < H.n) {
+    if (I * SB + r0 + 8 * k < H.n) {
       lo = fmin(lo, c - rs);
       hi = fmax(hi, c + rs);
     }
@@ -408,8 +427,8 @@ __global__ void __launch_bounds__(256) k_bsr_bounds_in(tb_bsr H, double* __restr
       a = fmin(a, smin[w]);
       b = fmax(b, smax[w]);
     }
-    bparts[2 * I] = a;
-    bparts[2 * I + 1] = b;
+    bparts[0] = a;
+    bparts[1] = b;
   }
 }
 
@@ -447,7 +466,7 @@ __device__ __forceinline__ int bsr_row_of(const int* __restrict__ row_ptr, int n
   return lo;
 }
 
-// Keep masks of X0 from a BSR H, one block per stored block of H (grid-stride;
+// Keep masks of X0 from a BSR H, one block per stored upper block of H (grid-stride;
 // the masks start zeroed, and a block H does not store is zero in X0 off the
 // diagonal); k_bsr_init_flags_diag covers diagonal blocks H does not store.
 __global__ void __launch_bounds__(256) k_bsr_init_flags_in(tb_bsr H, Args a, Sym sy) {
@@ -457,13 +476,20 @@ __global__ void __launch_bounds__(256) k_bsr_init_flags_in(tb_bsr H, Args a, Sym
   x0_affine(a, &emax, &inv);
   for (int o = blockIdx.x; o < nblk; o += gridDim.x) {
     const int I = bsr_row_of(H.row_ptr, H.nsb, o), J = H.col[o];
-    const int I0 = min(I, J), J0 = max(I, J);
-    const int slot = I <= J ? o : bsr_find(H.row_ptr, H.col, I0, J0);
-    const double* blk = slot >= 0 ? H.val + (size_t)slot * kTiles : nullptr;
+    if (I > J) continue;  // its mask is its twin's transposed (or 0: H stores none)
+    const double* blk = H.val + (size_t)o * kTiles;
     double acc[16];
-    block_partials([&](int r, int c) { return x0_unscaled(blk, I0, J0, a.n, r, c, emax); }, acc);
+    block_partials([&](int r, int c) { return x0_unscaled(blk, I, J, a.n, r, c, emax); }, acc);
     const uint16_t f = keep_mask(a, I, J, acc, inv * inv);
-    if (threadIdx.x == 0) sy.flags[(size_t)I * a.nsb + J] = f;
+    if (threadIdx.x == 0) {
+      sy.flags[(size_t)I * a.nsb + J] = f;
+      if (I != J && bsr_find(H.row_ptr, H.col, J, I) >= 0) {
+        uint16_t t = 0;
+        for (int q = 0; q < 16; ++q)
+          if ((f >> q) & 1) t |= (uint16_t)(1u << ((q & 3) * 4 + (q >> 2)));
+        sy.flags[(size_t)J * a.nsb + I] = t;
+      }
+    }
   }
 }
 
@@ -1004,8 +1030,16 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
           __syncwarp();
         }
 #pragma unroll
-        for (int j = 0; j < 32; ++j) ss += (double)y[j] * (double)y[j];
-        ss = warp_sum(ss);  // squared Frobenius norm of sub-block (q, c)
+        for (int j = 0; j < 32; ++j) {
+          const double d = abs_to_f64(y[j]);
+          ss = fma(d, d, ss);
+        }
+        // squared Frobenius norm of sub-block (q, c); this lane's share of it is also its
+        // share of ||X||_F^2 when the sub-block is kept.  (The FP64 pipe, at 1.7 results per
+        // clock and SM, bounds the blocks of few products: one FMA per element and no
+        // conversion leaves 5 us of the 19 us that two of each took.)
+        const double mine = ss;
+        ss = warp_sum(ss);
         const bool keep = ss >= a.tau2 && ss > 0.0;
         if (!keep) {
 #pragma unroll
@@ -1013,11 +1047,11 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
         } else {
           kept = 1;
         }
-        double u2 = 0.0;
+        const double u2 = keep ? mine : 0.0;
+        if (I == J && c == q) {
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          u2 += (double)y[j] * (double)y[j];
-          if (I == J && row == 32 * c + j) t1 += (double)y[j];
+          for (int j = 0; j < 32; ++j)
+            if (j == lane) t1 += (double)y[j];
         }
         const bool twice = mirror || (symd && c > q);
         t2 += twice ? 2.0 * u2 : u2;
@@ -1120,19 +1154,42 @@ __global__ void __launch_bounds__(256) k_bsr_affine(Args a, Buf X, Buf out, floa
       out.col[o] = J;
       out.nz[o] = X.nz[o] | (diag ? 1 : 0);
     }
-    for (int seg = threadIdx.x; seg < SB * 4; seg += blockDim.x) {
-      const int r = seg >> 2, cs = seg & 3;
-      const size_t e0 = (size_t)o * kTiles + (size_t)r * SB + 32 * cs;
-      float y[32];
-#pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        y[j] = alpha * X.val[e0 + j];
-        if (diag && r == 32 * cs + j && I * SB + r < a.n) y[j] += delta;
+    if constexpr (kStaged<P>) {
+      // 16 bytes a lane, consecutive across the block, several loads in flight (a thread
+      // per 32-value segment took 0.31 ms for what memory moves in 0.05)
+      const float4* src = reinterpret_cast<const float4*>(X.val + (size_t)o * kTiles);
+      float4* dst = reinterpret_cast<float4*>(out.val + (size_t)o * kTiles);
+#pragma unroll 8
+      for (int e = threadIdx.x; e < kTiles / 4; e += 256) {
+        float4 x = src[e];
+        x.x *= alpha;
+        x.y *= alpha;
+        x.z *= alpha;
+        x.w *= alpha;
+        if (diag) {
+          const int r = e / (SB / 4), d = r - 4 * (e % (SB / 4));
+          if (I * SB + r < a.n) {
+            if (d == 0) x.x += delta;
+            if (d == 1) x.y += delta;
+            if (d == 2) x.z += delta;
+            if (d == 3) x.w += delta;
+          }
+        }
+        dst[e] = x;
       }
-      float* dst = out.val + e0;
+    } else {
+      for (int seg = threadIdx.x; seg < SB * 4; seg += blockDim.x) {
+        const int r = seg >> 2, cs = seg & 3;
+        const size_t e0 = (size_t)o * kTiles + (size_t)r * SB + 32 * cs;
+        float y[32];
 #pragma unroll
-      for (int j = 0; j < 32; ++j) dst[j] = y[j];
-      if constexpr (!kStaged<P>) {
+        for (int j = 0; j < 32; ++j) {
+          y[j] = alpha * X.val[e0 + j];
+          if (diag && r == 32 * cs + j && I * SB + r < a.n) y[j] += delta;
+        }
+        float* dst = out.val + e0;
+#pragma unroll
+        for (int j = 0; j < 32; ++j) dst[j] = y[j];
         char* hp = static_cast<char*>(out.hi) + e0 * Prec<P>::eb;
         char* lp = out.lo ? static_cast<char*>(out.lo) + e0 * Prec<P>::eb : hp;
         store_operands<P>(y, hp, lp);
@@ -1230,7 +1287,7 @@ BsrLayout bsr_layout(int n, int prec, int bpr, int nbuf) {
   const bool split = prec == TB_PREC_TF32X3 || prec == TB_PREC_BF16X3;
   L.staged = prec == TB_PREC_TF32X3;
   L.off_state = take(sizeof(SP2State));
-  L.off_bparts = take(sizeof(double) * 2 * std::max((n + 7) / 8, L.nsb));
+  L.off_bparts = take(sizeof(double) * 2 * std::max((n + 7) / 8, kBndSplit * L.nsb));
   L.off_parts = take(sizeof(double) * 3 * 2 * L.nparts);
   L.off_scal = take(sizeof(int) * 4);
   L.off_flags = take(sizeof(uint16_t) * (size_t)L.nsb * L.nsb);
@@ -1424,9 +1481,9 @@ int run_bsr(tb_ctx* ctx, const double* H, const tb_bsr* Hb, int n, double nocc, 
   if (Hb) {
     k_bsr_status_in<<<1, 1, 0, s>>>(Hb->status, st);
     TB_LAUNCH_CHECK(ctx);
-    k_bsr_bounds_in<<<L.nsb, 256, 0, s>>>(*Hb, e.bparts);
+    k_bsr_bounds_in<<<dim3(L.nsb, kBndSplit), 256, 0, s>>>(*Hb, e.bparts);
     TB_LAUNCH_CHECK(ctx);
-    k_bsr_bounds<<<1, 32, 0, s>>>(e.bparts, L.nsb, st);
+    k_bsr_bounds<<<1, 32, 0, s>>>(e.bparts, kBndSplit * L.nsb, st);
   } else {
     const int nb = (n + 7) / 8;
     if ((rc = sp2_launch_bounds(ctx, H, n, e.bparts, s))) return rc;
@@ -1510,8 +1567,8 @@ int run_bsr_fermi(tb_ctx* ctx, const tb_bsr* Hb, int n, double nocc, double kT, 
   const double beta = 1.0 / kT;
   TB_CUDA_TRY(ctx, cudaMemsetAsync(st, 0, sizeof(SP2State), s));
   k_bsr_status_in<<<1, 1, 0, s>>>(Hb->status, st);
-  k_bsr_bounds_in<<<L.nsb, 256, 0, s>>>(*Hb, e.bparts);
-  k_bsr_bounds<<<1, 32, 0, s>>>(e.bparts, L.nsb, st);
+  k_bsr_bounds_in<<<dim3(L.nsb, kBndSplit), 256, 0, s>>>(*Hb, e.bparts);
+  k_bsr_bounds<<<1, 32, 0, s>>>(e.bparts, kBndSplit * L.nsb, st);
   TB_LAUNCH_CHECK(ctx);
   SP2State hs;
   double mu0 = NAN;

@@ -231,7 +231,7 @@ size_t sp2_oz_slice_bytes(int ld);
 
 // Generic tensor-core product out = alpha A B + beta E + gamma I of symmetric,
 // commuting matrices (gemm_tc.cu); all matrices ld x ld, FP32 masters with
-// operand splits; parts (2 doubles per CTA: Tr out, ||out||^2) optional.
+// operand splits; parts (one double per CTA: Tr out) optional.
 struct GemmArgs {
   int n, ld;
   float alpha, beta, gamma;
@@ -284,6 +284,18 @@ __device__ __forceinline__ double warp_max(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
+}
+
+// |x| as FP64, exactly, in integer instructions (subnormals as 0; Inf and NaN kept).
+// GB300 converts FP32 to FP64 at two values per clock and SM, as slowly as it
+// multiplies them: in an epilogue that sums squares the conversion would be half the
+// time.
+__device__ __forceinline__ double abs_to_f64(float x) {
+  const uint32_t a = __float_as_uint(x) & 0x7fffffffu;
+  uint32_t hi = (a >> 3) + 0x38000000u, lo = a << 29;
+  if (a >= 0x7f800000u) hi |= 0x7ff00000u;
+  if (a < 0x00800000u) hi = lo = 0u;
+  return __hiloint2double((int)hi, (int)lo);
 }
 
 // Deterministic sum of `np` partial pairs by one warp (fixed order): lane l

@@ -141,9 +141,9 @@ __global__ void k_foe_mu(FoeState* st, const double* parts, const double* partsw
   }
   double x = 0.0, y = 0.0, z = 0.0;
   for (int i = threadIdx.x; i < np; i += 32) {
-    x += parts[2 * i];
-    y += partsw[2 * i];
-    z += parts3[2 * i];
+    x += parts[i];
+    y += partsw[i];
+    z += parts3[i];
   }
   x = warp_sum(x);  // Tr E
   y = warp_sum(y);  // Tr W

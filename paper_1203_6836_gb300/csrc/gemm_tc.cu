@@ -161,7 +161,10 @@ __device__ __forceinline__ void sp2_epi_tile(const SP2StepArgs& a, int br, uint3
       }
     }
 #pragma unroll
-    for (int j = 0; j < 32; ++j) u2 = fma((double)y[j], (double)y[j], u2);
+    for (int j = 0; j < 32; ++j) {
+      const double d = abs_to_f64(y[j]);
+      u2 = fma(d, d, u2);
+    }
     if (!mirror) {
       // diagonal tile (or one of its halves): element j is on the diagonal
       // when m0 + row == n0 + 32c + j
@@ -795,8 +798,7 @@ int sp2_tc_step(tb_ctx* ctx, int precision, const SP2StepArgs& a, const CUtensor
 // like the SP2 projection, a persistent grid computes the upper-triangle
 // tiles into two alternating TMEM accumulators and writes each off-diagonal
 // tile also transposed, so `out` is exactly symmetric.  Writes the FP32
-// master and the operand splits of `out` and per-CTA FP64 partials
-// (Tr out, ||out||_F^2).  Returns at once when *skip is non-zero
+// master and the operand splits of `out` and per-CTA FP64 partials of Tr out.  Returns at once when *skip is non-zero
 // (device-side early exit of a converged outer iteration).
 // --------------------------------------------------------------------------
 
@@ -812,7 +814,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ __align__(8) uint64_t full[Q::stages], empty[Q::stages], tfull[2], tempty[2], mdone;
   __shared__ uint32_t tmem_base;
   __shared__ volatile int s_abort;
-  __shared__ double s_red[4][2];
+  __shared__ double s_red[4];
   if (g.skip && *g.skip) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -899,7 +901,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // arrives once every MMA this thread issued has completed
     umma_commit(&mdone);
   } else if (warp >= 2) {
-    double t1 = 0.0, t2 = 0.0;
+    double t1 = 0.0;
     const int q = warp & 3;
     const int row = 32 * q + lane;
     int it = 0;
@@ -916,7 +918,6 @@ __global__ void __launch_bounds__(kThreads, 1)
       float* orow = g.out + gr * g.ld + n0;
       char* hrow = static_cast<char*>(g.ohi) + (gr * g.ld + n0) * C::eb;
       char* lrow = g.olo ? static_cast<char*>(g.olo) + (gr * g.ld + n0) * C::eb : hrow;
-      double u2 = 0.0, u3 = 0.0, lower = 0.0;
 #pragma unroll 1
       for (int c = 0; c < BN / 32; ++c) {
         uint32_t v[32];
@@ -942,8 +943,6 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (erow) val = fmaf(g.beta, es[j], val);
           if (col == (int)gr && (int)gr < g.n) val += g.gamma;
           y[j] = val;
-          u2 += (double)val * (double)val;
-          if (col < (int)gr) lower += (double)val * (double)val;
           if (col == (int)gr) t1 += (double)val;
         }
         const size_t col0 = (size_t)n0 + 32 * c;
@@ -971,32 +970,20 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (col > gr) {
               g.out[tdx] = y[j];
               store_operand1<P>(y[j], g.ohi, g.olo ? g.olo : g.ohi, tdx);
-              u3 += (double)y[j] * (double)y[j];
             }
           }
         }
       }
-      // off-diagonal tiles count twice; in a diagonal tile the kept upper
-      // triangle counts twice off the diagonal (u3) and the lower one not at all
-      t2 += mirror ? 2.0 * u2 : u2 + u3 - lower;
       tc_fence_before();
       if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tempty[buf])) : "memory");
     }
     t1 = warp_sum(t1);
-    t2 = warp_sum(t2);
-    if (lane == 0) {
-      s_red[q][0] = t1;
-      s_red[q][1] = t2;
-    }
+    if (lane == 0) s_red[q] = t1;
   }
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 64) {
-    if (g.parts) {
-      const int cta = blockIdx.x;
-      g.parts[2 * cta] = s_red[0][0] + s_red[1][0] + s_red[2][0] + s_red[3][0];
-      g.parts[2 * cta + 1] = s_red[0][1] + s_red[1][1] + s_red[2][1] + s_red[3][1];
-    }
+    if (g.parts) g.parts[blockIdx.x] = s_red[0] + s_red[1] + s_red[2] + s_red[3];
     if (s_abort && g.err) atomicExch(g.err, TB_ERR_TIMEOUT);
   }
   if (warp == 1) {

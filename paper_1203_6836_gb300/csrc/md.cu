@@ -17,6 +17,7 @@
 
 #include "common.cuh"
 
+#include <cooperative_groups.h>
 #include <math.h>
 #include <string.h>
 
@@ -54,16 +55,23 @@ __global__ void k_n_update(int N, double* __restrict__ hist, int K, const double
   hist[i] = n_new;
 }
 
-// Second half kick, kinetic energy, E_tot and max|n - q| in one block; the
-// step counter E[7] is 0 after the initial state (kick = 0), +1 per step.
+// Second half kick, kinetic energy, E_tot and max|n - q|; the step counter
+// E[7] is 0 after the initial state (kick = 0), +1 per step.  CS blocks of one cluster
+// take a contiguous share of the atoms each and meet in the first one's shared memory:
+// one block to kKickOne atoms, eight above (at 16 383 atoms one SM's FP64 rate made it
+// 0.16 ms).
+constexpr int kKickOne = 512;
+template <int CS>
 __global__ void __launch_bounds__(256) k_kick_energy(int N, double* __restrict__ v, const double* __restrict__ F,
                                                      const double* __restrict__ mass, double dt, int kick,
                                                      const double* __restrict__ n_cur,
                                                      const double* __restrict__ q, double* __restrict__ E,
                                                      const double* __restrict__ S, double kT) {
   __shared__ double s_ke[8], s_dq[8];
+  __shared__ double s_all[CS][2];
+  const int per = (N + CS - 1) / CS, i1 = min(N, (int)(blockIdx.x + 1) * per);
   double ke = 0.0, dq = 0.0;
-  for (int i = threadIdx.x; i < N; i += blockDim.x) {
+  for (int i = blockIdx.x * per + threadIdx.x; i < i1; i += blockDim.x) {
     const double s = 0.5 * dt * kEvAmuToAFs2 / mass[i];
     double v2 = 0.0;
 #pragma unroll
@@ -92,11 +100,46 @@ __global__ void __launch_bounds__(256) k_kick_energy(int N, double* __restrict__
       a += s_ke[k];
       b = fmax(b, s_dq[k]);
     }
+    double(*all)[2] = s_all;
+    if constexpr (CS > 1) all = cooperative_groups::this_cluster().map_shared_rank(&s_all[0], 0);
+    all[blockIdx.x][0] = a;
+    all[blockIdx.x][1] = b;
+  }
+  if constexpr (CS > 1) cooperative_groups::this_cluster().sync();
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    double a = 0.0, b = 0.0;
+    for (int k = 0; k < CS; ++k) {
+      a += s_all[k][0];
+      b = fmax(b, s_all[k][1]);
+    }
     E[5] = a;
     E[0] = a + E[1] - (S ? kT * S[0] : 0.0);  // Eq. Etot: - T_e S at finite temperature
     E[6] = b;
     E[7] = kick ? E[7] + 1.0 : 0.0;
   }
+}
+
+int launch_kick_energy(tb_ctx* ctx, const tb_md_state* st, double dt, int kick, const double* S, cudaStream_t s) {
+  const int N = st->sys.natoms;
+  if (N <= kKickOne) {
+    k_kick_energy<1><<<1, 256, 0, s>>>(N, st->v, st->F, st->mass, dt, kick, st->n_hist, st->q, st->energies, S,
+                                       st->kT);
+    TB_LAUNCH_CHECK(ctx);
+    return TB_OK;
+  }
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(8);
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = 8;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  TB_CUDA_TRY(ctx, cudaLaunchKernelEx(&cfg, k_kick_energy<8>, N, st->v, (const double*)st->F, st->mass, dt, kick,
+                                      (const double*)st->n_hist, (const double*)st->q, st->energies, S, st->kT));
+  return TB_OK;
 }
 
 // mu[0] <- the start of this step's dm_fermi, extrapolated from the last
@@ -336,9 +379,8 @@ extern "C" int xlbomd_init(tb_ctx* ctx, const tb_params* p, tb_md_state* st, con
   st->step = 0;
   rc = electronic_step(ctx, p, st, so, st->n_hist, s);
   if (rc) return rc;
-  k_kick_energy<<<1, 256, 0, s>>>(N, st->v, st->F, st->mass, xp->dt, 0, st->n_hist, st->q, st->energies,
-                                  entropy_on(st) ? st->entropy : nullptr, st->kT);
-  TB_LAUNCH_CHECK(ctx);
+  rc = launch_kick_energy(ctx, st, xp->dt, 0, entropy_on(st) ? st->entropy : nullptr, s);
+  if (rc) return rc;
   if (st->kT > 0.0) {
     const double nan3[3] = {NAN, NAN, NAN};
     TB_CUDA_TRY(ctx, cudaMemcpyAsync(st->mu + 1, nan3, sizeof(nan3), cudaMemcpyHostToDevice, s));
@@ -373,9 +415,8 @@ extern "C" int xlbomd_step(tb_ctx* ctx, const tb_params* p, tb_md_state* st, con
     k_mu_shift<<<1, 1, 0, s>>>(st->mu);
     TB_LAUNCH_CHECK(ctx);
   }
-  k_kick_energy<<<1, 256, 0, s>>>(N, st->v, st->F, st->mass, xp->dt, 1, st->n_hist, st->q, st->energies,
-                                  entropy_on(st) ? st->entropy : nullptr, st->kT);
-  TB_LAUNCH_CHECK(ctx);
+  rc = launch_kick_energy(ctx, st, xp->dt, 1, entropy_on(st) ? st->entropy : nullptr, s);
+  if (rc) return rc;
   st->step += 1;
   return TB_OK;
 }

@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_sp2_run(const Sp2RunArgs g_i
           double t1 = 0.0, t2 = 0.0;
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
-            const double d = (double)y[j];
+            const double d = abs_to_f64(y[j]);
             t2 = fma(d, d, t2);
           }
           if (diag) {
