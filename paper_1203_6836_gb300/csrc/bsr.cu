@@ -56,13 +56,19 @@ constexpr int MW = 32;             // bitmap words per row (1024 super-rows: n <
 constexpr int kMaxNsb = MW * 32;
 constexpr int kThreads = 192;      // numeric kernel: TMA, MMA, 4 epilogue warps
 // tf32x3 keeps only the FP32 master of every block: the numeric kernel loads the
-// masters and four converter warps split them into hi and lo in shared memory
-// (the same rounding the stored splits had, so the products are bitwise those
-// of stored splits), at half the operand bytes and a third of the stores
+// masters and eight converter warps split them, A into TMEM and B in shared memory
+// (tc_ptx.cuh; the same rounding the stored splits had, so the products are bitwise
+// those of stored splits), at half the operand bytes and a third of the stores
 template <int P>
 constexpr bool kStaged = P == TB_PREC_TF32X3;
 template <int P>
-constexpr int kNumThreads = kStaged<P> ? 320 : kThreads;
+constexpr int kNumThreads = kStaged<P> ? 448 : kThreads;
+template <int P>
+constexpr int kNumStages = kStaged<P> ? kFsStages : Prec<P>::stages;
+template <int P>
+constexpr int kNumStageBytes = kStaged<P> ? kFsStage : Prec<P>::stage_bytes;
+template <int P>
+constexpr int kNumSmem = kStaged<P> ? kFsSmem : Prec<P>::smem_bytes;
 constexpr int kTiles = SB * SB;    // elements per super-block
 constexpr int kMaxGrid = 256;      // cap of the persistent numeric grid (which is also at most the SM count)
 constexpr int kBand = 8;           // block rows whose outputs the numeric kernel walks together
@@ -821,8 +827,10 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
                   const __grid_constant__ CUtensorMap bh, const __grid_constant__ CUtensorMap bl, Buf S, Buf bn,
                   Sym sy, Epi ep) {
   using C = Prec<P>;
+  constexpr int NS = kNumStages<P>;
+  constexpr uint32_t kCols = kStaged<P> ? kFsTmemCols : 2 * SB;
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t full[C::stages], empty[C::stages], tfull[2], tempty[2], mdone, conv[C::stages];
+  __shared__ __align__(8) uint64_t full[NS], empty[NS], tfull[2], tempty[2], mdone, conv[NS];
   __shared__ uint32_t tmem_base;
   __shared__ volatile int s_abort;
   __shared__ double s_red[4][3];
@@ -835,10 +843,10 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   if (threadIdx.x == 0) {
-    for (int s = 0; s < C::stages; ++s) {
+    for (int s = 0; s < NS; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
-      mbar_init(&conv[s], 4);
+      mbar_init(&conv[s], 8);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&tfull[b], 1);
@@ -848,7 +856,7 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
     s_abort = 0;
     fence_barrier_init();
   }
-  if (warp == 1) tmem_alloc(&tmem_base, 2 * SB);
+  if (warp == 1) tmem_alloc(&tmem_base, kCols);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -869,11 +877,11 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
       for (int p = p0; p < p1 && !s_abort; ++p) {
         const int2 pr = sy.pairs[p];
         for (int c = 0; c < chunks; ++c, ++g) {
-          const int s = g % C::stages;
-          if (g >= C::stages && !mbar_wait(&empty[s], ((g / C::stages) - 1) & 1, &s_abort)) break;
-          uint8_t* base = smem + s * C::stage_bytes;
+          const int s = g % NS;
+          if (g >= NS && !mbar_wait(&empty[s], ((g / NS) - 1) & 1, &s_abort)) break;
+          uint8_t* base = smem + s * kNumStageBytes<P>;
           // staged: the FP32 masters into the hi positions only
-          mbar_expect_tx(&full[s], kStaged<P> ? 2 * 128 * 128 : C::stage_bytes);
+          mbar_expect_tx(&full[s], kStaged<P> ? 2 * kFsTile : C::stage_bytes);
           tma_load_2d(base, &ah, &full[s], c * C::bk, pr.x * SB);
           tma_load_2d(base + 128 * 128, &bh, &full[s], c * C::bk, pr.y * SB);
           if constexpr (C::split && !kStaged<P>) {
@@ -885,9 +893,9 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
       }
     }
     if (s_abort) {
-      for (int q = (issued > C::stages ? issued - C::stages : 0); q < issued; ++q) {
+      for (int q = (issued > NS ? issued - NS : 0); q < issued; ++q) {
         const unsigned long long t0 = gtime();
-        while (!mbar_try(&full[q % C::stages], (q / C::stages) & 1) && gtime() - t0 < kWaitNs) {
+        while (!mbar_try(&full[q % NS], (q / NS) & 1) && gtime() - t0 < kWaitNs) {
         }
       }
     }
@@ -904,22 +912,27 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
       bool first = true;
       for (int p = p0; p < p1 && !s_abort; ++p) {
         for (int c = 0; c < chunks; ++c, ++g) {
-          const int s = g % C::stages;
-          if (!mbar_wait(kStaged<P> ? &conv[s] : &full[s], (g / C::stages) & 1, &s_abort)) break;
+          const int s = g % NS;
+          if (!mbar_wait(kStaged<P> ? &conv[s] : &full[s], (g / NS) & 1, &s_abort)) break;
           tc_fence_after();
-          const uint32_t base = smem_u32(smem + s * C::stage_bytes);
-#pragma unroll
-          for (int ks = 0; ks < C::bk / C::uk; ++ks) {
-            const uint32_t koff = ks * 32;
-            const uint64_t dah = sdesc(base + koff), dbh = sdesc(base + 128 * 128 + koff);
-            umma<C::tf32>(d, dah, dbh, id, first ? 0u : 1u);
+          const uint32_t base = smem_u32(smem + s * kNumStageBytes<P>);
+          if constexpr (kStaged<P>) {
+            fs_mma(base, tmem, s, d, id, first, ep.lolo);
             first = false;
-            if constexpr (C::split) {
-              const uint64_t dal = sdesc(base + 2 * 128 * 128 + koff), dbl = sdesc(base + 3 * 128 * 128 + koff);
-              umma<C::tf32>(d, dah, dbl, id, 1u);
-              umma<C::tf32>(d, dal, dbh, id, 1u);
-              // lo x lo: in a square it keeps the diagonal blocks' sums of squares unbiased
-              if (ep.lolo) umma<C::tf32>(d, dal, dbl, id, 1u);
+          } else {
+#pragma unroll
+            for (int ks = 0; ks < C::bk / C::uk; ++ks) {
+              const uint32_t koff = ks * 32;
+              const uint64_t dah = sdesc(base + koff), dbh = sdesc(base + 128 * 128 + koff);
+              umma<C::tf32>(d, dah, dbh, id, first ? 0u : 1u);
+              first = false;
+              if constexpr (C::split) {
+                const uint64_t dal = sdesc(base + 2 * 128 * 128 + koff), dbl = sdesc(base + 3 * 128 * 128 + koff);
+                umma<C::tf32>(d, dah, dbl, id, 1u);
+                umma<C::tf32>(d, dal, dbh, id, 1u);
+                // lo x lo: in a square it keeps the diagonal blocks' sums of squares unbiased
+                if (ep.lolo) umma<C::tf32>(d, dal, dbl, id, 1u);
+              }
             }
           }
           umma_commit(&empty[s]);
@@ -931,28 +944,17 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
     // arrives once every MMA this thread issued has completed
     umma_commit(&mdone);
   } else if (kStaged<P> && warp >= 6) {
-    // converters: each stage's FP32 tiles of A and B (16 KB each, the hi
-    // positions) become hi in place and lo at +32 KB, 16 float4 a thread
-    const int ct = threadIdx.x - 192;
-    constexpr int kHalf = 2 * 128 * 128 / 16;  // float4 of A and B
+    // converters: warps 6-9 A, 10-13 B
     int g = 0;
     for (int u = blockIdx.x; u < nu && !s_abort; u += gridDim.x) {
       const int o = sy.order[u];
       const int npc = (sy.pair_ptr[o + 1] - sy.pair_ptr[o]) * chunks;
       for (int i = 0; i < npc && !s_abort; ++i, ++g) {
-        const int s = g % C::stages;
-        if (!mbar_wait_warp(&full[s], (g / C::stages) & 1, &s_abort)) break;
-        float4* stage = reinterpret_cast<float4*>(smem + s * C::stage_bytes);
-#pragma unroll 4
-        for (int e = ct; e < kHalf; e += 128) {
-          const float4 x = stage[e];
-          const float4 h = make_float4(to_tf32(x.x), to_tf32(x.y), to_tf32(x.z), to_tf32(x.w));
-          stage[e] = h;
-          stage[e + kHalf] = make_float4(to_tf32(x.x - h.x), to_tf32(x.y - h.y), to_tf32(x.z - h.z),
-                                         to_tf32(x.w - h.w));
-        }
-        // the generic-proxy stores must be visible to the tensor core's reads
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        const int s = g % NS;
+        if (!mbar_wait_warp(&full[s], (g / NS) & 1, &s_abort)) break;
+        uint8_t* stage = smem + s * kFsStage;
+        if (warp < 10) fs_convert_a(stage, tmem, s, warp & 3, lane);
+        else fs_convert_b(stage, threadIdx.x - 320);
         __syncwarp();
         if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&conv[s])) : "memory");
       }
@@ -1115,7 +1117,7 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
       }
     }
     __syncwarp();
-    tmem_dealloc(tmem, 2 * SB);
+    tmem_dealloc(tmem, kCols);
   }
 }
 
@@ -1440,7 +1442,7 @@ int launch_product(tb_ctx* ctx, Engine& e, Args a, const Mat& A, const Mat& B, c
   k_bsr_order<<<1, 1024, 0, s>>>(a, out.b, e.sy);
   TB_LAUNCH_CHECK(ctx);
   if (prof_k >= 0) tb_prof_mark(ctx, 1, 2 * prof_k, s);
-  k_bsr_step_tc<P><<<grid, kNumThreads<P>, Prec<P>::smem_bytes, s>>>(a, A.mh, A.ml, B.mh, B.ml, Sb, out.b, e.sy, ep);
+  k_bsr_step_tc<P><<<grid, kNumThreads<P>, kNumSmem<P>, s>>>(a, A.mh, A.ml, B.mh, B.ml, Sb, out.b, e.sy, ep);
   TB_LAUNCH_CHECK(ctx);
   if (prof_k >= 0) tb_prof_mark(ctx, 1, 2 * prof_k + 1, s);
   return TB_OK;
@@ -1449,7 +1451,7 @@ int launch_product(tb_ctx* ctx, Engine& e, Args a, const Mat& A, const Mat& B, c
 template <int P>
 int prepare_numeric(tb_ctx* ctx, int* grid) {
   static unsigned long long attr_done = 0;
-  if (int rc = tb_smem_attr(ctx, k_bsr_step_tc<P>, Prec<P>::smem_bytes, &attr_done)) return rc;
+  if (int rc = tb_smem_attr(ctx, k_bsr_step_tc<P>, kNumSmem<P>, &attr_done)) return rc;
   *grid = tb_persistent_grid(ctx, kMaxGrid);
   return TB_OK;
 }

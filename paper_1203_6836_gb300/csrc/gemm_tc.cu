@@ -943,7 +943,14 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (erow) val = fmaf(g.beta, es[j], val);
           if (col == (int)gr && (int)gr < g.n) val += g.gamma;
           y[j] = val;
-          if (col == (int)gr) t1 += (double)val;
+        }
+        if (!mirror && c == q) {
+          // (diagonal tile, the chunk of this warp's diagonal: one FP64 addition)
+          float x = 0.0f;
+#pragma unroll
+          for (int j = 0; j < 32; ++j)
+            if (j == lane) x = y[j];
+          t1 += (double)x;
         }
         const size_t col0 = (size_t)n0 + 32 * c;
         if (mirror) {

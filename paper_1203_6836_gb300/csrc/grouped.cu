@@ -34,7 +34,7 @@ using namespace tcx;
 
 constexpr int BM = 128;
 constexpr int kThreads = 192;
-constexpr int kThreadsFs = 320;  // FP32-staged form: four converter warps more
+constexpr int kThreadsFs = 448;  // FP32-staged form: eight converter warps more
 constexpr int kMaxLd = 512;
 
 inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
@@ -83,11 +83,22 @@ __device__ __forceinline__ void tri_tile(int t, int nt, int* I, int* J) {
   *J = i + t;
 }
 
+// t1 += y[d] in the lanes whose row's diagonal element is among these 32 (one FP64
+// addition, and only in the warps that have any: a predicated one per element kept the
+// FP64 pipe half busy).
+__device__ __forceinline__ void add_diag(const float (&y)[32], int d, double* t1) {
+  if (!__any_sync(0xffffffffu, d >= 0 && d < 32)) return;
+  float x = 0.0f;
+#pragma unroll
+  for (int j = 0; j < 32; ++j)
+    if (j == d) x = y[j];
+  *t1 += (double)x;
+}
+
 // FS (tf32x3, BN = 128): the FP32-staged form.  TMA loads the FP32 masters
-// of X_k only; four converter warps split each stage into hi and lo in shared
-// memory, in place (the split is elementwise, so the 128B swizzle is kept),
-// and the epilogue writes only the FP32 master of X_{k+1}.  The operands are
-// bitwise those of the stored-split form, at half the operand bytes and a
+// of X_k only; eight converter warps split each stage, A into TMEM and B in shared
+// memory (tc_ptx.cuh), and the epilogue writes only the FP32 master of X_{k+1}.  The
+// operands are bitwise those of the stored-split form, at half the operand bytes and a
 // third of the epilogue's stores.
 template <int P, int BN, bool FS>
 __global__ void __launch_bounds__(FS ? kThreadsFs : kThreads, 1)
@@ -98,8 +109,11 @@ __global__ void __launch_bounds__(FS ? kThreadsFs : kThreads, 1)
   using C = Prec<P>;
   using G = GCfg<P, BN>;
   constexpr bool kSym = BN == BM;
+  constexpr int NS = FS ? kFsStages : G::stages;
+  constexpr int kStageBytes = FS ? kFsStage : G::stage_bytes;
+  constexpr uint32_t kCols = FS ? kFsTmemCols : 2 * BN;
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t full[G::stages], empty[G::stages], tfull[2], tempty[2], conv[G::stages];
+  __shared__ __align__(8) uint64_t full[NS], empty[NS], tfull[2], tempty[2], conv[NS];
   __shared__ uint32_t tmem_base;
   __shared__ volatile int s_abort;
   __shared__ int s_sys, s_stop, s_br;
@@ -111,10 +125,10 @@ __global__ void __launch_bounds__(FS ? kThreadsFs : kThreads, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   if (threadIdx.x == 0) {
-    for (int s = 0; s < G::stages; ++s) {
+    for (int s = 0; s < NS; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
-      mbar_init(&conv[s], 4);
+      mbar_init(&conv[s], 8);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&tfull[b], 1);
@@ -123,7 +137,7 @@ __global__ void __launch_bounds__(FS ? kThreadsFs : kThreads, 1)
     s_abort = 0;
     fence_barrier_init();
   }
-  if (warp == 1) tmem_alloc(&tmem_base, 2 * BN);
+  if (warp == 1) tmem_alloc(&tmem_base, kCols);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -192,7 +206,13 @@ __global__ void __launch_bounds__(FS ? kThreadsFs : kThreads, 1)
           if (r < n && c < n) x = ((r == c ? emaxf : 0.0f) - (float)d.H[(size_t)r * n + c]) * invf;
           y[j] = x;
           s2 = fmaf(x, x, s2);
-          if (r == c) t1 += (double)x;
+        }
+        if (r >= c0 && r < c0 + 32) {
+          float x = 0.0f;
+#pragma unroll
+          for (int j = 0; j < 32; ++j)
+            if (c0 + j == r) x = y[j];
+          t1 += (double)x;
         }
         t2 += (double)s2;
         const size_t e0 = (size_t)(ro + r) * ga.cols + c0;
@@ -265,11 +285,11 @@ __global__ void __launch_bounds__(FS ? kThreadsFs : kThreads, 1)
             n0 = J * BN;
           }
           for (int kb = 0; kb < nk; ++kb, ++g_prod) {
-            const int s = g_prod % G::stages;
-            if (g_prod >= G::stages && !mbar_wait(&empty[s], ((g_prod / G::stages) - 1) & 1, &s_abort)) break;
-            uint8_t* base = smem + s * G::stage_bytes;
-            // FS: the FP32 masters only, into the hi positions
-            mbar_expect_tx(&full[s], FS ? G::a_bytes + G::b_bytes : G::stage_bytes);
+            const int s = g_prod % NS;
+            if (g_prod >= NS && !mbar_wait(&empty[s], ((g_prod / NS) - 1) & 1, &s_abort)) break;
+            uint8_t* base = smem + s * kStageBytes;
+            // FS: the FP32 masters only
+            mbar_expect_tx(&full[s], FS ? 2 * kFsTile : G::stage_bytes);
             tma_load_2d(base, mah, &full[s], kb * C::bk, ro + m0);
             tma_load_2d(base + G::a_bytes, mbh, &full[s], kb * C::bk, ro + n0);
             if constexpr (C::split && !FS) {
@@ -286,21 +306,25 @@ __global__ void __launch_bounds__(FS ? kThreadsFs : kThreads, 1)
           tc_fence_after();
           const uint32_t dt = tmem + acc * BN;
           for (int kb = 0; kb < nk; ++kb, ++g_mma) {
-            const int s = g_mma % G::stages;
-            if (!mbar_wait(FS ? &conv[s] : &full[s], (g_mma / G::stages) & 1, &s_abort)) break;
+            const int s = g_mma % NS;
+            if (!mbar_wait(FS ? &conv[s] : &full[s], (g_mma / NS) & 1, &s_abort)) break;
             tc_fence_after();
-            const uint32_t base = smem_u32(smem + s * G::stage_bytes);
+            const uint32_t base = smem_u32(smem + s * kStageBytes);
+            if constexpr (FS) {
+              fs_mma(base, tmem, s, dt, id, kb == 0, true);  // lo*lo too: X X is a square (unbiased diagonal)
+            } else {
 #pragma unroll
-            for (int ks = 0; ks < C::bk / C::uk; ++ks) {
-              const uint32_t koff = ks * 32;
-              const uint64_t a0 = sdesc(base + koff), b0 = sdesc(base + G::a_bytes + koff);
-              umma<C::tf32>(dt, a0, b0, id, (kb | ks) != 0);
-              if constexpr (C::split) {
-                const uint64_t a1 = sdesc(base + G::a_bytes + G::b_bytes + koff);
-                const uint64_t b1 = sdesc(base + 2 * G::a_bytes + G::b_bytes + koff);
-                umma<C::tf32>(dt, a0, b1, id, 1u);
-                umma<C::tf32>(dt, a1, b0, id, 1u);
-                umma<C::tf32>(dt, a1, b1, id, 1u);  // lo*lo: X X is a square (unbiased diagonal)
+              for (int ks = 0; ks < C::bk / C::uk; ++ks) {
+                const uint32_t koff = ks * 32;
+                const uint64_t a0 = sdesc(base + koff), b0 = sdesc(base + G::a_bytes + koff);
+                umma<C::tf32>(dt, a0, b0, id, (kb | ks) != 0);
+                if constexpr (C::split) {
+                  const uint64_t a1 = sdesc(base + G::a_bytes + G::b_bytes + koff);
+                  const uint64_t b1 = sdesc(base + 2 * G::a_bytes + G::b_bytes + koff);
+                  umma<C::tf32>(dt, a0, b1, id, 1u);
+                  umma<C::tf32>(dt, a1, b0, id, 1u);
+                  umma<C::tf32>(dt, a1, b1, id, 1u);  // lo*lo: X X is a square (unbiased diagonal)
+                }
               }
             }
             umma_commit(&empty[s]);
@@ -308,25 +332,14 @@ __global__ void __launch_bounds__(FS ? kThreadsFs : kThreads, 1)
           umma_commit(&tfull[acc]);
         }
       } else if (FS && warp >= 6) {
-        // converters: each stage's FP32 tiles of A and B (16 KB each, the hi
-        // positions) become hi in place and lo at +32 KB, 16 float4 a thread
-        const int ct = threadIdx.x - 192;
+        // converters: warps 6-9 A, 10-13 B
         for (int t = 0; t < ntiles && !s_abort; ++t) {
           for (int kb = 0; kb < nk; ++kb, ++g_conv) {
-            const int s = g_conv % G::stages;
-            if (!mbar_wait_warp(&full[s], (g_conv / G::stages) & 1, &s_abort)) break;
-            float4* stage = reinterpret_cast<float4*>(smem + s * G::stage_bytes);
-            constexpr int kHalf = (G::a_bytes + G::b_bytes) / 16;  // float4 of A and B
-#pragma unroll 4
-            for (int i = ct; i < kHalf; i += 128) {
-              const float4 x = stage[i];
-              const float4 h = make_float4(to_tf32(x.x), to_tf32(x.y), to_tf32(x.z), to_tf32(x.w));
-              stage[i] = h;
-              stage[i + kHalf] = make_float4(to_tf32(x.x - h.x), to_tf32(x.y - h.y), to_tf32(x.z - h.z),
-                                             to_tf32(x.w - h.w));
-            }
-            // the generic-proxy stores must be visible to the tensor core's reads
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            const int s = g_conv % NS;
+            if (!mbar_wait_warp(&full[s], (g_conv / NS) & 1, &s_abort)) break;
+            uint8_t* stage = smem + s * kFsStage;
+            if (warp < 10) fs_convert_a(stage, tmem, s, warp & 3, lane);
+            else fs_convert_b(stage, threadIdx.x - 320);
             __syncwarp();
             if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&conv[s])) : "memory");
           }
@@ -357,9 +370,10 @@ __global__ void __launch_bounds__(FS ? kThreadsFs : kThreads, 1)
           for (int c = 0; c < BN / 32; ++c) {
             uint32_t v[32];
             tmem_ld32(tmem + (static_cast<uint32_t>(32 * q) << 16) + acc * BN + 32 * c, v);
-            // X_k's row segment: eight 16-byte loads instead of 32 scalar ones
+            // X_k's row segment, where the branch takes it: eight 16-byte loads instead of
+            // 32 scalar ones
             float xs[32];
-            {
+            if (br) {
               const float4* x4 = reinterpret_cast<const float4*>(xin + 32 * c);
 #pragma unroll
               for (int j = 0; j < 8; ++j) {
@@ -375,11 +389,10 @@ __global__ void __launch_bounds__(FS ? kThreadsFs : kThreads, 1)
 #pragma unroll
             for (int j = 0; j < 32; ++j) {
               const float cxx = __uint_as_float(v[j]);
-              const float x = xs[j];
-              y[j] = br ? fmaf(2.0f, x, -cxx) : cxx;
+              y[j] = br ? fmaf(2.0f, xs[j], -cxx) : cxx;
               c2 = fmaf(y[j], y[j], c2);
-              if (m0 + row == n0 + 32 * c + j) t1 += (double)y[j];
             }
+            add_diag(y, m0 + row - n0 - 32 * c, &t1);
             u2 += (double)c2;
             float4* xo = reinterpret_cast<float4*>(xout + 32 * c);
 #pragma unroll
@@ -450,7 +463,7 @@ __global__ void __launch_bounds__(FS ? kThreadsFs : kThreads, 1)
       }
     }
     __syncwarp();
-    tmem_dealloc(tmem, 2 * BN);
+    tmem_dealloc(tmem, kCols);
   }
 }
 
@@ -604,7 +617,13 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (r < n && c < n) x = ((r == c ? emaxf : 0.0f) - (float)d.H[(size_t)r * n + c]) * invf;
           y[j] = x;
           s2 = fmaf(x, x, s2);
-          if (r == c) t1 += (double)x;
+        }
+        if (r >= c0 && r < c0 + 32) {
+          float x = 0.0f;
+#pragma unroll
+          for (int j = 0; j < 32; ++j)
+            if (c0 + j == r) x = y[j];
+          t1 += (double)x;
         }
         t2 += (double)s2;
         const size_t e0 = (size_t)(ro + r) * ga.cols + c0;
@@ -765,8 +784,8 @@ __global__ void __launch_bounds__(kThreads, 1)
               const float x = xs[j];
               y[j] = br ? fmaf(2.0f, x, -cxx) : cxx;
               c2 = fmaf(y[j], y[j], c2);
-              if (m0 + row == n0 + 32 * c + j) t1 += (double)y[j];
             }
+            add_diag(y, m0 + row - n0 - 32 * c, &t1);
             u2 += (double)c2;
             float4* xo = reinterpret_cast<float4*>(xout + 32 * c);
 #pragma unroll
@@ -933,17 +952,18 @@ template <int P, int BN, bool FS = false>
 int launch(tb_ctx* ctx, const Plan& p, char* base, int grid, cudaStream_t s) {
   using G = GCfg<P, BN>;
   static unsigned long long attr_done = 0;
-  if (int rc_attr = tb_smem_attr(ctx, k_sp2_grouped<P, BN, FS>, G::smem, &attr_done)) return rc_attr;
+  constexpr int smem = FS ? kFsSmem : G::smem;
+  if (int rc_attr = tb_smem_attr(ctx, k_sp2_grouped<P, BN, FS>, smem, &attr_done)) return rc_attr;
   const GArgs ga = make_args(p, base);
   TB_CUDA_TRY(ctx, cudaMemsetAsync(ga.queue, 0, sizeof(int), s));
   if constexpr (FS) {
     // A and B are row panels of the FP32 masters (BN = BM: one map per buffer)
-    k_sp2_grouped<P, BN, true><<<grid, kThreadsFs, G::smem, s>>>(ga, p.am[0], p.am[0], p.am[0], p.am[0], p.am[1],
+    k_sp2_grouped<P, BN, true><<<grid, kThreadsFs, smem, s>>>(ga, p.am[0], p.am[0], p.am[0], p.am[0], p.am[1],
                                                                  p.am[1], p.am[1], p.am[1]);
   } else {
     const CUtensorMap* bh = BN == 64 ? p.bh64 : p.bh128;
     const CUtensorMap* bl = BN == 64 ? p.bl64 : p.bl128;
-    k_sp2_grouped<P, BN, false><<<grid, kThreads, G::smem, s>>>(ga, p.ah[0], p.al[0], bh[0], bl[0], p.ah[1],
+    k_sp2_grouped<P, BN, false><<<grid, kThreads, smem, s>>>(ga, p.ah[0], p.al[0], bh[0], bl[0], p.ah[1],
                                                                 p.al[1], bh[1], bl[1]);
   }
   TB_LAUNCH_CHECK(ctx);

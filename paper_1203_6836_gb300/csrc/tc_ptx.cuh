@@ -240,6 +240,110 @@ __device__ __forceinline__ float to_tf32(float x) {
 
 
 
+// A operand in TMEM: the M x K tile's row r in lane r, one 32-bit column per tf32
+// element, from column `a`; B through its shared-memory descriptor.
+__device__ __forceinline__ void umma_ts_tf32(uint32_t tmem_d, uint32_t a, uint64_t b, uint32_t id, uint32_t acc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}" ::"r"(tmem_d),
+      "r"(a), "l"(b), "r"(id), "r"(acc)
+      : "memory");
+}
+// 16 consecutive 32-bit columns of this warp's 32 TMEM lanes, written.
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+      "%14, %15, %16};" ::"r"(taddr),
+      "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), "f"(v[9]),
+      "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15])
+      : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// hi = tf32(x), lo = tf32(x - hi), rounded to nearest with ties away as cvt.rna does,
+// in integer instructions (an addition of half a unit to the magnitude's bits and a
+// mask: 97 a clock and SM against 21 conversions).  The bits of an infinity or a NaN
+// would not survive that, so such values take the conversion.
+__device__ __forceinline__ void split_tf32(const float4& x, float4& h, float4& l) {
+  auto rna = [](float v) { return __uint_as_float((__float_as_uint(v) + 0x1000u) & 0xffffe000u); };
+  h = make_float4(rna(x.x), rna(x.y), rna(x.z), rna(x.w));
+  l = make_float4(rna(x.x - h.x), rna(x.y - h.y), rna(x.z - h.z), rna(x.w - h.w));
+  const float t = (x.x + x.y) + (x.z + x.w);
+  if (t - t != 0.0f) {
+    h = make_float4(to_tf32(x.x), to_tf32(x.y), to_tf32(x.z), to_tf32(x.w));
+    l = make_float4(to_tf32(x.x - h.x), to_tf32(x.y - h.y), to_tf32(x.z - h.z), to_tf32(x.w - h.w));
+  }
+}
+
+// The FP32-staged operand pipeline of the block-sparse and grouped kernels (tf32x3):
+// TMA loads the FP32 128 x 32 tiles of A and B; warps of a converter group of four turn
+// A into hi and lo in TMEM (row r in lane r: 32 columns each) and another group
+// turns B into hi (in place) and lo in shared memory.  What bounds such a kernel is the
+// shared-memory pipe (128 bytes a clock): with both operands split in shared memory a
+// K-step of 32 moved 32 KB in by TMA, 32 KB out and 64 KB in by the converters and 96-128
+// KB by the MMAs, 1800-2050 cycles against 1070-1420 of MMA; with A in TMEM the MMAs read
+// only B and A's split is not stored: 1150-1280.
+constexpr int kFsTile = 128 * 128;          // bytes of a 128 x 32 FP32 tile
+constexpr int kFsStage = 3 * kFsTile;       // A, B (then its hi), B's lo
+constexpr int kFsStages = 4;
+constexpr int kFsSmem = kFsStages * kFsStage + 1024;
+constexpr int kFsTmemA = 256;               // first TMEM column of the A stages (64 each)
+constexpr int kFsTmemCols = 512;            // two accumulators of 128, four A stages
+// A converter (128 threads of warps whose index mod 4 is their TMEM lane quarter).
+__device__ __forceinline__ void fs_convert_a(const uint8_t* stage, uint32_t tmem, int s, int q, int lane) {
+  const int row = 32 * q + lane;
+  const uint32_t ta = tmem + (static_cast<uint32_t>(32 * q) << 16) + kFsTmemA + 64 * s;
+  // all loads first: one warp per scheduler works on a stage, so its own instructions
+  // have to hide the latencies
+  float4 x[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) x[j] = *reinterpret_cast<const float4*>(stage + row * 128 + ((j ^ (row & 7)) << 4));
+#pragma unroll
+  for (int half = 0; half < 2; ++half) {
+    float h[16], l[16];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      float4 a, b;
+      split_tf32(x[4 * half + j], a, b);
+      h[4 * j] = a.x, h[4 * j + 1] = a.y, h[4 * j + 2] = a.z, h[4 * j + 3] = a.w;
+      l[4 * j] = b.x, l[4 * j + 1] = b.y, l[4 * j + 2] = b.z, l[4 * j + 3] = b.w;
+    }
+    tmem_st16(ta + 16 * half, h);
+    tmem_st16(ta + 32 + 16 * half, l);
+  }
+  tmem_st_wait();
+  tc_fence_before();
+}
+// B converter (128 threads, t = 0..127): elementwise, so the 128-byte swizzle is kept.
+__device__ __forceinline__ void fs_convert_b(uint8_t* stage, int t) {
+  float4* b = reinterpret_cast<float4*>(stage + kFsTile) + t;
+  float4 x[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) x[i] = b[128 * i];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    float4 h, l;
+    split_tf32(x[i], h, l);
+    b[128 * i] = h;
+    b[128 * i + kFsTile / 16] = l;
+  }
+  // the generic-proxy stores must be visible to the tensor core's reads
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+// The MMAs of one stage, in the order of the stored-split kernels.
+__device__ __forceinline__ void fs_mma(uint32_t stage, uint32_t tmem, int s, uint32_t d, uint32_t id, bool first,
+                                       bool lolo) {
+  const uint32_t ta = tmem + kFsTmemA + 64 * s;
+#pragma unroll
+  for (int ks = 0; ks < 4; ++ks) {
+    const uint64_t bh = sdesc(stage + kFsTile + ks * 32), bl = sdesc(stage + 2 * kFsTile + ks * 32);
+    umma_ts_tf32(d, ta + 8 * ks, bh, id, !(first && ks == 0));
+    umma_ts_tf32(d, ta + 8 * ks, bl, id, 1u);
+    umma_ts_tf32(d, ta + 32 + 8 * ks, bh, id, 1u);
+    if (lolo) umma_ts_tf32(d, ta + 32 + 8 * ks, bl, id, 1u);
+  }
+}
+
 // Traits of the tensor-core precisions: operand bytes, elements per 128-byte
 // row (one 128B-swizzle atom), K of one MMA instruction, hi/lo split.
 template <int P>
