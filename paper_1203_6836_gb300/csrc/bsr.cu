@@ -834,7 +834,7 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
   __shared__ uint32_t tmem_base;
   __shared__ volatile int s_abort;
   __shared__ double s_red[4][3];
-  __shared__ float s_sym[4][32][33];  // per epilogue warp: one 32 x 32 diagonal sub-block
+  __shared__ __align__(16) float s_sym[4][32][36];  // per epilogue warp: one 32 x 32 sub-block
   SP2State* st = a.st;
   if (st->done || st->err) return;
   const int br = ep.branch ? (int)((st->branch[a.k >> 6] >> (a.k & 63)) & 1ull) : 0;
@@ -977,8 +977,9 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
       const int om = mirror ? bn.row_ptr[J] + popc_below(sy.cand + J * MW, I) : o;
       float* xmir = bn.val + (size_t)om * kTiles;
       const int oi = sy.old_idx[o];
-      const float* xold = oi >= 0 ? S.val + (size_t)oi * kTiles + (size_t)row * SB : nullptr;
-      float* xnew = bn.val + (size_t)o * kTiles + (size_t)row * SB;
+      // this warp's 32 rows of S_IJ and of the new block
+      const float* xold = S.val + (size_t)(oi >= 0 ? oi : 0) * kTiles + (size_t)(32 * q) * SB;
+      float* xnew = bn.val + (size_t)o * kTiles + (size_t)(32 * q) * SB;
       // stored splits (not with kStaged)
       char* hrow = kStaged<P> ? nullptr : static_cast<char*>(bn.hi) + ((size_t)o * kTiles + (size_t)row * SB) * C::eb;
       char* lrow = bn.lo ? static_cast<char*>(bn.lo) + ((size_t)o * kTiles + (size_t)row * SB) * C::eb : hrow;
@@ -989,6 +990,8 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
 #pragma unroll 1
       for (int c = 0; c < 4; ++c) {
         if (symd && c < q) continue;  // written as the mirror of sub-block (c, q)
+        float4 xg[8];
+        if (oi >= 0) tile_fetch(xold + 32 * c, SB, lane, xg);
         uint32_t v[32];
         if (has) {
           tmem_ld32(tmem + (static_cast<uint32_t>(32 * q) << 16) + buf * SB + 32 * c, v);
@@ -996,19 +999,10 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
 #pragma unroll
           for (int j = 0; j < 32; ++j) v[j] = 0u;
         }
-        // S's row segment: eight 16-byte loads (a scalar load per element would
-        // touch 32 rows' lines per warp instruction 32 times over)
+        // S's sub-tile
         float xs[32];
-        if (xold) {
-          const float4* x4 = reinterpret_cast<const float4*>(xold + 32 * c);
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const float4 t = x4[j];
-            xs[4 * j] = t.x;
-            xs[4 * j + 1] = t.y;
-            xs[4 * j + 2] = t.z;
-            xs[4 * j + 3] = t.w;
-          }
+        if (oi >= 0) {
+          tile_turn_in(reinterpret_cast<uint8_t*>(s_sym[q]), lane, xg, xs);
         } else {
 #pragma unroll
           for (int j = 0; j < 32; ++j) xs[j] = 0.0f;
@@ -1057,18 +1051,7 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
         }
         const bool twice = mirror || (symd && c > q);
         t2 += twice ? 2.0 * u2 : u2;
-        {
-          // the 32 x 32 sub-tile through shared memory (lane l holds row l), so
-          // that each warp store writes one row's 128 contiguous bytes
-          __syncwarp();
-#pragma unroll
-          for (int j = 0; j < 32; ++j) s_sym[q][lane][j] = y[j];
-          __syncwarp();
-          float* rows = xnew - (size_t)lane * SB + 32 * c;  // row 32 q of the block, column 32 c
-#pragma unroll 8
-          for (int rr = 0; rr < 32; ++rr) rows[(size_t)rr * SB + lane] = s_sym[q][rr][lane];
-          __syncwarp();
-        }
+        tile_store(reinterpret_cast<uint8_t*>(s_sym[q]), lane, y, xnew + 32 * c, SB);
         if constexpr (!kStaged<P>) store_operands<P>(y, hrow + 32 * c * C::eb, lrow + 32 * c * C::eb);
         if (twice) {
           // element (row, 32c + j) of block (I, J) is element (32c + j, row) of

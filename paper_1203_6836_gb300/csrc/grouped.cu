@@ -121,6 +121,7 @@ __global__ void __launch_bounds__(FS ? kThreadsFs : kThreads, 1)
   __shared__ double s_t1, s_t2, s_lo, s_hi;
   __shared__ double s_hist[2][SP2_MAX_ITER + 2];
   __shared__ unsigned long long s_branch[2];
+  __shared__ __align__(16) uint8_t s_turn[4][4096];  // the epilogue warps' sub-tiles
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -350,8 +351,6 @@ __global__ void __launch_bounds__(FS ? kThreadsFs : kThreads, 1)
         double t1 = 0.0, t2 = 0.0;
         for (int t = 0; t < ntiles; ++t, ++t_epi) {
           const int acc = t_epi & 1;
-          if (!mbar_wait_warp(&tfull[acc], (t_epi >> 1) & 1, &s_abort)) break;
-          tc_fence_after();
           int m0 = (t / nt_n) * BM, n0 = (t % nt_n) * BN;
           if constexpr (kSym) {
             int I, J;
@@ -359,31 +358,27 @@ __global__ void __launch_bounds__(FS ? kThreadsFs : kThreads, 1)
             m0 = I * BM;
             n0 = J * BN;
           }
+          // X_k's first sub-tile is fetched while the MMAs run
+          float4 xg[8];
+          if (br) tile_fetch(ga.M[ib] + (size_t)(ro + m0 + 32 * q) * ga.cols + n0, ga.cols, lane, xg);
+          if (!mbar_wait_warp(&tfull[acc], (t_epi >> 1) & 1, &s_abort)) break;
+          tc_fence_after();
           const bool mirror = kSym && m0 != n0;
           const size_t grow = (size_t)(ro + m0 + row);
           double u2 = 0.0;
-          const float* xin = ga.M[ib] + grow * ga.cols + n0;
-          float* xout = ga.M[ob] + grow * ga.cols + n0;
+          // this warp's 32 rows of the tile
+          const float* xw = ga.M[ib] + (grow - lane) * ga.cols + n0;
+          float* xout = ga.M[ob] + (grow - lane) * ga.cols + n0;
           char* hrow = static_cast<char*>(ga.Hi[ob]) + (grow * ga.cols + n0) * C::eb;
           char* lrow = ga.Lo[ob] ? static_cast<char*>(ga.Lo[ob]) + (grow * ga.cols + n0) * C::eb : hrow;
 #pragma unroll 1
           for (int c = 0; c < BN / 32; ++c) {
             uint32_t v[32];
             tmem_ld32(tmem + (static_cast<uint32_t>(32 * q) << 16) + acc * BN + 32 * c, v);
-            // X_k's row segment, where the branch takes it: eight 16-byte loads instead of
-            // 32 scalar ones
+            // X_k's sub-tile, where the branch takes it
             float xs[32];
-            if (br) {
-              const float4* x4 = reinterpret_cast<const float4*>(xin + 32 * c);
-#pragma unroll
-              for (int j = 0; j < 8; ++j) {
-                const float4 t = x4[j];
-                xs[4 * j] = t.x;
-                xs[4 * j + 1] = t.y;
-                xs[4 * j + 2] = t.z;
-                xs[4 * j + 3] = t.w;
-              }
-            }
+            if (br) tile_turn_in(s_turn[q], lane, xg, xs);
+            if (br && c + 1 < BN / 32) tile_fetch(xw + 32 * (c + 1), ga.cols, lane, xg);
             float y[32];
             float c2 = 0.0f;  // chunk sum in FP32, accumulated in FP64 (GB300 FP64 is slow)
 #pragma unroll
@@ -394,9 +389,7 @@ __global__ void __launch_bounds__(FS ? kThreadsFs : kThreads, 1)
             }
             add_diag(y, m0 + row - n0 - 32 * c, &t1);
             u2 += (double)c2;
-            float4* xo = reinterpret_cast<float4*>(xout + 32 * c);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) xo[j] = make_float4(y[4 * j], y[4 * j + 1], y[4 * j + 2], y[4 * j + 3]);
+            tile_store(s_turn[q], lane, y, xout + 32 * c, ga.cols);
             if constexpr (!FS) store_operands<P>(y, hrow + 32 * c * C::eb, lrow + 32 * c * C::eb);
             if (mirror) {
               // element (m0 + row, n0 + 32c + j) is also (n0 + 32c + j, m0 + row):

@@ -5,6 +5,8 @@
 
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 namespace tcx {
 
 constexpr unsigned long long kWaitNs = 2000000000ull;  // bounded waits give up after 2 s
@@ -263,16 +265,23 @@ __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.
 // hi = tf32(x), lo = tf32(x - hi), rounded to nearest with ties away as cvt.rna does,
 // in integer instructions (an addition of half a unit to the magnitude's bits and a
 // mask: 97 a clock and SM against 21 conversions).  The bits of an infinity or a NaN
-// would not survive that, so such values take the conversion.
+// would not survive that: such values take the conversion (Any).
+template <bool Any>
 __device__ __forceinline__ void split_tf32(const float4& x, float4& h, float4& l) {
-  auto rna = [](float v) { return __uint_as_float((__float_as_uint(v) + 0x1000u) & 0xffffe000u); };
+  auto rna = [](float v) {
+    return Any ? to_tf32(v) : __uint_as_float((__float_as_uint(v) + 0x1000u) & 0xffffe000u);
+  };
   h = make_float4(rna(x.x), rna(x.y), rna(x.z), rna(x.w));
   l = make_float4(rna(x.x - h.x), rna(x.y - h.y), rna(x.z - h.z), rna(x.w - h.w));
-  const float t = (x.x + x.y) + (x.z + x.w);
-  if (t - t != 0.0f) {
-    h = make_float4(to_tf32(x.x), to_tf32(x.y), to_tf32(x.z), to_tf32(x.w));
-    l = make_float4(to_tf32(x.x - h.x), to_tf32(x.y - h.y), to_tf32(x.z - h.z), to_tf32(x.w - h.w));
-  }
+}
+// Whether 32 values are all finite (one test for all: a branch per float4 kept their
+// splits from overlapping, 1050 cycles a step against 600).
+__device__ __forceinline__ bool all_finite(const float4 (&x)[8]) {
+  float t[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) t[j] = (x[j].x + x[j].y) + (x[j].z + x[j].w);
+  const float s = ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]));
+  return s - s == 0.0f;
 }
 
 // The FP32-staged operand pipeline of the block-sparse and grouped kernels (tf32x3):
@@ -298,19 +307,24 @@ __device__ __forceinline__ void fs_convert_a(const uint8_t* stage, uint32_t tmem
   float4 x[8];
 #pragma unroll
   for (int j = 0; j < 8; ++j) x[j] = *reinterpret_cast<const float4*>(stage + row * 128 + ((j ^ (row & 7)) << 4));
+  auto go = [&](auto any) {
 #pragma unroll
-  for (int half = 0; half < 2; ++half) {
-    float h[16], l[16];
+    for (int half = 0; half < 2; ++half) {
+      float h[16], l[16];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      float4 a, b;
-      split_tf32(x[4 * half + j], a, b);
-      h[4 * j] = a.x, h[4 * j + 1] = a.y, h[4 * j + 2] = a.z, h[4 * j + 3] = a.w;
-      l[4 * j] = b.x, l[4 * j + 1] = b.y, l[4 * j + 2] = b.z, l[4 * j + 3] = b.w;
+      for (int j = 0; j < 4; ++j) {
+        float4 a, b;
+        split_tf32<decltype(any)::value>(x[4 * half + j], a, b);
+        h[4 * j] = a.x, h[4 * j + 1] = a.y, h[4 * j + 2] = a.z, h[4 * j + 3] = a.w;
+        l[4 * j] = b.x, l[4 * j + 1] = b.y, l[4 * j + 2] = b.z, l[4 * j + 3] = b.w;
+      }
+      tmem_st16(ta + 16 * half, h);
+      tmem_st16(ta + 32 + 16 * half, l);
     }
-    tmem_st16(ta + 16 * half, h);
-    tmem_st16(ta + 32 + 16 * half, l);
-  }
+  };
+  // (the stores to TMEM are of the whole warp)
+  if (__all_sync(0xffffffffu, all_finite(x))) go(std::false_type{});
+  else go(std::true_type{});
   tmem_st_wait();
   tc_fence_before();
 }
@@ -320,13 +334,17 @@ __device__ __forceinline__ void fs_convert_b(uint8_t* stage, int t) {
   float4 x[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) x[i] = b[128 * i];
+  auto go = [&](auto any) {
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    float4 h, l;
-    split_tf32(x[i], h, l);
-    b[128 * i] = h;
-    b[128 * i + kFsTile / 16] = l;
-  }
+    for (int i = 0; i < 8; ++i) {
+      float4 h, l;
+      split_tf32<decltype(any)::value>(x[i], h, l);
+      b[128 * i] = h;
+      b[128 * i + kFsTile / 16] = l;
+    }
+  };
+  if (all_finite(x)) go(std::false_type{});
+  else go(std::true_type{});
   // the generic-proxy stores must be visible to the tensor core's reads
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
@@ -341,6 +359,45 @@ __device__ __forceinline__ void fs_mma(uint32_t stage, uint32_t tmem, int s, uin
     umma_ts_tf32(d, ta + 8 * ks, bl, id, 1u);
     umma_ts_tf32(d, ta + 32 + 8 * ks, bh, id, 1u);
     if (lolo) umma_ts_tf32(d, ta + 32 + 8 * ks, bl, id, 1u);
+  }
+}
+
+// A warp's 32 x 32 FP32 sub-tile (row pitch ld) between global memory and registers, lane
+// l holding row l: eight 16-byte accesses a lane, each of four whole 128-byte rows, and a
+// turn through 4 KB of shared memory (16-byte chunks swizzled by row: no bank
+// conflicts).  A lane reading or writing its own row touches 32 lines per
+// instruction, 13-18 thousand cycles for the epilogue of a 128 x 128 tile.
+__device__ __forceinline__ void tile_fetch(const float* src, size_t ld, int lane, float4 (&g)[8]) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    g[i] = *reinterpret_cast<const float4*>(src + (size_t)(4 * i + (lane >> 3)) * ld + 4 * (lane & 7));
+}
+__device__ __forceinline__ void tile_turn_in(uint8_t* sm, int lane, const float4 (&g)[8], float (&y)[32]) {
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int r = 4 * i + (lane >> 3);
+    *reinterpret_cast<float4*>(sm + r * 128 + (((lane & 7) ^ (r & 7)) << 4)) = g[i];
+  }
+  __syncwarp();
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const float4 v = *reinterpret_cast<const float4*>(sm + lane * 128 + ((j ^ (lane & 7)) << 4));
+    y[4 * j] = v.x, y[4 * j + 1] = v.y, y[4 * j + 2] = v.z, y[4 * j + 3] = v.w;
+  }
+}
+__device__ __forceinline__ void tile_store(uint8_t* sm, int lane, const float (&y)[32], float* dst, size_t ld) {
+  __syncwarp();
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    *reinterpret_cast<float4*>(sm + lane * 128 + ((j ^ (lane & 7)) << 4)) =
+        make_float4(y[4 * j], y[4 * j + 1], y[4 * j + 2], y[4 * j + 3]);
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int r = 4 * i + (lane >> 3);
+    *reinterpret_cast<float4*>(dst + (size_t)r * ld + 4 * (lane & 7)) =
+        *reinterpret_cast<const float4*>(sm + r * 128 + (((lane & 7) ^ (r & 7)) << 4));
   }
 }
 
