@@ -120,6 +120,27 @@ __device__ __forceinline__ void unit_tile(const Units& w, int u, int* t, int* ha
   }
 }
 
+// The operand splits of a warp's 32 x 32 sub-tile at element e0 (row pitch ld), lane l
+// holding row l (at hrow, lrow): whole rows through the turning buffer for tf32, each
+// lane's own 64 bytes for bf16.
+template <int P>
+__device__ __forceinline__ void store_rows(uint8_t* turn, int lane, const float (&y)[32], void* hi, void* lo,
+                                           size_t e0, size_t ld, char* hrow, char* lrow) {
+  if constexpr (Prec<P>::tf32) {
+    float h[32];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) h[j] = to_tf32(y[j]);
+    tile_store(turn, lane, h, static_cast<float*>(hi) + e0, ld);
+    if constexpr (Prec<P>::split) {
+#pragma unroll
+      for (int j = 0; j < 32; ++j) h[j] = to_tf32(y[j] - h[j]);
+      tile_store(turn, lane, h, static_cast<float*>(lo) + e0, ld);
+    }
+  } else {
+    store_operands<P>(y, hrow, lrow);
+  }
+}
+
 // Epilogue of one output tile of a projection: rows m0 + [0, 128) (this
 // thread: row m0 + row, TMEM lane row), columns n0 + [0, 32 nchunk) read from
 // TMEM at `tcol` (lane offset included).  Applies the branch (X^2, or
@@ -131,12 +152,12 @@ template <int P>
 __device__ __forceinline__ void sp2_epi_tile(const SP2StepArgs& a, int br, uint32_t tcol, int row, int m0, int n0,
                                              int nchunk, bool mirror, const float* __restrict__ Xin,
                                              float* __restrict__ Xout, void* __restrict__ ohi,
-                                             void* __restrict__ olo, double& t1, double& t2) {
+                                             void* __restrict__ olo, uint8_t* turn, double& t1, double& t2) {
   using C = Prec<P>;
   const double w = mirror ? 2.0 : 1.0;  // the transposed copy counts too
+  const int lane = row & 31;
   const size_t gr = (size_t)(m0 + row);
-  const float* xin = Xin + gr * a.ld + n0;
-  float* xout = Xout + gr * a.ld + n0;
+  const size_t w0 = (gr - lane) * a.ld + n0;  // this warp's 32 rows
   char* hrow = static_cast<char*>(ohi) + (gr * a.ld + n0) * C::eb;
   char* lrow = olo ? static_cast<char*>(olo) + (gr * a.ld + n0) * C::eb : hrow;
   // (the X^2 branch needs no X_k: its FP32 master is read only for 2X - X^2;
@@ -150,15 +171,12 @@ __device__ __forceinline__ void sp2_epi_tile(const SP2StepArgs& a, int br, uint3
 #pragma unroll
     for (int j = 0; j < 32; ++j) y[j] = __uint_as_float(v[j]);
     if (br) {
-      const float4* xi = reinterpret_cast<const float4*>(xin + 32 * c);
+      float4 g[8];
+      float x[32];
+      tile_fetch(Xin + w0 + 32 * c, a.ld, lane, g);
+      tile_turn_in(turn, lane, g, x);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const float4 x4 = xi[j];
-        y[4 * j] = fmaf(2.0f, x4.x, -y[4 * j]);
-        y[4 * j + 1] = fmaf(2.0f, x4.y, -y[4 * j + 1]);
-        y[4 * j + 2] = fmaf(2.0f, x4.z, -y[4 * j + 2]);
-        y[4 * j + 3] = fmaf(2.0f, x4.w, -y[4 * j + 3]);
-      }
+      for (int j = 0; j < 32; ++j) y[j] = fmaf(2.0f, x[j], -y[j]);
     }
 #pragma unroll
     for (int j = 0; j < 32; ++j) {
@@ -175,10 +193,8 @@ __device__ __forceinline__ void sp2_epi_tile(const SP2StepArgs& a, int br, uint3
           if (j == dc) t1 += (double)y[j];
       }
     }
-    float4* xo = reinterpret_cast<float4*>(xout + 32 * c);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) xo[j] = make_float4(y[4 * j], y[4 * j + 1], y[4 * j + 2], y[4 * j + 3]);
-    store_operands<P>(y, hrow + 32 * c * C::eb, lrow + 32 * c * C::eb);
+    tile_store(turn, lane, y, Xout + w0 + 32 * c, a.ld);
+    store_rows<P>(turn, lane, y, ohi, olo, w0 + 32 * c, a.ld, hrow + 32 * c * C::eb, lrow + 32 * c * C::eb);
     if (mirror) {
       // element (row, 32c + j) of tile (I, J) is element (32c + j, row) of
       // tile (J, I): for each j the 32 lanes write 32 consecutive values
@@ -208,6 +224,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ int s_dec[3];
   __shared__ volatile int s_abort;
   __shared__ double s_red[4][3];
+  __shared__ __align__(16) uint8_t s_turn[4][4096];  // the epilogue warps' sub-tiles
 
   SP2State* st = a_in.st;
   SP2StepArgs a = a_in;
@@ -362,7 +379,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       tri_tile(t, nt, &I, &J);
       const int m0 = I * BM, n0 = J * BN + (half > 0 ? 64 : 0);
       sp2_epi_tile<P>(a, br, tmem + (static_cast<uint32_t>(32 * q) << 16) + buf * BN, row, m0, n0,
-                      half < 0 ? BN / 32 : 2, I != J, Xin, Xout, ohi, olo, t1, t2);
+                      half < 0 ? BN / 32 : 2, I != J, Xin, Xout, ohi, olo, s_turn[q], t1, t2);
       tc_fence_before();
       if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tempty[buf])) : "memory");
     }
@@ -436,6 +453,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   __shared__ uint32_t s_go;
   __shared__ volatile int s_abort;
   __shared__ double s_red[4][3];
+  __shared__ __align__(16) uint8_t s_turn[4][4096];  // the epilogue warps' sub-tiles
 
   SP2State* st = a_in.st;
   SP2StepArgs a = a_in;
@@ -604,7 +622,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         const int J = half < 0 ? 2 * J2 + h : 2 * J2 + half;
         if (I > J) continue;  // below the diagonal: written as the mirror of (J, I)
         sp2_epi_tile<P>(a, br, tmem + (static_cast<uint32_t>(32 * q) << 16) + buf * BN2 + (half < 0 ? BM * h : 0),
-                        row, I * BM, J * BM, BM / 32, I != J, Xin, Xout, ohi, olo, t1, t2);
+                        row, I * BM, J * BM, BM / 32, I != J, Xin, Xout, ohi, olo, s_turn[q], t1, t2);
       }
       tc_fence_before();
       __syncwarp();
@@ -815,6 +833,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ uint32_t tmem_base;
   __shared__ volatile int s_abort;
   __shared__ double s_red[4];
+  __shared__ __align__(16) uint8_t s_turn[4][4096];  // the epilogue warps' sub-tiles
   if (g.skip && *g.skip) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -914,33 +933,25 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int m0 = I * BM, n0 = J * BN;
       const bool mirror = I != J;
       const size_t gr = (size_t)(m0 + row);
-      const float* erow = g.E ? g.E + gr * g.ld + n0 : nullptr;
-      float* orow = g.out + gr * g.ld + n0;
+      const size_t w0 = (gr - lane) * g.ld + n0;  // this warp's 32 rows
       char* hrow = static_cast<char*>(g.ohi) + (gr * g.ld + n0) * C::eb;
       char* lrow = g.olo ? static_cast<char*>(g.olo) + (gr * g.ld + n0) * C::eb : hrow;
 #pragma unroll 1
       for (int c = 0; c < BN / 32; ++c) {
         uint32_t v[32];
         tmem_ld32(tmem + (static_cast<uint32_t>(32 * q) << 16) + buf * BN + 32 * c, v);
-        // E's row segment: eight 16-byte loads instead of 32 scalar ones
         float es[32];
-        if (erow) {
-          const float4* e4 = reinterpret_cast<const float4*>(erow + 32 * c);
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const float4 t = e4[j];
-            es[4 * j] = t.x;
-            es[4 * j + 1] = t.y;
-            es[4 * j + 2] = t.z;
-            es[4 * j + 3] = t.w;
-          }
+        if (g.E) {
+          float4 eg[8];
+          tile_fetch(g.E + w0 + 32 * c, g.ld, lane, eg);
+          tile_turn_in(s_turn[q], lane, eg, es);
         }
         float y[32];
 #pragma unroll
         for (int j = 0; j < 32; ++j) {
           const int col = n0 + 32 * c + j;
           float val = g.alpha * __uint_as_float(v[j]);
-          if (erow) val = fmaf(g.beta, es[j], val);
+          if (g.E) val = fmaf(g.beta, es[j], val);
           if (col == (int)gr && (int)gr < g.n) val += g.gamma;
           y[j] = val;
         }
@@ -954,10 +965,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         const size_t col0 = (size_t)n0 + 32 * c;
         if (mirror) {
-          float4* xo = reinterpret_cast<float4*>(orow + 32 * c);
-#pragma unroll
-          for (int j = 0; j < 8; ++j) xo[j] = make_float4(y[4 * j], y[4 * j + 1], y[4 * j + 2], y[4 * j + 3]);
-          store_operands<P>(y, hrow + 32 * c * C::eb, lrow + 32 * c * C::eb);
+          tile_store(s_turn[q], lane, y, g.out + w0 + 32 * c, g.ld);
+          store_rows<P>(s_turn[q], lane, y, g.ohi, g.olo, w0 + 32 * c, g.ld, hrow + 32 * c * C::eb,
+                        lrow + 32 * c * C::eb);
 #pragma unroll
           for (int j = 0; j < 32; ++j) {
             const size_t idx = (col0 + j) * g.ld + gr;
