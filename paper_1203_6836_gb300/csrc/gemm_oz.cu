@@ -55,7 +55,8 @@ constexpr int kThreads = 320;
 constexpr int kNacc = 4;       // TMEM accumulators of 128 columns
 
 struct SliceMaps {
-  CUtensorMap m[kS];
+  CUtensorMap m[kS];  // 128-row boxes
+  CUtensorMap b[kS];  // boxes of a unit's rows
 };
 
 __device__ __forceinline__ void pair_of(int p, int* s, int* t) {
@@ -173,6 +174,13 @@ __global__ void __launch_bounds__(kSplitThreads) k_oz_split(const SP2State* st, 
   }
 }
 
+// v 2^e rounded once to FP64, as ldexp((double)v, e) (the conversion rounds; the scale is
+// a factor built from its exponent: exact, or below 2^-1022, where a row whose entries
+// are that small has no digits left to lose, or infinite).
+__device__ __forceinline__ double oz_scaled(long long v, int e) {
+  return (double)v * __hiloint2double((min(max(e, -1022), 1024) + 1023) << 20, 0);
+}
+
 // Row-major upper-triangle tile t -> (I, J), I <= J, of an nt x nt tiling.
 __device__ __forceinline__ void tri_tile(int t, int nt, int* I, int* J) {
   int i = 0;
@@ -184,6 +192,11 @@ __device__ __forceinline__ void tri_tile(int t, int nt, int* I, int* J) {
   *J = i + t;
 }
 
+// NC: columns of a CTA's unit.  A matrix of few tiles is cut into 64- or 32-column units
+// of its 128 x 128 tiles, so that more SMs share the FP64 arithmetic of the epilogue (seven
+// FP64 results an element at 1.7 a clock and SM: 35 us for a whole tile, and twice that
+// before the scale was applied by exponent), the drains and the MMAs.
+template <int NC>
 __global__ void __launch_bounds__(kThreads, 1)
     k_sp2_step_oz(SP2StepArgs a, const __grid_constant__ SliceMaps maps, const int* __restrict__ exps,
                   const double* __restrict__ Xin, double* __restrict__ Xout) {
@@ -237,11 +250,12 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (stop) return;
 
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  // X X is symmetric: CTA b computes upper-triangle tile b and also writes it
-  // transposed
+  // X X is symmetric: CTA b computes unit b of the upper triangle's tiles and also
+  // writes it transposed
+  constexpr int kPer = kTile / NC, kHalf = NC / 2;
   int tI, tJ;
-  tri_tile(blockIdx.x, a.ld / kTile, &tI, &tJ);
-  const int m0 = tI * kTile, n0 = tJ * kTile;
+  tri_tile(blockIdx.x / kPer, a.ld / kTile, &tI, &tJ);
+  const int m0 = tI * kTile, n0 = tJ * kTile + (blockIdx.x % kPer) * NC;
   const bool mirror = tI != tJ;
   const int nk = a.ld / kBK;
 
@@ -257,7 +271,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     s_abort = 0;
     fence_barrier_init();
   }
-  if (warp == 1) tmem_alloc(&tmem_base, kNacc * kTile);
+  if (warp == 1) tmem_alloc(&tmem_base, kNacc * NC);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -274,9 +288,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int stg = g % kStages;
         if (g >= kStages && !mbar_wait(&empty[stg], ((g / kStages) - 1) & 1, &s_abort)) break;
         uint8_t* base = smem + stg * kStageBytes;
-        mbar_expect_tx(&full[stg], kStageBytes);
+        mbar_expect_tx(&full[stg], kTileBytes + NC * 128);
         tma_load_2d(base, &maps.m[s - 1], &full[stg], kb * kBK, m0);
-        tma_load_2d(base + kTileBytes, &maps.m[t - 1], &full[stg], kb * kBK, n0);
+        tma_load_2d(base + kTileBytes, &maps.b[t - 1], &full[stg], kb * kBK, n0);
         issued = g + 1;
       }
     }
@@ -289,13 +303,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp == 1 && lane == 0) {
     // ---------------------------------------------------------- MMA issuer
-    constexpr uint32_t id = idesc(1u);
+    constexpr uint32_t id = idesc(1u, kTile, NC);
     int g = 0;
     for (int p = 0; p < kPairs && !s_abort; ++p) {
       const int acc = p % kNacc;
       if (p >= kNacc && !mbar_wait(&tempty[acc], ((p / kNacc) - 1) & 1, &s_abort)) break;
       tc_fence_after();
-      const uint32_t d = tmem + acc * kTile;
+      const uint32_t d = tmem + acc * NC;
       bool ok = true;
       for (int kb = 0; kb < nk; ++kb, ++g) {
         const int stg = g % kStages;
@@ -319,9 +333,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int q = warp & 3;          // TMEM lane quarter
     const int h = (warp - 2) >> 2;   // column half
     const int row = 32 * q + lane;
-    long long acc64[64];
+    long long acc64[kHalf];
 #pragma unroll
-    for (int j = 0; j < 64; ++j) acc64[j] = 0;
+    for (int j = 0; j < kHalf; ++j) acc64[j] = 0;
     bool ok = true;
     for (int p = 0; p < kPairs && ok; ++p) {
       int s, t;
@@ -339,9 +353,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int lsh = shift > 0 ? shift : 0;
       const float fs = shift >= 0 ? 1.0f : 1.0f / (float)(1 << -shift);
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
+      for (int c = 0; c < kHalf / 16; ++c) {
         uint32_t v[16];
-        tmem_ld16(tmem + (static_cast<uint32_t>(32 * q) << 16) + acc * kTile + 64 * h + 16 * c, v);
+        tmem_ld16(tmem + (static_cast<uint32_t>(32 * q) << 16) + acc * NC + kHalf * h + 16 * c, v);
 #pragma unroll
         for (int j = 0; j < 16; ++j) acc64[16 * c + j] += (long long)__float2int_rn(__uint_as_float(v[j]) * fs) << lsh;
       }
@@ -353,23 +367,24 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (ok) {
       const int gr = m0 + row;
       const int er = exps[gr];
-      const double* xin = Xin + (size_t)gr * a.ld + n0 + 64 * h;
-      double* xout = Xout + (size_t)gr * a.ld + n0 + 64 * h;
-      const int* ec = exps + n0 + 64 * h;
+      const int c0 = n0 + kHalf * h;
+      const double* xin = Xin + (size_t)gr * a.ld + c0;
+      double* xout = Xout + (size_t)gr * a.ld + c0;
+      const int* ec = exps + c0;
       const double w = mirror ? 2.0 : 1.0;  // the transposed copy counts too
       double u2 = 0.0, u3 = 0.0;
 #pragma unroll
-      for (int j = 0; j < 64; ++j) {
-        const double cxx = ldexp((double)acc64[j], er + ec[j] - kBeta * (kS + 1));
+      for (int j = 0; j < kHalf; ++j) {
+        const double cxx = oz_scaled(acc64[j], er + ec[j] - kBeta * (kS + 1));
         const double x = xin[j];
         const double y = br ? 2.0 * x - cxx : cxx;
         xout[j] = y;
-        // element (gr, n0 + 64h + j) is also element (n0 + 64h + j, gr): for
-        // each j the 32 lanes write 32 consecutive values
-        if (mirror) Xout[(size_t)(n0 + 64 * h + j) * a.ld + gr] = y;
-        if (gr == n0 + 64 * h + j) t1 += y;
-        u2 += y * y;
-        u3 += (cxx - x) * (cxx - x);
+        // element (gr, c0 + j) is also element (c0 + j, gr): for each j the 32 lanes
+        // write 32 consecutive values
+        if (mirror) Xout[(size_t)(c0 + j) * a.ld + gr] = y;
+        if (gr == c0 + j) t1 += y;
+        u2 = fma(y, y, u2);
+        u3 = fma(cxx - x, cxx - x, u3);
       }
       t2 = w * u2;
       t3 = w * u3;
@@ -410,7 +425,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
     __syncwarp();
-    tmem_dealloc(tmem, kNacc * kTile);
+    tmem_dealloc(tmem, kNacc * NC);
   }
 }
 
@@ -646,7 +661,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         if (lane == 0) mbar_arrive_cluster(tempty0 + 8u * set);
       }
       if (!ok || I > J) continue;  // below the diagonal: written as the mirror of (J, I)
-      const bool mirror = I != J;
+      const bool mirror = I != J, diag = !mirror;
       const int m0 = I * kTile, n0 = J * kTile;
       const int gr = m0 + row;
       const int er = exps[gr];
@@ -657,14 +672,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       double u2 = 0.0, u3 = 0.0;
 #pragma unroll
       for (int j = 0; j < 64; ++j) {
-        const double cxx = ldexp((double)acc64[j], er + ec[j] - kBeta * (kS + 1));
+        const double cxx = oz_scaled(acc64[j], er + ec[j] - kBeta * (kS + 1));
         const double x = xin[j];
         const double y = br ? 2.0 * x - cxx : cxx;
         xout[j] = y;
         if (mirror) Xout[(size_t)(n0 + 64 * h + j) * a.ld + gr] = y;
-        if (gr == n0 + 64 * h + j) t1 += y;
-        u2 += y * y;
-        u3 += (cxx - x) * (cxx - x);
+        if (diag && gr == n0 + 64 * h + j) t1 += y;
+        u2 = fma(y, y, u2);
+        u3 = fma(cxx - x, cxx - x, u3);
       }
       t2 += w * u2;
       t3 += w * u3;
@@ -727,17 +742,35 @@ int oz_pair_capacity(tb_ctx* ctx) {
   return n;
 }
 
+// Columns of a unit of the single-CTA form: the narrowest whose units all run at once.
+int oz_unit(const tb_ctx* ctx, int ld) {
+  const int nt = ld / kTile, T = nt * (nt + 1) / 2;
+  return 4 * T <= ctx->sm_count ? 32 : 2 * T <= ctx->sm_count ? 64 : 128;
+}
+
 // Clusters of the pair form for this ld (0: the single-CTA form).  The pair
 // form moves half the operand bytes per MMA at the same tile count per SM, so
-// it is taken wherever ld allows unless the single form is forced.
+// it is taken wherever ld allows, except where the single form's narrow units spread the
+// product over more SMs (below ld = 1536) or is forced.
 int oz_pairs(tb_ctx* ctx, int ld) {
   if (ld % (2 * kTile) != 0 || ctx->sp2_form == TB_SP2_FORM_SINGLE) return 0;
+  if (ctx->sp2_form == TB_SP2_FORM_AUTO && oz_unit(ctx, ld) < kTile) return 0;
   int C = oz_pair_capacity(ctx);
   if (ctx->grid_limit > 0) C = std::min(C, ctx->grid_limit / 2);
   const int nt = ld / kTile, nt2 = ld / (2 * kTile);
   const int U = nt * nt2 - nt2 * (nt2 - 1);
   C = std::min(C, U);
   return C > 0 ? C : 0;
+}
+
+template <int NC>
+int launch_oz(tb_ctx* ctx, int grid, const SP2StepArgs& a, const SliceMaps& maps, const int* exps, const double* Xin,
+              double* Xout, cudaStream_t s) {
+  static unsigned long long attr_done = 0;
+  if (int rc = tb_smem_attr(ctx, k_sp2_step_oz<NC>, kSmem, &attr_done)) return rc;
+  k_sp2_step_oz<NC><<<grid, kThreads, kSmem, s>>>(a, maps, exps, Xin, Xout);
+  TB_LAUNCH_CHECK(ctx);
+  return TB_OK;
 }
 
 }  // namespace
@@ -747,15 +780,13 @@ int sp2_oz_num_parts(tb_ctx* ctx, int ld) {
   const int p = oz_pairs(ctx, ld);
   if (p > 0) return 2 * p;
   const int nt = ld / kTile;
-  return nt * (nt + 1) / 2;
+  return nt * (nt + 1) / 2 * (kTile / oz_unit(ctx, ld));
 }
 size_t sp2_oz_slice_bytes(int ld) { return (size_t)kS * ld * ld * sizeof(__nv_bfloat16); }
 
 int sp2_oz_step(tb_ctx* ctx, const SP2StepArgs& a, const double* Xin, double* Xout, void* slices, int* exps,
                 cudaStream_t s) {
   if (a.ld > 4096 || a.ld % kTile) return tb_fail(ctx, TB_ERR_UNSUPPORTED, "emulated FP64 needs ld <= 4096");
-  static unsigned long long attr_done = 0;
-  if (int rc_attr = tb_smem_attr(ctx, k_sp2_step_oz, kSmem, &attr_done)) return rc_attr;
   k_oz_split<<<a.ld, kSplitThreads, 0, s>>>(a.st, Xin, a.ld, static_cast<__nv_bfloat16*>(slices), exps);
   TB_LAUNCH_CHECK(ctx);
   const size_t plane = (size_t)a.ld * a.ld * sizeof(__nv_bfloat16);
@@ -774,13 +805,18 @@ int sp2_oz_step(tb_ctx* ctx, const SP2StepArgs& a, const double* Xin, double* Xo
     TB_LAUNCH_CHECK(ctx);
     return TB_OK;
   }
+  const int nc = oz_unit(ctx, a.ld);
   SliceMaps maps;
   for (int i = 0; i < kS; ++i) {
-    int rc = sp2_tc_make_map(ctx, TB_PREC_BF16, static_cast<char*>(slices) + i * plane, a.ld, &maps.m[i]);
+    const void* sl = static_cast<char*>(slices) + i * plane;
+    int rc = sp2_tc_make_map(ctx, TB_PREC_BF16, sl, a.ld, &maps.m[i], 128, 128);
+    if (!rc) rc = sp2_tc_make_map(ctx, TB_PREC_BF16, sl, a.ld, &maps.b[i], 128, nc);
     if (rc) return rc;
   }
-  const int nt = a.ld / kTile;
-  k_sp2_step_oz<<<nt * (nt + 1) / 2, kThreads, kSmem, s>>>(a, maps, exps, Xin, Xout);
-  TB_LAUNCH_CHECK(ctx);
-  return TB_OK;
+  const int grid = sp2_oz_num_parts(ctx, a.ld);
+  switch (nc) {
+    case 32: return launch_oz<32>(ctx, grid, a, maps, exps, Xin, Xout, s);
+    case 64: return launch_oz<64>(ctx, grid, a, maps, exps, Xin, Xout, s);
+    default: return launch_oz<128>(ctx, grid, a, maps, exps, Xin, Xout, s);
+  }
 }
