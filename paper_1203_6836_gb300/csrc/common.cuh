@@ -159,7 +159,7 @@ struct SP2State {
   unsigned long long rbranch;
   unsigned long long block_products;  // block-sparse path: executed 128^3 block products
   int kc[2];                     // main-phase projection index inside a while graph node
-  unsigned bar;                  // arrivals at the grid barriers of the single-launch form
+  unsigned bar, pad_[31], bar_tr;  // arrivals at the grid barriers of the single-launch forms (own lines)
 };
 
 // Parameters of a purification step shared by the FP64 and tensor-core kernels.

@@ -81,14 +81,15 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_foe_run(const FoeRunArgs a, 
   using Q = RunCfg<P, BN>;
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full[Q::stages], conv[Q::stages], empty[Q::stages], tfull[2], tempty[2], go, mdone;
+  __shared__ __align__(8) uint64_t sfull[Q::bufs], sfree[Q::bufs];
   __shared__ uint32_t tmem_base;
   __shared__ volatile int s_abort;
   __shared__ int s_go;
   __shared__ FoeState fs;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* staging = smem + Q::stages * Q::stage_bytes;
+  const StageRing ring{smem + Q::stages * Q::stage_bytes, sfull, sfree};
   const unsigned G = gridDim.x;
   const RunUnits wu = run_units<BN>(a.ld, (int)G);
   // the CTAs that have units arrive at the barriers (a cluster may have a few more)
@@ -110,6 +111,10 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_foe_run(const FoeRunArgs a, 
       mbar_init(&tfull[b], 1);
       mbar_init(&tempty[b], 8);
     }
+    for (int b = 0; b < Q::bufs; ++b) {
+      mbar_init(&sfull[b], 8);
+      mbar_init(&sfree[b], 1);
+    }
     mbar_init(&go, 1);
     mbar_init(&mdone, 1);
     s_abort = 0;
@@ -125,6 +130,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_foe_run(const FoeRunArgs a, 
   const int np = 2 + m * (2 * a.ns + 2) + 2;
 
   int g = 0, t_mma = 0, t_epi = 0, issued = 0;  // g: stages gone through by this role
+  int used = 0;                                 // arrays put through the staging ring
   uint32_t cpar = 0, gopar = 0;                 // parities of the next conv (a bit per stage) and go phase
   const int mine = (int)blockIdx.x < wu.U ? (wu.U - 1 - (int)blockIdx.x) / (int)G + 1 : 0;  // units of this CTA
   unsigned phase = 0;                           // barrier phases completed before this expansion
@@ -153,31 +159,52 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_foe_run(const FoeRunArgs a, 
           }
         }
       }
-    } else if (warp == 1 && lane == 0) {
-      // ------------------------------------------------------------ MMA issuer
-      for (int p = 0; p < np && !s_abort; ++p) {
-        const Prod r = prod_of(p, m, a.ns);
-        const bool lolo = r.lolo;
-        for (int u = blockIdx.x; u < wu.U && !s_abort; u += G, ++t_mma) {
-          const RunUnit un = run_unit<BN>(wu, u);
-          const uint32_t id = idesc(2u, 128, un.nc);
-          const int buf = t_mma & 1;
-          if (t_mma >= 2 && !mbar_wait(&tempty[buf], ((t_mma >> 1) - 1) & 1, &s_abort, wl)) break;
-          tc_fence_after();
-          for (int kb = 0; kb < nk; ++kb, ++g) {
-            const int s = g % Q::stages;
-            if (r.patch) {
-              if (!mbar_wait(&conv[s], (cpar >> s) & 1, &s_abort, wl)) break;
-              cpar ^= 1u << s;
-            } else if (!mbar_wait(&full[s], (g / Q::stages) & 1, &s_abort, wl)) {
-              break;
-            }
+    } else if (warp == 1) {
+      if (elect_one()) {
+        // ------------------------------------------------------------ MMA issuer
+        const uint32_t lo0 = sdesc_lo(smem_u32(smem));
+        for (int p = 0; p < np && !s_abort; ++p) {
+          const Prod r = prod_of(p, m, a.ns);
+          const bool lolo = r.lolo;
+          for (int u = blockIdx.x; u < wu.U && !s_abort; u += G, ++t_mma) {
+            const RunUnit un = run_unit<BN>(wu, u);
+            const uint32_t id = idesc(2u, 128, un.nc);
+            const int buf = t_mma & 1;
+            if (t_mma >= 2 && !mbar_wait(&tempty[buf], ((t_mma >> 1) - 1) & 1, &s_abort, wl)) break;
             tc_fence_after();
-            stage_mma<P, BN>(smem_u32(smem + s * Q::stage_bytes), tmem + buf * BN, id, kb == 0, lolo);
-            umma_commit(&empty[s]);
+            for (int kb = 0; kb < nk; ++kb, ++g) {
+              const int s = g % Q::stages;
+              if (r.patch) {
+                if (!mbar_wait(&conv[s], (cpar >> s) & 1, &s_abort, wl)) break;
+                cpar ^= 1u << s;
+              } else if (!mbar_wait(&full[s], (g / Q::stages) & 1, &s_abort, wl)) {
+                break;
+              }
+              tc_fence_after();
+              stage_mma<P, BN>(lo0 + s * (Q::stage_bytes >> 4), tmem + buf * BN, id, kb == 0, lolo);
+              umma_commit(&empty[s]);
+            }
+            umma_commit(&tfull[buf]);
           }
-          umma_commit(&tfull[buf]);
         }
+      }
+      __syncwarp();
+    } else if (warp == 11) {
+      // ------------------------------------------------------------ stores
+      for (int p = 0; p < np && lane == 0 && !s_abort; ++p) {
+        const Prod r = prod_of(p, m, a.ns);
+        const bool master = r.kind == kE0 || r.kind == kE || r.kind == kW || r.kind == kEW;
+        const int h0 = master ? 0 : 1, h1 = r.kind == kEW ? 1 : Q::C::split ? 3 : 2;
+        for (int u = blockIdx.x; u < wu.U && !s_abort; u += G) {
+          const RunUnit un = run_unit<BN>(wu, u);
+          for (int c = 0; c < un.nc; c += 32)
+            for (int h = h0; h < h1; ++h)
+              if (!ring_store<P, BN>(ring, used, &mp.a[r.out][h], &mp.s[r.out][h], un.I * 128, un.J * 128 + un.c0 + c,
+                                     un.I == un.J ? (un.c0 + c) >> 5 : kOff, &s_abort, wl))
+                break;
+        }
+        tma_store_wait();
+        if (works && !s_abort) run_arrive(bar);
       }
     } else if (warp == 10) {
       // ------------------------------------------------------------ diagonal patches
@@ -246,16 +273,13 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_foe_run(const FoeRunArgs a, 
         if (eid == 0 && works) run_arrive(bar);
       }
       const int q = warp & 3, half = (warp - 2) >> 2;
-      // (the epilogue warps leave the chain together: epi_any is the same in all)
-      bool stop = false;
-      for (int p = 0; p < np && !stop; ++p) {
+      for (int p = 0; p < np && !s_abort; ++p) {
         const Prod r = prod_of(p, m, a.ns);
         double* const trace = r.kind == kW ? a.partsw : r.kind == kEW ? a.parts3 : a.parts;
         const float al = r.kind == kE0 ? -4.0f / 3.0f : r.kind == kZ1 ? 32.0f / 99.0f : r.kind == kW ? -4.0f : 1.0f;
         const float be = r.kind == kZ1 ? -144.0f / 99.0f : 1.0f;
         const float gam = r.kind == kT ? 2.0f : r.kind == kZ1 ? 210.0f / 99.0f : 0.0f;
         const bool master = r.kind == kE0 || r.kind == kE || r.kind == kW || r.kind == kEW;
-        int used = 0;
         for (int u = blockIdx.x; u < wu.U; u += G, ++t_epi) {
           const int buf = t_epi & 1;
           const RunUnit un = run_unit<BN>(wu, u);
@@ -276,8 +300,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_foe_run(const FoeRunArgs a, 
             }
           };
           if (r.e >= 0) load_e(gr, un.J * 128 + un.c0 + 16 * half);
-          const bool ok = mbar_wait_warp(&tfull[buf], (t_epi >> 1) & 1, &s_abort, wl);
-          if (epi_any(!ok)) break;  // the warps meet in every chunk below
+          if (!mbar_wait_warp(&tfull[buf], (t_epi >> 1) & 1, &s_abort, wl)) break;
           tc_fence_after();
 #pragma unroll 1
           for (int c = 0; c < un.nc; c += 32) {
@@ -297,7 +320,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_foe_run(const FoeRunArgs a, 
               for (int j = 0; j < 16; ++j) y[j] = fmaf(be, ev[j], y[j]);
               if (c + 32 < un.nc) load_e(gr, col0 + 32);
             }
-            const int dk = diag ? (un.c0 + c) >> 5 : -1;
+            const int dk = diag ? (un.c0 + c) >> 5 : kOff;
             if (diag) {
               if (gr < a.n) {
 #pragma unroll
@@ -321,20 +344,14 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_foe_run(const FoeRunArgs a, 
                 }
               }
             }
-            if (master)
-              put_chunk<P, BN>(staging, used, y, q, half, lane, eid == 0, &mp.a[r.out][0], &mp.s[r.out][0], r0, chunk0,
-                               dk);
-            if (r.kind != kEW)
-              put_split<P, BN>(staging, used, y, q, half, lane, eid == 0, mp.a[r.out], mp.s[r.out], r0, chunk0, dk);
+            if (master) ring_put<P, BN>(ring, used, y, q, half, lane, dk, &s_abort, wl);
+            if (r.kind != kEW) ring_put_split<P, BN>(ring, used, y, q, half, lane, dk, &s_abort, wl);
           }
           tc_fence_before();
           __syncwarp();
           if (lane == 0)
             asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tempty[buf])) : "memory");
         }
-        if (eid == 0) tma_store_wait();
-        stop = epi_any(s_abort);
-        if (eid == 0 && works && !stop) run_arrive(bar);
       }
     }
     phase += np + 1;
@@ -398,7 +415,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_foe_run(const FoeRunArgs a, 
     foe_report(&fs, s_abort ? TB_ERR_TIMEOUT : fs.err, a.n, a.nocc, a.tol, a.mu_out, a.rep);
   tc_fence_before();
   if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       // every issued MMA retired (bounded) before TMEM is freed
       umma_commit(&mdone);
       const unsigned long long t0 = gtime();

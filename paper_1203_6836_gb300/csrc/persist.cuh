@@ -9,7 +9,8 @@
 //     step against 0.8)
 // so the operands are stored split, once, and the epilogue stages its chunk and
 // its transpose in shared memory for TMA stores: no global store is scattered, and
-// none needs a proxy fence before the next product's loads.
+// none needs a proxy fence before the next product's loads.  A warp of its own issues
+// and awaits those stores and arrives at the barrier.
 #pragma once
 
 #include "tc_ptx.cuh"
@@ -19,7 +20,8 @@
 namespace tcx {
 
 constexpr int kRunEpi = 256;   // warps 2-9: epilogue
-constexpr int kRunThreads = 64 + kRunEpi + 32;  // warp 0 producer, 1 MMA, 10 diagonal patches
+// warp 0 producer, 1 MMA, 10 diagonal patches or decisions, 11 stores
+constexpr int kRunThreads = 64 + kRunEpi + 64;
 constexpr int kRunChunk = 32 * 1024;  // staging of one 128 x 32 chunk and its transpose
 
 // 128 x BN output units; a stage holds 32 columns of the A rows (128) and of
@@ -181,23 +183,35 @@ __device__ __forceinline__ void patch_diag(uint8_t* tile, int lo_off, int row0, 
   if constexpr (Prec<P>::split) *reinterpret_cast<float*>(p + lo_off) = to_tf32(v - h);
 }
 
-// The MMAs of one stage: a K-slice of 32, in the order of the stored-split
-// kernels (hi hi, hi lo, lo hi, and lo lo for a square), so the sums round alike.
+// One thread of a warp, picked the way the compiler knows to be one (so that what it
+// computes for tcgen05 instructions can stay in uniform registers).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+// sdesc() from its low word: address / 16 and the fixed fields.
+__device__ __forceinline__ uint32_t sdesc_lo(uint32_t saddr) { return ((saddr & 0x3FFFFu) >> 4) | (1u << 16); }
+__device__ __forceinline__ uint64_t sdesc_at(uint32_t lo) {
+  return (static_cast<uint64_t>((1024u >> 4) | (1u << 14) | (2u << 29)) << 32) | lo;
+}
+
+// The MMAs of one stage (lo: descriptor of its first byte): a K-slice of 32, in the
+// order of the stored-split kernels (hi hi, hi lo, lo hi, and lo lo for a square), so
+// the sums round alike.
 template <int P, int BN>
-__device__ __forceinline__ void stage_mma(uint32_t base, uint32_t d, uint32_t id, bool first, bool lolo) {
+__device__ __forceinline__ void stage_mma(uint32_t lo, uint32_t d, uint32_t id, bool first, bool lolo) {
   using C = Prec<P>;
   using Q = RunCfg<P, BN>;
+  constexpr uint32_t kB = Q::a_bytes >> 4, kLo = Q::half_bytes >> 4;
 #pragma unroll
   for (int ks = 0; ks < 4; ++ks) {
-    const uint32_t koff = ks * 32;
-    const uint64_t a0 = sdesc(base + koff), b0 = sdesc(base + Q::a_bytes + koff);
-    umma<true>(d, a0, b0, id, !(first && ks == 0));
+    const uint32_t a = lo + 2 * ks;
+    umma<true>(d, sdesc_at(a), sdesc_at(a + kB), id, !(first && ks == 0));
     if constexpr (C::split) {
-      const uint64_t a1 = sdesc(base + Q::half_bytes + koff);
-      const uint64_t b1 = sdesc(base + Q::half_bytes + Q::a_bytes + koff);
-      umma<true>(d, a0, b1, id, 1u);
-      umma<true>(d, a1, b0, id, 1u);
-      if (lolo) umma<true>(d, a1, b1, id, 1u);
+      umma<true>(d, sdesc_at(a), sdesc_at(a + kLo + kB), id, 1u);
+      umma<true>(d, sdesc_at(a + kLo), sdesc_at(a + kB), id, 1u);
+      if (lolo) umma<true>(d, sdesc_at(a + kLo), sdesc_at(a + kLo + kB), id, 1u);
     }
   }
 }
@@ -254,51 +268,72 @@ __device__ __forceinline__ void store_chunk_diag(const uint8_t* st, const CUtens
   tma_store_commit();
 }
 
-// Stages and stores one array of an epilogue chunk (all 256 epilogue threads),
-// through the next of the staging buffers; `used` counts the arrays stored in this
-// product.  dk < 0: off the diagonal; else chunk dk of a diagonal tile, mirrored
-// from its upper triangle, or (kAsIs) stored as computed.
-constexpr int kAsIs = 4;
+// The staging buffers as a ring between the epilogue warps and the store warp; `used`
+// counts the arrays each side has put through it, over the whole kernel.
+struct StageRing {
+  uint8_t* buf;
+  uint64_t *full, *free;  // 8 epilogue warps have written / the stores have read
+};
+// How a chunk is stored: off the diagonal with its transpose; chunk 0-3 of a diagonal
+// tile, mirrored from its upper triangle; or as it is.
+constexpr int kOff = -1, kAsIs = 4;
+
+// One array of a chunk (all 8 epilogue warps).  (After a wait that gave up the buffer is
+// written all the same: the call fails, and the warps stay together.)
 template <int P, int BN>
-__device__ __forceinline__ void put_chunk(uint8_t* staging, int& used, const float (&y)[16], int q, int half, int lane,
-                                          bool lead, const CUtensorMap* m128, const CUtensorMap* m32, int r0, int c0,
-                                          int dk) {
+__device__ __forceinline__ void ring_put(const StageRing& r, int& used, const float (&y)[16], int q, int half, int lane,
+                                         int mode, volatile int* abort, unsigned long long wl) {
   constexpr int NB = RunCfg<P, BN>::bufs;
-  if (used >= NB) {
-    if (lead) tma_store_read_wait<NB - 1>();
-    epi_sync();
-  }
-  uint8_t* st = staging + (used % NB) * kRunChunk;
-  if (dk < 0 || dk >= kAsIs) stage_chunk(st, y, q, half, lane);
-  else stage_chunk_diag(st, y, q, half, lane, dk);
+  const int b = used % NB;
+  if (used >= NB) mbar_wait_warp(&r.free[b], ((used / NB) - 1) & 1, abort, wl);
+  uint8_t* st = r.buf + b * kRunChunk;
+  if (mode < 0 || mode >= kAsIs) stage_chunk(st, y, q, half, lane);
+  else stage_chunk_diag(st, y, q, half, lane, mode);
   fence_async_shared();
-  epi_sync();
-  if (lead) {
-    if (dk < 0) {
-      store_chunk(st, m128, m32, r0, c0);
-    } else if (dk >= kAsIs) {
-      tma_store_2d(m128, st, c0, r0);
-      tma_store_commit();
-    } else {
-      store_chunk_diag(st, m32, r0, dk);
-    }
-  }
+  __syncwarp();
+  if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&r.full[b])) : "memory");
   ++used;
 }
-// hi and lo of the same.
+// hi and lo of 16 values.
 template <int P, int BN>
-__device__ __forceinline__ void put_split(uint8_t* staging, int& used, const float (&y)[16], int q, int half, int lane,
-                                          bool lead, const CUtensorMap (&m128)[3], const CUtensorMap (&m32)[3], int r0,
-                                          int c0, int dk) {
+__device__ __forceinline__ void ring_put_split(const StageRing& r, int& used, const float (&y)[16], int q, int half,
+                                               int lane, int mode, volatile int* abort, unsigned long long wl) {
   float v[16];
 #pragma unroll
   for (int j = 0; j < 16; ++j) v[j] = to_tf32(y[j]);
-  put_chunk<P, BN>(staging, used, v, q, half, lane, lead, &m128[1], &m32[1], r0, c0, dk);
+  ring_put<P, BN>(r, used, v, q, half, lane, mode, abort, wl);
   if constexpr (Prec<P>::split) {
 #pragma unroll
     for (int j = 0; j < 16; ++j) v[j] = to_tf32(y[j] - v[j]);
-    put_chunk<P, BN>(staging, used, v, q, half, lane, lead, &m128[2], &m32[2], r0, c0, dk);
+    ring_put<P, BN>(r, used, v, q, half, lane, mode, abort, wl);
   }
+}
+// The store warp's side (one thread): issues the array's TMA stores and frees the buffer
+// whose stores have read it.
+template <int P, int BN>
+__device__ __forceinline__ bool ring_store(const StageRing& r, int& used, const CUtensorMap* m128,
+                                           const CUtensorMap* m32, int r0, int c0, int mode, volatile int* abort,
+                                           unsigned long long wl) {
+  constexpr int NB = RunCfg<P, BN>::bufs;
+  const int b = used % NB;
+  if (!mbar_wait(&r.full[b], (used / NB) & 1, abort, wl)) return false;
+  const uint8_t* st = r.buf + b * kRunChunk;
+  if (mode < 0) {
+    store_chunk(st, m128, m32, r0, c0);
+  } else if (mode >= kAsIs) {
+    tma_store_2d(m128, st, c0, r0);
+    tma_store_commit();
+  } else {
+    store_chunk_diag(st, m32, r0, mode);
+  }
+  // the group before the last NB - 1 has been read
+  tma_store_read_wait<NB - 1>();
+  if (used >= NB - 1) {
+    const int f = (used - (NB - 1)) % NB;
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&r.free[f])) : "memory");
+  }
+  ++used;
+  return true;
 }
 
 }  // namespace tcx

@@ -589,6 +589,7 @@ extern "C" int dm_sp2(tb_ctx* ctx, const double* H, int n, double nocc, const tb
       g.parts[b] = slot[b];
     }
     g.bar = &st->bar;
+    g.bar_tr = &st->bar_tr;
     const int rc = sp2_run(ctx, o->precision, g, captured, &ran, s);
     if (rc) return rc;
   }

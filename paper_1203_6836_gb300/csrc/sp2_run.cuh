@@ -13,7 +13,7 @@ struct Sp2RunArgs {
   void* hi[2];
   void* lo[2];
   double* parts[2];     // (Tr X, ||X||_F^2) of each 128 x 32 chunk of the upper triangle
-  unsigned* bar;        // grid barrier counter, zero
+  unsigned *bar, *bar_tr;  // grid barrier counters (operands stored, traces summed), zero
 };
 // Launches it on `s` and sets *ran, or leaves *ran 0 where the launched form is to be
 // used: other precisions, the CTA-pair form, a large captured call.
