@@ -840,7 +840,7 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
   const int br = ep.branch ? (int)((st->branch[a.k >> 6] >> (a.k & 63)) & 1ull) : 0;
   const float alpha = br ? ep.a1 : ep.a0, gamma = br ? ep.g1 : ep.g0;
   const int nu = sy.scal[2];  // upper output blocks, walked in sy.order
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   if (threadIdx.x == 0) {
     for (int s = 0; s < NS; ++s) {
@@ -899,50 +899,54 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
         }
       }
     }
-  } else if (warp == 1 && lane == 0) {
-    constexpr uint32_t id = idesc(C::tf32 ? 2u : 1u);
-    int g = 0, it = 0;
-    for (int u = blockIdx.x; u < nu && !s_abort; u += gridDim.x) {
-      const int o = sy.order[u];
-      const int buf = it & 1;
-      if (it >= 2 && !mbar_wait(&tempty[buf], ((it >> 1) - 1) & 1, &s_abort)) break;
-      tc_fence_after();
-      const uint32_t d = tmem + buf * SB;
-      const int p0 = sy.pair_ptr[o], p1 = sy.pair_ptr[o + 1];
-      bool first = true;
-      for (int p = p0; p < p1 && !s_abort; ++p) {
-        for (int c = 0; c < chunks; ++c, ++g) {
-          const int s = g % NS;
-          if (!mbar_wait(kStaged<P> ? &conv[s] : &full[s], (g / NS) & 1, &s_abort)) break;
-          tc_fence_after();
-          const uint32_t base = smem_u32(smem + s * kNumStageBytes<P>);
-          if constexpr (kStaged<P>) {
-            fs_mma(base, tmem, s, d, id, first, ep.lolo);
-            first = false;
-          } else {
-#pragma unroll
-            for (int ks = 0; ks < C::bk / C::uk; ++ks) {
-              const uint32_t koff = ks * 32;
-              const uint64_t dah = sdesc(base + koff), dbh = sdesc(base + 128 * 128 + koff);
-              umma<C::tf32>(d, dah, dbh, id, first ? 0u : 1u);
+  } else if (warp == 1) {
+    if (elect_one()) {
+      const uint32_t lo0 = sdesc_lo(smem_u32(smem));
+      constexpr uint32_t id = idesc(C::tf32 ? 2u : 1u);
+      int g = 0, it = 0;
+      for (int u = blockIdx.x; u < nu && !s_abort; u += gridDim.x) {
+        const int o = sy.order[u];
+        const int buf = it & 1;
+        if (it >= 2 && !mbar_wait(&tempty[buf], ((it >> 1) - 1) & 1, &s_abort)) break;
+        tc_fence_after();
+        const uint32_t d = tmem + buf * SB;
+        const int p0 = sy.pair_ptr[o], p1 = sy.pair_ptr[o + 1];
+        bool first = true;
+        for (int p = p0; p < p1 && !s_abort; ++p) {
+          for (int c = 0; c < chunks; ++c, ++g) {
+            const int s = g % NS;
+            if (!mbar_wait(kStaged<P> ? &conv[s] : &full[s], (g / NS) & 1, &s_abort)) break;
+            tc_fence_after();
+            const uint32_t base = lo0 + s * (kNumStageBytes<P> >> 4);
+            if constexpr (kStaged<P>) {
+              fs_mma(base, tmem, s, d, id, first, ep.lolo);
               first = false;
-              if constexpr (C::split) {
-                const uint64_t dal = sdesc(base + 2 * 128 * 128 + koff), dbl = sdesc(base + 3 * 128 * 128 + koff);
-                umma<C::tf32>(d, dah, dbl, id, 1u);
-                umma<C::tf32>(d, dal, dbh, id, 1u);
-                // lo x lo: in a square it keeps the diagonal blocks' sums of squares unbiased
-                if (ep.lolo) umma<C::tf32>(d, dal, dbl, id, 1u);
+            } else {
+#pragma unroll
+              for (int ks = 0; ks < C::bk / C::uk; ++ks) {
+                const uint32_t koff = ks * 2;
+                const uint64_t dah = sdesc_at(base + koff), dbh = sdesc_at(base + (kFsTile >> 4) + koff);
+                umma<C::tf32>(d, dah, dbh, id, first ? 0u : 1u);
+                first = false;
+                if constexpr (C::split) {
+                  const uint64_t dal = sdesc_at(base + (2 * kFsTile >> 4) + koff), dbl = sdesc_at(base + (3 * kFsTile >> 4) + koff);
+                  umma<C::tf32>(d, dah, dbl, id, 1u);
+                  umma<C::tf32>(d, dal, dbh, id, 1u);
+                  // lo x lo: in a square it keeps the diagonal blocks' sums of squares unbiased
+                  if (ep.lolo) umma<C::tf32>(d, dal, dbl, id, 1u);
+                }
               }
             }
+            umma_commit(&empty[s]);
           }
-          umma_commit(&empty[s]);
         }
+        umma_commit(&tfull[buf]);
+        ++it;
       }
-      umma_commit(&tfull[buf]);
-      ++it;
+      // arrives once every MMA this thread issued has completed
+      umma_commit(&mdone);
     }
-    // arrives once every MMA this thread issued has completed
-    umma_commit(&mdone);
+    __syncwarp();
   } else if (kStaged<P> && warp >= 6) {
     // converters: warps 6-9 A, 10-13 B
     int g = 0;

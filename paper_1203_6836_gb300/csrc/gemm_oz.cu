@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   SP2State* st = a.st;
   if (st->rdone || st->err) return;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
   if (warp == 0) {
     double x = 0, y = 0, z = 0;
@@ -301,33 +301,37 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
     }
-  } else if (warp == 1 && lane == 0) {
-    // ---------------------------------------------------------- MMA issuer
-    constexpr uint32_t id = idesc(1u, kTile, NC);
-    int g = 0;
-    for (int p = 0; p < kPairs && !s_abort; ++p) {
-      const int acc = p % kNacc;
-      if (p >= kNacc && !mbar_wait(&tempty[acc], ((p / kNacc) - 1) & 1, &s_abort)) break;
-      tc_fence_after();
-      const uint32_t d = tmem + acc * NC;
-      bool ok = true;
-      for (int kb = 0; kb < nk; ++kb, ++g) {
-        const int stg = g % kStages;
-        if (!mbar_wait(&full[stg], (g / kStages) & 1, &s_abort)) {
-          ok = false;
-          break;
-        }
+  } else if (warp == 1) {
+    if (elect_one()) {
+      const uint32_t lo0 = sdesc_lo(smem_u32(smem));
+      // ---------------------------------------------------------- MMA issuer
+      constexpr uint32_t id = idesc(1u, kTile, NC);
+      int g = 0;
+      for (int p = 0; p < kPairs && !s_abort; ++p) {
+        const int acc = p % kNacc;
+        if (p >= kNacc && !mbar_wait(&tempty[acc], ((p / kNacc) - 1) & 1, &s_abort)) break;
         tc_fence_after();
-        const uint32_t base = smem_u32(smem + stg * kStageBytes);
+        const uint32_t d = tmem + acc * NC;
+        bool ok = true;
+        for (int kb = 0; kb < nk; ++kb, ++g) {
+          const int stg = g % kStages;
+          if (!mbar_wait(&full[stg], (g / kStages) & 1, &s_abort)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t base = lo0 + stg * (kStageBytes >> 4);
 #pragma unroll
-        for (int ks = 0; ks < kBK / 16; ++ks) {
-          umma<false>(d, sdesc(base + ks * 32), sdesc(base + kTileBytes + ks * 32), id, (kb | ks) != 0);
+          for (int ks = 0; ks < kBK / 16; ++ks) {
+            umma<false>(d, sdesc_at(base + ks * 2), sdesc_at(base + (kTileBytes >> 4) + ks * 2), id, (kb | ks) != 0);
+          }
+          umma_commit(&empty[stg]);
         }
-        umma_commit(&empty[stg]);
+        umma_commit(&tfull[acc]);
+        if (!ok) break;
       }
-      umma_commit(&tfull[acc]);
-      if (!ok) break;
     }
+    __syncwarp();
   } else if (warp >= 2) {
     // ---------------------------------------------------------- epilogue
     const int q = warp & 3;          // TMEM lane quarter
@@ -484,7 +488,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 
   SP2State* st = a.st;
   const int over = st->rdone || st->err;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
 
   if (warp == 0) {
@@ -589,35 +593,39 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         }
       }
     }
-  } else if (warp == 1 && lane == 0 && rank == 0) {
-    // ---------------------------------------------------------- MMA issuer (even CTA)
-    constexpr uint32_t id = idesc(1u, 256, 128);
-    const unsigned long long wl = a.wait_ns ? a.wait_ns : kWaitNs;
-    int g = 0, gb = 0;
-    for (int u = cl; u < U && !s_abort; u += ncl) {
-      for (int b = 0; b < kBatches && !s_abort; ++b, ++gb) {
-        const int nb = c_batch_n[b];
-        const int set = gb & 1;
-        if (gb >= 2 && !mbar_wait(&tempty[set], ((gb >> 1) - 1) & 1, &s_abort, wl)) break;
-        tc_fence_after();
-        const uint32_t d0 = tmem + 2 * set * kTile;
-        for (int kb = 0; kb < nk; ++kb, ++g) {
-          const int stg = g % kStages2;
-          if (!mbar_wait(&full[stg], (g / kStages2) & 1, &s_abort, wl)) break;
+  } else if (warp == 1) {
+    if (rank == 0 && elect_one()) {
+      const uint32_t lo0 = sdesc_lo(smem_u32(smem));
+      // ---------------------------------------------------------- MMA issuer (even CTA)
+      constexpr uint32_t id = idesc(1u, 256, 128);
+      const unsigned long long wl = a.wait_ns ? a.wait_ns : kWaitNs;
+      int g = 0, gb = 0;
+      for (int u = cl; u < U && !s_abort; u += ncl) {
+        for (int b = 0; b < kBatches && !s_abort; ++b, ++gb) {
+          const int nb = c_batch_n[b];
+          const int set = gb & 1;
+          if (gb >= 2 && !mbar_wait(&tempty[set], ((gb >> 1) - 1) & 1, &s_abort, wl)) break;
           tc_fence_after();
-          const uint32_t base = smem_u32(smem + stg * kStage2);
+          const uint32_t d0 = tmem + 2 * set * kTile;
+          for (int kb = 0; kb < nk; ++kb, ++g) {
+            const int stg = g % kStages2;
+            if (!mbar_wait(&full[stg], (g / kStages2) & 1, &s_abort, wl)) break;
+            tc_fence_after();
+            const uint32_t base = lo0 + stg * (kStage2 >> 4);
 #pragma unroll
-          for (int ks = 0; ks < kBK / 16; ++ks) {
-            const uint64_t ad = sdesc(base + ks * 32);
-            umma_pair<false>(d0, ad, sdesc(base + kTileBytes + ks * 32), id, (kb | ks) != 0);
-            if (nb > 1) umma_pair<false>(d0 + kTile, ad, sdesc(base + kTileBytes + kHalfBytes + ks * 32), id, (kb | ks) != 0);
+            for (int ks = 0; ks < kBK / 16; ++ks) {
+              const uint64_t ad = sdesc_at(base + ks * 2);
+              umma_pair<false>(d0, ad, sdesc_at(base + (kTileBytes >> 4) + ks * 2), id, (kb | ks) != 0);
+              if (nb > 1) umma_pair<false>(d0 + kTile, ad, sdesc_at(base + ((kTileBytes + kHalfBytes) >> 4) + ks * 2), id, (kb | ks) != 0);
+            }
+            umma_commit_pair(&empty[stg], 3);
           }
-          umma_commit_pair(&empty[stg], 3);
+          umma_commit_pair(&tfull[set], 3);
         }
-        umma_commit_pair(&tfull[set], 3);
       }
+      umma_commit_pair(&mdone, 3);
     }
-    umma_commit_pair(&mdone, 3);
+    __syncwarp();
   } else if (warp >= 2) {
     // ---------------------------------------------------------- epilogue (both CTAs)
     const int q = warp & 3;          // TMEM lane quarter

@@ -45,13 +45,6 @@ constexpr int kThreads = 192;
 // 192 KB: three 64 KB stages for the split precisions.  (64-byte slices fit
 // six stages but measured 18% slower per projection at n = 4096: twice the
 // TMA requests of half a cache line each.)
-// Shared-memory descriptor of a K-major tile with `row`-byte swizzle rows.
-template <int ROW>
-__device__ __forceinline__ uint64_t Pipe_sdesc(uint32_t saddr) {
-  if constexpr (ROW == 64) return sdesc64(saddr);
-  else return sdesc(saddr);
-}
-
 template <int P>
 struct Pipe {
   using C = Prec<P>;
@@ -230,7 +223,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   SP2StepArgs a = a_in;
   a.k = sp2_step_index(a_in, st->done || st->err);
   if (st->done || st->err) return;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
   // ---- decision for projection k from the partials of X_k (same in every CTA)
   if (warp == 0) {
@@ -326,44 +319,48 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
     }
-  } else if (warp == 1 && lane == 0) {
-    // ------------------------------------------------------------ MMA issuer
-    constexpr uint32_t id128 = idesc(C::tf32 ? 2u : 1u);
-    constexpr uint32_t id64 = idesc(C::tf32 ? 2u : 1u, 128, 64);
-    int g = 0, it = 0;
-    for (int u = blockIdx.x; u < wu.U && !s_abort; u += gridDim.x, ++it) {
-      int t, half;
-      unit_tile(wu, u, &t, &half);
-      const uint32_t id = half < 0 ? id128 : id64;
-      // a half unit multiplies by rows [64 half, 64 half + 64) of the B tile:
-      // 64 rows into it, a whole number of 8-row swizzle atoms
-      const uint32_t boff = half > 0 ? 64 * Q::row : 0;
-      const int buf = it & 1;
-      if (it >= 2 && !mbar_wait(&tempty[buf], ((it >> 1) - 1) & 1, &s_abort, wl)) break;
-      tc_fence_after();
-      const uint32_t d = tmem + buf * BN;
-      for (int kb = 0; kb < nk; ++kb, ++g) {
-        const int s = g % Q::stages;
-        if (!mbar_wait(&full[s], (g / Q::stages) & 1, &s_abort, wl)) break;
+  } else if (warp == 1) {
+    if (elect_one()) {
+      const uint32_t lo0 = sdesc_lo(smem_u32(smem));
+      // ------------------------------------------------------------ MMA issuer
+      constexpr uint32_t id128 = idesc(C::tf32 ? 2u : 1u);
+      constexpr uint32_t id64 = idesc(C::tf32 ? 2u : 1u, 128, 64);
+      int g = 0, it = 0;
+      for (int u = blockIdx.x; u < wu.U && !s_abort; u += gridDim.x, ++it) {
+        int t, half;
+        unit_tile(wu, u, &t, &half);
+        const uint32_t id = half < 0 ? id128 : id64;
+        // a half unit multiplies by rows [64 half, 64 half + 64) of the B tile:
+        // 64 rows into it, a whole number of 8-row swizzle atoms
+        const uint32_t boff = half > 0 ? (64 * Q::row) >> 4 : 0;
+        const int buf = it & 1;
+        if (it >= 2 && !mbar_wait(&tempty[buf], ((it >> 1) - 1) & 1, &s_abort, wl)) break;
         tc_fence_after();
-        const uint32_t base = smem_u32(smem + s * Q::stage_bytes);
+        const uint32_t d = tmem + buf * BN;
+        for (int kb = 0; kb < nk; ++kb, ++g) {
+          const int s = g % Q::stages;
+          if (!mbar_wait(&full[s], (g / Q::stages) & 1, &s_abort, wl)) break;
+          tc_fence_after();
+          const uint32_t base = lo0 + s * (Q::stage_bytes >> 4);
 #pragma unroll
-        for (int ks = 0; ks < Q::bk / C::uk; ++ks) {
-          const uint32_t koff = ks * 32;
-          const uint64_t ah = Pipe_sdesc<Q::row>(base + koff);
-          const uint64_t bh = Pipe_sdesc<Q::row>(base + Q::tile + boff + koff);
-          umma<C::tf32>(d, ah, bh, id, (kb | ks) != 0);
-          if constexpr (C::split) {
-            umma<C::tf32>(d, ah, Pipe_sdesc<Q::row>(base + 3 * Q::tile + boff + koff), id, 1u);
-            umma<C::tf32>(d, Pipe_sdesc<Q::row>(base + 2 * Q::tile + koff), bh, id, 1u);
+          for (int ks = 0; ks < Q::bk / C::uk; ++ks) {
+            const uint32_t koff = ks * 2;
+            const uint64_t ah = sdesc_at(base + koff);
+            const uint64_t bh = sdesc_at(base + (Q::tile >> 4) + boff + koff);
+            umma<C::tf32>(d, ah, bh, id, (kb | ks) != 0);
+            if constexpr (C::split) {
+              umma<C::tf32>(d, ah, sdesc_at(base + (3 * Q::tile >> 4) + boff + koff), id, 1u);
+              umma<C::tf32>(d, sdesc_at(base + (2 * Q::tile >> 4) + koff), bh, id, 1u);
+            }
           }
+          umma_commit(&empty[s]);
         }
-        umma_commit(&empty[s]);
+        umma_commit(&tfull[buf]);
       }
-      umma_commit(&tfull[buf]);
+      // arrives once every MMA this thread issued has completed
+      umma_commit(&mdone);
     }
-    // arrives once every MMA this thread issued has completed
-    umma_commit(&mdone);
+    __syncwarp();
   } else if (warp >= 2) {
     // ------------------------------------------------------------ epilogue
     double t1 = 0.0, t2 = 0.0, t3 = 0.0;
@@ -459,7 +456,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   SP2StepArgs a = a_in;
   const int over = st->done || st->err;
   a.k = sp2_step_index(a_in, over);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
 
   // ---- decision for projection k (same partials in every CTA); no CTA
@@ -568,41 +565,45 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         }
       }
     }
-  } else if (warp == 1 && lane == 0 && rank == 0) {
-    // ------------------------------------------------------------ MMA issuer (even CTA)
-    constexpr uint32_t idf = idesc(C::tf32 ? 2u : 1u, 256, 256);
-    constexpr uint32_t idh = idesc(C::tf32 ? 2u : 1u, 256, 128);
-    int g = 0, it = 0;
-    for (int u = cl; u < wu.U && !s_abort; u += ncl, ++it) {
-      int t, half;
-      unit_tile(wu, u, &t, &half);
-      const uint32_t id = half < 0 ? idf : idh;
-      const int buf = it & 1;
-      if (it >= 2 && !mbar_wait(&tempty[buf], ((it >> 1) - 1) & 1, &s_abort, wl)) break;
-      tc_fence_after();
-      const uint32_t d = tmem + buf * BN2;
-      for (int kb = 0; kb < nk; ++kb, ++g) {
-        const int s = g % Q::stages;
-        if (!mbar_wait(&full[s], (g / Q::stages) & 1, &s_abort, wl)) break;
+  } else if (warp == 1) {
+    if (rank == 0 && elect_one()) {
+      const uint32_t lo0 = sdesc_lo(smem_u32(smem));
+      // ------------------------------------------------------------ MMA issuer (even CTA)
+      constexpr uint32_t idf = idesc(C::tf32 ? 2u : 1u, 256, 256);
+      constexpr uint32_t idh = idesc(C::tf32 ? 2u : 1u, 256, 128);
+      int g = 0, it = 0;
+      for (int u = cl; u < wu.U && !s_abort; u += ncl, ++it) {
+        int t, half;
+        unit_tile(wu, u, &t, &half);
+        const uint32_t id = half < 0 ? idf : idh;
+        const int buf = it & 1;
+        if (it >= 2 && !mbar_wait(&tempty[buf], ((it >> 1) - 1) & 1, &s_abort, wl)) break;
         tc_fence_after();
-        const uint32_t base = smem_u32(smem + s * Q::stage_bytes);
+        const uint32_t d = tmem + buf * BN2;
+        for (int kb = 0; kb < nk; ++kb, ++g) {
+          const int s = g % Q::stages;
+          if (!mbar_wait(&full[s], (g / Q::stages) & 1, &s_abort, wl)) break;
+          tc_fence_after();
+          const uint32_t base = lo0 + s * (Q::stage_bytes >> 4);
 #pragma unroll
-        for (int ks = 0; ks < Q::bk / C::uk; ++ks) {
-          const uint32_t koff = ks * 32;
-          const uint64_t ah = Pipe_sdesc<Q::row>(base + koff);
-          const uint64_t bh = Pipe_sdesc<Q::row>(base + Q::tile + koff);
-          umma_pair<C::tf32>(d, ah, bh, id, (kb | ks) != 0);
-          if constexpr (C::split) {
-            umma_pair<C::tf32>(d, ah, Pipe_sdesc<Q::row>(base + 3 * Q::tile + koff), id, 1u);
-            umma_pair<C::tf32>(d, Pipe_sdesc<Q::row>(base + 2 * Q::tile + koff), bh, id, 1u);
+          for (int ks = 0; ks < Q::bk / C::uk; ++ks) {
+            const uint32_t koff = ks * 2;
+            const uint64_t ah = sdesc_at(base + koff);
+            const uint64_t bh = sdesc_at(base + (Q::tile >> 4) + koff);
+            umma_pair<C::tf32>(d, ah, bh, id, (kb | ks) != 0);
+            if constexpr (C::split) {
+              umma_pair<C::tf32>(d, ah, sdesc_at(base + (3 * Q::tile >> 4) + koff), id, 1u);
+              umma_pair<C::tf32>(d, sdesc_at(base + (2 * Q::tile >> 4) + koff), bh, id, 1u);
+            }
           }
+          umma_commit_pair(&empty[s], 3);
         }
-        umma_commit_pair(&empty[s], 3);
+        umma_commit_pair(&tfull[buf], 3);
       }
-      umma_commit_pair(&tfull[buf], 3);
+      // arrives (in both CTAs) once every MMA of the pair has completed
+      umma_commit_pair(&mdone, 3);
     }
-    // arrives (in both CTAs) once every MMA of the pair has completed
-    umma_commit_pair(&mdone, 3);
+    __syncwarp();
   } else if (warp >= 2) {
     // ------------------------------------------------------------ epilogue (both CTAs)
     double t1 = 0.0, t2 = 0.0;
@@ -835,7 +836,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ double s_red[4];
   __shared__ __align__(16) uint8_t s_turn[4][4096];  // the epilogue warps' sub-tiles
   if (g.skip && *g.skip) return;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int nt = g.ld / BM;
   const int ntiles = nt * (nt + 1) / 2;
@@ -887,38 +888,42 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
     }
-  } else if (warp == 1 && lane == 0) {
-    constexpr uint32_t id = idesc(C::tf32 ? 2u : 1u);
-    int gk = 0, it = 0;
-    for (int t = blockIdx.x; t < ntiles && !s_abort; t += gridDim.x, ++it) {
-      const int buf = it & 1;
-      if (it >= 2 && !mbar_wait(&tempty[buf], ((it >> 1) - 1) & 1, &s_abort, wl)) break;
-      tc_fence_after();
-      const uint32_t d = tmem + buf * BN;
-      for (int kb = 0; kb < nk; ++kb, ++gk) {
-        const int s = gk % Q::stages;
-        if (!mbar_wait(&full[s], (gk / Q::stages) & 1, &s_abort, wl)) break;
+  } else if (warp == 1) {
+    if (elect_one()) {
+      const uint32_t lo0 = sdesc_lo(smem_u32(smem));
+      constexpr uint32_t id = idesc(C::tf32 ? 2u : 1u);
+      int gk = 0, it = 0;
+      for (int t = blockIdx.x; t < ntiles && !s_abort; t += gridDim.x, ++it) {
+        const int buf = it & 1;
+        if (it >= 2 && !mbar_wait(&tempty[buf], ((it >> 1) - 1) & 1, &s_abort, wl)) break;
         tc_fence_after();
-        const uint32_t base = smem_u32(smem + s * Q::stage_bytes);
+        const uint32_t d = tmem + buf * BN;
+        for (int kb = 0; kb < nk; ++kb, ++gk) {
+          const int s = gk % Q::stages;
+          if (!mbar_wait(&full[s], (gk / Q::stages) & 1, &s_abort, wl)) break;
+          tc_fence_after();
+          const uint32_t base = lo0 + s * (Q::stage_bytes >> 4);
 #pragma unroll
-        for (int ks = 0; ks < Q::bk / C::uk; ++ks) {
-          const uint32_t koff = ks * 32;
-          const uint64_t a0 = Pipe_sdesc<Q::row>(base + koff), b0 = Pipe_sdesc<Q::row>(base + Q::tile + koff);
-          umma<C::tf32>(d, a0, b0, id, (kb | ks) != 0);
-          if constexpr (C::split) {
-            const uint64_t a1 = Pipe_sdesc<Q::row>(base + 2 * Q::tile + koff);
-            const uint64_t b1 = Pipe_sdesc<Q::row>(base + 3 * Q::tile + koff);
-            umma<C::tf32>(d, a0, b1, id, 1u);
-            umma<C::tf32>(d, a1, b0, id, 1u);
-            if (g.lolo) umma<C::tf32>(d, a1, b1, id, 1u);
+          for (int ks = 0; ks < Q::bk / C::uk; ++ks) {
+            const uint32_t koff = ks * 2;
+            const uint64_t a0 = sdesc_at(base + koff), b0 = sdesc_at(base + (Q::tile >> 4) + koff);
+            umma<C::tf32>(d, a0, b0, id, (kb | ks) != 0);
+            if constexpr (C::split) {
+              const uint64_t a1 = sdesc_at(base + (2 * Q::tile >> 4) + koff);
+              const uint64_t b1 = sdesc_at(base + (3 * Q::tile >> 4) + koff);
+              umma<C::tf32>(d, a0, b1, id, 1u);
+              umma<C::tf32>(d, a1, b0, id, 1u);
+              if (g.lolo) umma<C::tf32>(d, a1, b1, id, 1u);
+            }
           }
+          umma_commit(&empty[s]);
         }
-        umma_commit(&empty[s]);
+        umma_commit(&tfull[buf]);
       }
-      umma_commit(&tfull[buf]);
+      // arrives once every MMA this thread issued has completed
+      umma_commit(&mdone);
     }
-    // arrives once every MMA this thread issued has completed
-    umma_commit(&mdone);
+    __syncwarp();
   } else if (warp >= 2) {
     double t1 = 0.0;
     const int q = warp & 3;

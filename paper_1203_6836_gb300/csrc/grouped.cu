@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(FS ? kThreadsFs : kThreads, 1)
   __shared__ unsigned long long s_branch[2];
   __shared__ __align__(16) uint8_t s_turn[4][4096];  // the epilogue warps' sub-tiles
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   if (threadIdx.x == 0) {
     for (int s = 0; s < NS; ++s) {
@@ -299,39 +299,43 @@ __global__ void __launch_bounds__(FS ? kThreadsFs : kThreads, 1)
             }
           }
         }
-      } else if (warp == 1 && lane == 0) {
-        constexpr uint32_t id = idesc(C::tf32 ? 2u : 1u, BM, BN);
-        for (int t = 0; t < ntiles && !s_abort; ++t, ++t_mma) {
-          const int acc = t_mma & 1;
-          if (t_mma >= 2 && !mbar_wait(&tempty[acc], ((t_mma >> 1) - 1) & 1, &s_abort)) break;
-          tc_fence_after();
-          const uint32_t dt = tmem + acc * BN;
-          for (int kb = 0; kb < nk; ++kb, ++g_mma) {
-            const int s = g_mma % NS;
-            if (!mbar_wait(FS ? &conv[s] : &full[s], (g_mma / NS) & 1, &s_abort)) break;
+      } else if (warp == 1) {
+        if (elect_one()) {
+          const uint32_t lo0 = sdesc_lo(smem_u32(smem));
+          constexpr uint32_t id = idesc(C::tf32 ? 2u : 1u, BM, BN);
+          for (int t = 0; t < ntiles && !s_abort; ++t, ++t_mma) {
+            const int acc = t_mma & 1;
+            if (t_mma >= 2 && !mbar_wait(&tempty[acc], ((t_mma >> 1) - 1) & 1, &s_abort)) break;
             tc_fence_after();
-            const uint32_t base = smem_u32(smem + s * kStageBytes);
-            if constexpr (FS) {
-              fs_mma(base, tmem, s, dt, id, kb == 0, true);  // lo*lo too: X X is a square (unbiased diagonal)
-            } else {
+            const uint32_t dt = tmem + acc * BN;
+            for (int kb = 0; kb < nk; ++kb, ++g_mma) {
+              const int s = g_mma % NS;
+              if (!mbar_wait(FS ? &conv[s] : &full[s], (g_mma / NS) & 1, &s_abort)) break;
+              tc_fence_after();
+              const uint32_t base = lo0 + s * (kStageBytes >> 4);
+              if constexpr (FS) {
+                fs_mma(base, tmem, s, dt, id, kb == 0, true);  // lo*lo too: X X is a square (unbiased diagonal)
+              } else {
 #pragma unroll
-              for (int ks = 0; ks < C::bk / C::uk; ++ks) {
-                const uint32_t koff = ks * 32;
-                const uint64_t a0 = sdesc(base + koff), b0 = sdesc(base + G::a_bytes + koff);
-                umma<C::tf32>(dt, a0, b0, id, (kb | ks) != 0);
-                if constexpr (C::split) {
-                  const uint64_t a1 = sdesc(base + G::a_bytes + G::b_bytes + koff);
-                  const uint64_t b1 = sdesc(base + 2 * G::a_bytes + G::b_bytes + koff);
-                  umma<C::tf32>(dt, a0, b1, id, 1u);
-                  umma<C::tf32>(dt, a1, b0, id, 1u);
-                  umma<C::tf32>(dt, a1, b1, id, 1u);  // lo*lo: X X is a square (unbiased diagonal)
+                for (int ks = 0; ks < C::bk / C::uk; ++ks) {
+                  const uint32_t koff = ks * 2;
+                  const uint64_t a0 = sdesc_at(base + koff), b0 = sdesc_at(base + (G::a_bytes >> 4) + koff);
+                  umma<C::tf32>(dt, a0, b0, id, (kb | ks) != 0);
+                  if constexpr (C::split) {
+                    const uint64_t a1 = sdesc_at(base + ((G::a_bytes + G::b_bytes) >> 4) + koff);
+                    const uint64_t b1 = sdesc_at(base + ((2 * G::a_bytes + G::b_bytes) >> 4) + koff);
+                    umma<C::tf32>(dt, a0, b1, id, 1u);
+                    umma<C::tf32>(dt, a1, b0, id, 1u);
+                    umma<C::tf32>(dt, a1, b1, id, 1u);  // lo*lo: X X is a square (unbiased diagonal)
+                  }
                 }
               }
+              umma_commit(&empty[s]);
             }
-            umma_commit(&empty[s]);
+            umma_commit(&tfull[acc]);
           }
-          umma_commit(&tfull[acc]);
         }
+        __syncwarp();
       } else if (FS && warp >= 6) {
         // converters: warps 6-9 A, 10-13 B
         for (int t = 0; t < ntiles && !s_abort; ++t) {

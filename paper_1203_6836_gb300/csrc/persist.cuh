@@ -183,19 +183,6 @@ __device__ __forceinline__ void patch_diag(uint8_t* tile, int lo_off, int row0, 
   if constexpr (Prec<P>::split) *reinterpret_cast<float*>(p + lo_off) = to_tf32(v - h);
 }
 
-// One thread of a warp, picked the way the compiler knows to be one (so that what it
-// computes for tcgen05 instructions can stay in uniform registers).
-__device__ __forceinline__ bool elect_one() {
-  uint32_t p;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
-  return p != 0;
-}
-// sdesc() from its low word: address / 16 and the fixed fields.
-__device__ __forceinline__ uint32_t sdesc_lo(uint32_t saddr) { return ((saddr & 0x3FFFFu) >> 4) | (1u << 16); }
-__device__ __forceinline__ uint64_t sdesc_at(uint32_t lo) {
-  return (static_cast<uint64_t>((1024u >> 4) | (1u << 14) | (2u << 29)) << 32) | lo;
-}
-
 // The MMAs of one stage (lo: descriptor of its first byte): a K-slice of 32, in the
 // order of the stored-split kernels (hi hi, hi lo, lo hi, and lo lo for a square), so
 // the sums round alike.

@@ -111,6 +111,19 @@ __device__ __forceinline__ uint64_t sdesc64(uint32_t saddr) {
   d |= static_cast<uint64_t>(4) << 61;
   return d;
 }
+// One thread of a warp, picked the way the compiler knows to be one (so that what it
+// computes for tcgen05 instructions can stay in uniform registers).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+// sdesc() from its low word: address / 16 and the fixed fields.
+__device__ __forceinline__ uint32_t sdesc_lo(uint32_t saddr) { return ((saddr & 0x3FFFFu) >> 4) | (1u << 16); }
+__device__ __forceinline__ uint64_t sdesc_at(uint32_t lo) {
+  return (static_cast<uint64_t>((1024u >> 4) | (1u << 14) | (2u << 29)) << 32) | lo;
+}
+
 // Instruction descriptor: D = F32, A/B format `fmt` (bf16 = 1, tf32 = 2),
 // both K-major, N x M tile.
 __host__ __device__ constexpr uint32_t idesc(uint32_t fmt, int M = 128, int N = 128) {
@@ -348,13 +361,14 @@ __device__ __forceinline__ void fs_convert_b(uint8_t* stage, int t) {
   // the generic-proxy stores must be visible to the tensor core's reads
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
-// The MMAs of one stage, in the order of the stored-split kernels.
-__device__ __forceinline__ void fs_mma(uint32_t stage, uint32_t tmem, int s, uint32_t d, uint32_t id, bool first,
+// The MMAs of one stage (lo: descriptor of its first byte), in the order of the
+// stored-split kernels.
+__device__ __forceinline__ void fs_mma(uint32_t lo, uint32_t tmem, int s, uint32_t d, uint32_t id, bool first,
                                        bool lolo) {
   const uint32_t ta = tmem + kFsTmemA + 64 * s;
 #pragma unroll
   for (int ks = 0; ks < 4; ++ks) {
-    const uint64_t bh = sdesc(stage + kFsTile + ks * 32), bl = sdesc(stage + 2 * kFsTile + ks * 32);
+    const uint64_t bh = sdesc_at(lo + (kFsTile >> 4) + 2 * ks), bl = sdesc_at(lo + (2 * kFsTile >> 4) + 2 * ks);
     umma_ts_tf32(d, ta + 8 * ks, bh, id, !(first && ks == 0));
     umma_ts_tf32(d, ta + 8 * ks, bl, id, 1u);
     umma_ts_tf32(d, ta + 32 + 8 * ks, bh, id, 1u);
