@@ -124,7 +124,8 @@ struct ModelDev {
   double Bhop[6], Bpair[6];
   double zhop[3], zpair[3];  // A2..A4 of zeta(R) for the bond integrals and phi
   double range;  // reach of the image loops: max(rcut, gcut), or rcut with the Ewald gamma
-  double box;
+  double box, inv_box;
+  double inv_gcut;
   int gamma_form;     // 0: windowed gamma, 1: Ewald-summed Gaussian charges
   double ealpha;      // Ewald splitting (1/A)
   double gwidth;      // Gaussian width c = 2k/(U sqrt(pi))

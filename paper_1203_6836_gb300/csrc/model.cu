@@ -99,6 +99,8 @@ int tb_model_from_params(tb_ctx* ctx, const tb_params* p, double box, ModelDev* 
   m->gamma_form = p->gamma_form;
   m->range = p->gamma_form == 0 ? fmax(p->rcut, p->gamma_cut) : p->rcut;
   m->box = box;
+  m->inv_box = 1.0 / box;
+  m->inv_gcut = p->gamma_form == 0 ? 1.0 / p->gamma_cut : 0.0;
   m->ealpha = p->ewald_alpha > 0.0 ? p->ewald_alpha : 6.5 / fmax(box, 10.0);
   m->gwidth = 2.0 * p->coulomb_k / (p->hubbard_u * sqrt(M_PI));
   m->erange = fmax(6.6 / m->ealpha, 6.6 * m->gwidth);
@@ -173,10 +175,10 @@ __device__ __forceinline__ void gamma_radial(const ModelDev& m, double r, double
     *dg = 0.0;
     return;
   }
-  const double x = r / m.gcut, om = 1.0 - x;
+  const double x = r * m.inv_gcut, om = 1.0 - x;
   const double om3 = om * om * om;
   const double w = om3 * om * (1.0 + 4.0 * x);
-  const double dw = (-4.0 * om3 * (1.0 + 4.0 * x) + 4.0 * om3 * om) / m.gcut;
+  const double dw = (-4.0 * om3 * (1.0 + 4.0 * x) + 4.0 * om3 * om) * m.inv_gcut;
   const double s = rsqrt(r * r + m.a2);
   const double ko = m.kc * s;
   const double dko = -m.kc * r * s * s * s;
@@ -212,10 +214,59 @@ __device__ __forceinline__ bool screen_f32(const double* Ra, const double* Rb, f
   return r2 < lim * lim;
 }
 
+// The same from coordinates already in FP32 (GB300 converts FP64 to FP32 at two values a
+// clock and SM: once per atom, not per pair).
+__device__ __forceinline__ bool screen_xyz(const float* a, const float* b, float L, float range) {
+  float r2 = 0.f;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    float x = b[c] - a[c];
+    x -= L * rintf(x / L);
+    r2 += x * x;
+  }
+  const float lim = range + 0.01f;
+  return r2 < lim * lim;
+}
+
 // Image range along one axis: all k with |d + k L| < range.
 __device__ __forceinline__ void image_range(double d, double L, double range, int* lo, int* hi) {
   *lo = (int)ceil((-range - d) / L);
   *hi = (int)floor((range - d) / L);
+}
+
+// fn(d, r) for every periodic image of b within `range` of a (not a itself when `self`).
+// In a box of at least twice the range only the nearest image can be: no image bounds (six
+// FP64 divisions, about a third of a pair's FP64 work) and the nearest one by a
+// multiplication (where the two roundings could choose differently, at half the box, the
+// image is out of range).
+template <class Fn>
+__device__ __forceinline__ void for_images(const ModelDev& m, double range, const double* Ra, const double* Rb,
+                                           bool self, Fn fn) {
+  if (m.box >= 2.0 * range) {
+    if (self) return;
+    double d[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const double x = Rb[c] - Ra[c];
+      d[c] = x - m.box * rint(x * m.inv_box);
+    }
+    const double r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
+    if (r < range) fn(d, r);
+    return;
+  }
+  double d0[3];
+  min_image(Ra, Rb, m.box, d0);
+  int lo[3], hi[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) image_range(d0[c], m.box, range, &lo[c], &hi[c]);
+  for (int kx = lo[0]; kx <= hi[0]; ++kx)
+    for (int ky = lo[1]; ky <= hi[1]; ++ky)
+      for (int kz = lo[2]; kz <= hi[2]; ++kz) {
+        if (self && kx == 0 && ky == 0 && kz == 0) continue;
+        const double d[3] = {d0[0] + kx * m.box, d0[1] + ky * m.box, d0[2] + kz * m.box};
+        const double r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
+        if (r < range) fn(d, r);
+      }
 }
 
 // --------------------------------------------------------------------------
@@ -243,99 +294,114 @@ __device__ __forceinline__ void sk_block(int ta, int tb, const double l[3], doub
   }
 }
 
-// One thread per unordered atom pair (i <= j): accumulate the hopping block
-// and gamma over all periodic images, write both (i,j) and (j,i) blocks.
+// Unordered atom pairs (i <= j): the hopping block and gamma over all periodic images,
+// written to both (i,j) and (j,i).  A block takes `rows` x 256 pairs: an FP32 screen first,
+// then the pairs in range, from a list, so that the FP64 part (hundreds of
+// instructions at 76 cycles a warp and scheduler) runs with full warps: at 0.1 g/cc one
+// pair in 250 is in range, and a warp of 32 pairs ran all of it for one (1023 atoms in a
+// dilute box: 132 us before).  Few atoms take fewer rows a block: their pairs should
+// spread over the SMs, not fill the warps of one.
+constexpr int kPairI = 16;
+static int pair_rows(int N) { return max(1, min(kPairI, N / 64)); }
 __global__ void __launch_bounds__(256) k_build_pairs(ModelDev m, int N, const int32_t* __restrict__ types,
                                                      const int32_t* __restrict__ offs,
                                                      const double* __restrict__ R,
                                                      double* __restrict__ H, int n,
-                                                     double* __restrict__ G, double* __restrict__ S) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  const int i = blockIdx.y;
-  if (i >= N || j >= N || j < i) return;
-  const double* Ri = R + 3 * i;
-  const double* Rj = R + 3 * j;
-  const int ti = types[i], tj = types[j];
-  const int ni = norb_of(ti), nj = norb_of(tj);
-  const int oi = offs[i], oj = offs[j];
-  double B[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) B[a][b] = 0.0;
-  double Bs[4][4];  // overlap block (S): unit on site, minus the table with s(r) between atoms
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) Bs[a][b] = (i == j && a == b) ? 1.0 : 0.0;
-  const bool ovl = S != nullptr && m.s0 != 0.0;
-  double gsum = (i == j) ? m.U : 0.0;
-  if (S && i == j)
-    for (int a = 0; a < ni; ++a) S[(size_t)(oi + a) * n + (oi + a)] = 1.0;
-  // H, gamma (and S) were zeroed: pairs with no image in range write nothing
-  // (gamma's window and h's tail both end at the cut-off)
-  if (!(screen_f32(Ri, Rj, (float)m.box, (float)m.range) || i == j)) return;
+                                                     double* __restrict__ G, double* __restrict__ S, int rows) {
+  __shared__ int s_list[kPairI * 256];  // i - i0 (high half), j - j0
+  __shared__ float s_R[kPairI][3];
+  __shared__ int s_cnt;
+  const int i0 = blockIdx.y * rows, j0 = blockIdx.x * blockDim.x;
+  if (j0 + (int)blockDim.x <= i0) return;  // every pair has j < i
+  if (threadIdx.x < rows * 3 && i0 + (int)threadIdx.x / 3 < N)
+    s_R[threadIdx.x / 3][threadIdx.x % 3] = (float)R[3 * i0 + threadIdx.x];
+  if (threadIdx.x == 0) s_cnt = 0;
+  __syncthreads();
   {
-    double d0[3];
-    min_image(Ri, Rj, m.box, d0);
-    int lo[3], hi[3];
+    const int j = j0 + threadIdx.x;
+    float x[3] = {0.f, 0.f, 0.f};
+    if (j < N)
+      for (int c = 0; c < 3; ++c) x[c] = (float)R[3 * j + c];
+    for (int k = 0; k < rows; ++k) {
+      const int i = i0 + k;
+      // H, gamma (and S) were zeroed: pairs with no image in range write nothing
+      // (gamma's window and h's tail both end at the cut-off)
+      const bool hit = i < N && j < N && j >= i && (i == j || screen_xyz(s_R[k], x, (float)m.box, (float)m.range));
+      const unsigned mk = __ballot_sync(0xffffffffu, hit);
+      int at = 0;
+      if (mk && (threadIdx.x & 31) == 0) at = atomicAdd(&s_cnt, __popc(mk));
+      at = __shfl_sync(0xffffffffu, at, 0);
+      if (hit) s_list[at + __popc(mk & ((1u << (threadIdx.x & 31)) - 1u))] = (k << 16) | (int)threadIdx.x;
+    }
+  }
+  __syncthreads();
+  const bool ovl = S != nullptr && m.s0 != 0.0;
+  for (int e = threadIdx.x; e < s_cnt; e += blockDim.x) {
+    const int i = i0 + (s_list[e] >> 16), j = j0 + (s_list[e] & 0xffff);
+    const int ti = types[i], tj = types[j];
+    const int ni = norb_of(ti), nj = norb_of(tj);
+    const int oi = offs[i], oj = offs[j];
+    double B[4][4];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) image_range(d0[c], m.box, m.range, &lo[c], &hi[c]);
-    for (int kx = lo[0]; kx <= hi[0]; ++kx)
-      for (int ky = lo[1]; ky <= hi[1]; ++ky)
-        for (int kz = lo[2]; kz <= hi[2]; ++kz) {
-          if (i == j && kx == 0 && ky == 0 && kz == 0) continue;
-          const double d[3] = {d0[0] + kx * m.box, d0[1] + ky * m.box, d0[2] + kz * m.box};
-          const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-          const double r = sqrt(r2);
-          if (r >= m.range) continue;
-          if (m.gamma_form == 0) {
-            double g, dg;
-            gamma_radial(m, r, &g, &dg);
-            gsum += g;
-          }
-          if (r < m.rcut) {
-            double V, dV;
-            hop_radial(m, r, &V, &dV);
-            const double l[3] = {d[0] / r, d[1] / r, d[2] / r};
-            double Bi[4][4];
-            sk_block(ti, tj, l, V, Bi);
-            for (int a = 0; a < ni; ++a)
-              for (int b = 0; b < nj; ++b) B[a][b] += Bi[a][b];
-            if (ovl) {
-              double sv, dsv;
-              ovl_radial(m, r, &sv, &dsv);
-              sk_block(ti, tj, l, sv, Bi);
-              for (int a = 0; a < ni; ++a)
-                for (int b = 0; b < nj; ++b) Bs[a][b] -= Bi[a][b];
-            }
-          }
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) B[a][b] = 0.0;
+    double Bs[4][4];  // overlap block (S): unit on site, minus the table with s(r) between atoms
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) Bs[a][b] = (i == j && a == b) ? 1.0 : 0.0;
+    double gsum = (i == j) ? m.U : 0.0;
+    if (S && i == j)
+      for (int a = 0; a < ni; ++a) S[(size_t)(oi + a) * n + (oi + a)] = 1.0;
+    for_images(m, m.range, R + 3 * i, R + 3 * j, i == j, [&](const double (&d)[3], double r) {
+      if (m.gamma_form == 0) {
+        double g, dg;
+        gamma_radial(m, r, &g, &dg);
+        gsum += g;
+      }
+      if (r < m.rcut) {
+        double V, dV;
+        hop_radial(m, r, &V, &dV);
+        const double ir = 1.0 / r, l[3] = {d[0] * ir, d[1] * ir, d[2] * ir};
+        double Bi[4][4];
+        sk_block(ti, tj, l, V, Bi);
+        for (int a = 0; a < ni; ++a)
+          for (int b = 0; b < nj; ++b) B[a][b] += Bi[a][b];
+        if (ovl) {
+          double sv, dsv;
+          ovl_radial(m, r, &sv, &dsv);
+          sk_block(ti, tj, l, sv, Bi);
+          for (int a = 0; a < ni; ++a)
+            for (int b = 0; b < nj; ++b) Bs[a][b] -= Bi[a][b];
         }
-  }
-  if (i == j) {
-    // onsite energies on the diagonal of the (i,i) block
-    if (ti == TB_TYPE_O) {
-      B[0][0] += m.eps_s_O;
-      B[1][1] += m.eps_p_O;
-      B[2][2] += m.eps_p_O;
-      B[3][3] += m.eps_p_O;
-    } else {
-      B[0][0] += m.eps_s_H;
+      }
+    });
+    if (i == j) {
+      // onsite energies on the diagonal of the (i,i) block
+      if (ti == TB_TYPE_O) {
+        B[0][0] += m.eps_s_O;
+        B[1][1] += m.eps_p_O;
+        B[2][2] += m.eps_p_O;
+        B[3][3] += m.eps_p_O;
+      } else {
+        B[0][0] += m.eps_s_H;
+      }
     }
-  }
-  for (int a = 0; a < ni; ++a)
-    for (int b = 0; b < nj; ++b) {
-      H[(size_t)(oi + a) * n + (oj + b)] = B[a][b];
-      if (i != j) H[(size_t)(oj + b) * n + (oi + a)] = B[a][b];
-    }
-  G[(size_t)i * N + j] = gsum;
-  if (i != j) G[(size_t)j * N + i] = gsum;
-  if (ovl)
     for (int a = 0; a < ni; ++a)
       for (int b = 0; b < nj; ++b) {
-        S[(size_t)(oi + a) * n + (oj + b)] = Bs[a][b];
-        if (i != j) S[(size_t)(oj + b) * n + (oi + a)] = Bs[a][b];
+        H[(size_t)(oi + a) * n + (oj + b)] = B[a][b];
+        if (i != j) H[(size_t)(oj + b) * n + (oi + a)] = B[a][b];
       }
+    G[(size_t)i * N + j] = gsum;
+    if (i != j) G[(size_t)j * N + i] = gsum;
+    if (ovl)
+      for (int a = 0; a < ni; ++a)
+        for (int b = 0; b < nj; ++b) {
+          S[(size_t)(oi + a) * n + (oj + b)] = Bs[a][b];
+          if (i != j) S[(size_t)(oj + b) * n + (oi + a)] = Bs[a][b];
+        }
+  }
 }
 
 // --------------------------------------------------------------------------
@@ -535,8 +601,9 @@ extern "C" int tb_build_H(tb_ctx* ctx, const tb_params* p, const tb_system* sys,
   const int N = sys->natoms, n = sys->norb;
   TB_CUDA_TRY(ctx, cudaMemsetAsync(H, 0, sizeof(double) * (size_t)n * n, s));
   TB_CUDA_TRY(ctx, cudaMemsetAsync(gamma, 0, sizeof(double) * (size_t)N * N, s));
-  dim3 grid((N + 255) / 256, N);
-  k_build_pairs<<<grid, 256, 0, s>>>(m, N, sys->types, sys->orb_off, R, H, n, gamma, nullptr);
+  const int rows = pair_rows(N);
+  dim3 grid((N + 255) / 256, (N + rows - 1) / rows);
+  k_build_pairs<<<grid, 256, 0, s>>>(m, N, sys->types, sys->orb_off, R, H, n, gamma, nullptr, rows);
   TB_LAUNCH_CHECK(ctx);
   if (m.gamma_form == 1) {
     k_gamma_ewald<<<dim3((N + kGChunk - 1) / kGChunk, N), kGChunk, 0, s>>>(m, N, R, gamma);
@@ -601,8 +668,9 @@ extern "C" int tb_build_HS(tb_ctx* ctx, const tb_params* p, const tb_system* sys
   TB_CUDA_TRY(ctx, cudaMemsetAsync(H, 0, sizeof(double) * (size_t)n * n, s));
   TB_CUDA_TRY(ctx, cudaMemsetAsync(S, 0, sizeof(double) * (size_t)n * n, s));
   TB_CUDA_TRY(ctx, cudaMemsetAsync(gamma, 0, sizeof(double) * (size_t)N * N, s));
-  dim3 grid((N + 255) / 256, N);
-  k_build_pairs<<<grid, 256, 0, s>>>(m, N, sys->types, sys->orb_off, R, H, n, gamma, S);
+  const int rows = pair_rows(N);
+  dim3 grid((N + 255) / 256, (N + rows - 1) / rows);
+  k_build_pairs<<<grid, 256, 0, s>>>(m, N, sys->types, sys->orb_off, R, H, n, gamma, S, rows);
   TB_LAUNCH_CHECK(ctx);
   if (m.gamma_form == 1) {
     k_gamma_ewald<<<dim3((N + kGChunk - 1) / kGChunk, N), kGChunk, 0, s>>>(m, N, R, gamma);
@@ -700,9 +768,10 @@ __device__ __forceinline__ void band_pair_g(int ta, int tb, Get Dg, const double
 #pragma unroll
     for (int c = 0; c < 3; ++c) u[c] -= Dg(1 + c, 0);
   const double ul = u[0] * l[0] + u[1] * l[1] + u[2] * l[2];
+  const double Vr = V / r;
   double E = -V * Dss + V * ul;
 #pragma unroll
-  for (int k = 0; k < 3; ++k) g[k] = -dV * Dss * l[k] + V * (u[k] - ul * l[k]) / r + dV * ul * l[k];
+  for (int k = 0; k < 3; ++k) g[k] = -dV * Dss * l[k] + Vr * (u[k] - ul * l[k]) + dV * ul * l[k];
   if (ta == TB_TYPE_O && tb == TB_TYPE_O) {
     double P[3][3];
 #pragma unroll
@@ -717,7 +786,7 @@ __device__ __forceinline__ void band_pair_g(int ta, int tb, Get Dg, const double
     const double lSl = l[0] * Sl[0] + l[1] * Sl[1] + l[2] * Sl[2];  // = 2 l^T P l
     E += V * lSl - V * trP;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) g[k] += 2.0 * V * (Sl[k] - lSl * l[k]) / r + dV * lSl * l[k] - dV * trP * l[k];
+    for (int k = 0; k < 3; ++k) g[k] += 2.0 * Vr * (Sl[k] - lSl * l[k]) + dV * lSl * l[k] - dV * trP * l[k];
   }
   *Eblk = E;
 }
@@ -764,60 +833,49 @@ __global__ void __launch_bounds__(256) k_forces(ModelDev m, int N, const int32_t
     const int tb = types[b], ob = offs[b];
     const double wb = 2.0 * q[b] - n_aux[b];
     const double nb = n_aux[b];
-    double d0[3];
-    min_image(Ra, Rb, m.box, d0);
-    int lo[3], hi[3];
+    for_images(m, m.range, Ra, Rb, b == a, [&](const double (&d)[3], double r) {
+      const double ir = 1.0 / r, l[3] = {d[0] * ir, d[1] * ir, d[2] * ir};
+      if (r < m.rcut) {
+        double V, dV;
+        hop_radial(m, r, &V, &dV);
+        double Eblk, g[3];
+        band_pair(ta, tb, D, n, oa, ob, l, r, V, dV, &Eblk, g);
+        if (b != a) {
+          // unordered pair energy 4*Eblk, shared half per atom
+          e_band += 2.0 * Eblk;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) image_range(d0[c], m.box, m.range, &lo[c], &hi[c]);
-    for (int kx = lo[0]; kx <= hi[0]; ++kx)
-      for (int ky = lo[1]; ky <= hi[1]; ++ky)
-        for (int kz = lo[2]; kz <= hi[2]; ++kz) {
-          if (b == a && kx == 0 && ky == 0 && kz == 0) continue;
-          const double d[3] = {d0[0] + kx * m.box, d0[1] + ky * m.box, d0[2] + kz * m.box};
-          const double r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-          if (r >= m.range) continue;
-          const double l[3] = {d[0] / r, d[1] / r, d[2] / r};
-          if (r < m.rcut) {
-            double V, dV;
-            hop_radial(m, r, &V, &dV);
-            double Eblk, g[3];
-            band_pair(ta, tb, D, n, oa, ob, l, r, V, dV, &Eblk, g);
-            if (b != a) {
-              // unordered pair energy 4*Eblk, shared half per atom
-              e_band += 2.0 * Eblk;
-#pragma unroll
-              for (int k = 0; k < 3; ++k) f[k] += 4.0 * g[k];
-            } else {
-              e_band += 2.0 * Eblk;  // self-image block of h_aa
-            }
-            if constexpr (OVL) if (b != a) {
-              // overlap terms: Tr[(V rho + rho V - 2 W) S] over the blocks (a,b) and
-              // (b,a); S's block is minus the table with s(r), and V is v_a, v_b on
-              // the two atoms' orbitals
-              double sv, dsv, Er, Ew, gr[3], gw[3];
-              ovl_radial(m, r, &sv, &dsv);
-              band_pair(ta, tb, D, n, oa, ob, l, r, sv, dsv, &Er, gr);
-              band_pair(ta, tb, W, n, oa, ob, l, r, sv, dsv, &Ew, gw);
-              const double vv = vscc[a] + vscc[b];
-#pragma unroll
-              for (int k = 0; k < 3; ++k) f[k] -= 2.0 * (vv * gr[k] - 2.0 * gw[k]);
-            }
-            double ph, dph;
-            pair_radial(m, r, &ph, &dph);
-            e_pair += 0.5 * ph;
-            if (b != a)
-#pragma unroll
-              for (int k = 0; k < 3; ++k) f[k] += dph * l[k];
-          }
-          if (b != a && m.gamma_form == 0) {
-            double gg, dgg;
-            gamma_radial(m, r, &gg, &dgg);
-            const double c = 0.5 * (wa * nb + wb * na) * dgg;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) f[k] += c * l[k];
-          }
+          for (int k = 0; k < 3; ++k) f[k] += 4.0 * g[k];
+        } else {
+          e_band += 2.0 * Eblk;  // self-image block of h_aa
         }
-    };
+        if constexpr (OVL) if (b != a) {
+          // overlap terms: Tr[(V rho + rho V - 2 W) S] over the blocks (a,b) and
+          // (b,a); S's block is minus the table with s(r), and V is v_a, v_b on
+          // the two atoms' orbitals
+          double sv, dsv, Er, Ew, gr[3], gw[3];
+          ovl_radial(m, r, &sv, &dsv);
+          band_pair(ta, tb, D, n, oa, ob, l, r, sv, dsv, &Er, gr);
+          band_pair(ta, tb, W, n, oa, ob, l, r, sv, dsv, &Ew, gw);
+          const double vv = vscc[a] + vscc[b];
+#pragma unroll
+          for (int k = 0; k < 3; ++k) f[k] -= 2.0 * (vv * gr[k] - 2.0 * gw[k]);
+        }
+        double ph, dph;
+        pair_radial(m, r, &ph, &dph);
+        e_pair += 0.5 * ph;
+        if (b != a)
+#pragma unroll
+          for (int k = 0; k < 3; ++k) f[k] += dph * l[k];
+      }
+      if (b != a && m.gamma_form == 0) {
+        double gg, dgg;
+        gamma_radial(m, r, &gg, &dgg);
+        const double c = 0.5 * (wa * nb + wb * na) * dgg;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) f[k] += c * l[k];
+      }
+    });
+  };
   int cnt = 0;
   for (int b0 = 0; b0 < N; b0 += 32) {
     const int b = b0 + lane;
@@ -1105,6 +1163,11 @@ __device__ __forceinline__ bool box_in_range(const ModelDev& m, const BsrModelWs
   return g2 < reach * reach;
 }
 
+constexpr int kPairList = 4096;
+// Bound by the 64-bit work of the pairs in range (few of a block's pairs) and by the stores
+// of the zeroed blocks: 959 us with every warp running the pairs' branch for whichever of
+// its lanes were in range and the six divisions of the image bounds, 363 us with the list
+// (16383 orbitals, 0.1 g/cc).
 // The h elements of stored block o (one CTA per block, grid-stride): every
 // ordered atom pair (i, j) of the two rows, summed over the images within the
 // cut-off, onsite energies for i == j; each element belongs to one pair.
@@ -1112,7 +1175,8 @@ __global__ void __launch_bounds__(256) k_h_blocks(ModelDev m, int N, const int32
                                                   const int32_t* __restrict__ offs, const double* __restrict__ R,
                                                   BsrModelWs w, tb_bsr H) {
   __shared__ int s_near[kBB];  // a block row holds at most kBB atoms (each has an orbital in it)
-  __shared__ int s_nnear;
+  __shared__ int s_nnear, s_cnt;
+  __shared__ int s_list[kPairList];
   if (*H.status != TB_OK) return;
   const int nblk = H.row_ptr[H.nsb];
   for (int o = blockIdx.x; o < nblk; o += gridDim.x) {
@@ -1124,7 +1188,12 @@ __global__ void __launch_bounds__(256) k_h_blocks(ModelDev m, int N, const int32
     }
     const int I = lo, J = H.col[o];
     double* blk = H.val + (size_t)o * kBB * kBB;
-    for (int e = threadIdx.x; e < kBB * kBB; e += blockDim.x) blk[e] = 0.0;
+    if ((reinterpret_cast<uintptr_t>(blk) & 15) == 0) {  // a caller's array may be aligned to 8 bytes only
+      double2* blk2 = reinterpret_cast<double2*>(blk);
+      for (int e = threadIdx.x; e < kBB * kBB / 2; e += blockDim.x) blk2[e] = make_double2(0.0, 0.0);
+    } else {
+      for (int e = threadIdx.x; e < kBB * kBB; e += blockDim.x) blk[e] = 0.0;
+    }
     __syncthreads();
     const int ilo = w.atom_lo[I], ihi = w.atom_hi[I], jlo = w.atom_lo[J], jhi = w.atom_hi[J];
     // the atoms of row block I within range of column block J's atom box (the
@@ -1147,87 +1216,122 @@ __global__ void __launch_bounds__(256) k_h_blocks(ModelDev m, int N, const int32
     __syncthreads();
     const int nj = jhi - jlo, npair = s_nnear * nj;
     const int r0 = I * kBB, c0 = J * kBB;
-    for (int p = threadIdx.x; p < npair; p += blockDim.x) {
-      const int i = s_near[p / nj], j = jlo + p % nj;
-      const int ti = types[i], tj = types[j];
-      const int ni = norb_of(ti), njo = norb_of(tj);
-      const int oi = offs[i], oj = offs[j];
-      double B[4][4];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) B[a][b] = 0.0;
-      const double* Ri = R + 3 * i;
-      const double* Rj = R + 3 * j;
-      if (i == j || screen_f32(Ri, Rj, (float)m.box, (float)m.rcut)) {
-        double d0[3];
-        min_image(Ri, Rj, m.box, d0);
-        int lo3[3], hi3[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) image_range(d0[c], m.box, m.rcut, &lo3[c], &hi3[c]);
-        for (int kx = lo3[0]; kx <= hi3[0]; ++kx)
-          for (int ky = lo3[1]; ky <= hi3[1]; ++ky)
-            for (int kz = lo3[2]; kz <= hi3[2]; ++kz) {
-              if (i == j && kx == 0 && ky == 0 && kz == 0) continue;
-              const double d[3] = {d0[0] + kx * m.box, d0[1] + ky * m.box, d0[2] + kz * m.box};
-              const double r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-              if (r >= m.rcut) continue;
-              double V, dV;
-              hop_radial(m, r, &V, &dV);
-              const double l[3] = {d[0] / r, d[1] / r, d[2] / r};
-              double Bi[4][4];
-              sk_block(ti, tj, l, V, Bi);
-              for (int a = 0; a < ni; ++a)
-                for (int b = 0; b < njo; ++b) B[a][b] += Bi[a][b];
-            }
+    // the pairs in range are listed by an FP32 screen and worked through by full warps
+    for (int p0 = 0; p0 < npair; p0 += kPairList) {
+      const int p1 = min(npair, p0 + kPairList);
+      if (threadIdx.x == 0) s_cnt = 0;
+      __syncthreads();
+      for (int pb = p0; pb < p1; pb += blockDim.x) {
+        const int p = pb + threadIdx.x;
+        bool hit = false;
+        int ia = 0, ja = 0;
+        if (p < p1) {
+          ia = p / nj;
+          ja = p - ia * nj;
+          const int i = s_near[ia], j = jlo + ja;
+          hit = i == j || screen_f32(R + 3 * i, R + 3 * j, (float)m.box, (float)m.rcut);
+        }
+        const unsigned mk = __ballot_sync(0xffffffffu, hit);
+        int at = 0;
+        if (mk && (threadIdx.x & 31) == 0) at = atomicAdd(&s_cnt, __popc(mk));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (hit) s_list[at + __popc(mk & ((1u << (threadIdx.x & 31)) - 1u))] = (ia << 16) | ja;
       }
-      if (i == j) {
-        if (ti == TB_TYPE_O) {
-          B[0][0] += m.eps_s_O;
-          B[1][1] += m.eps_p_O;
-          B[2][2] += m.eps_p_O;
-          B[3][3] += m.eps_p_O;
-        } else {
-          B[0][0] += m.eps_s_H;
+      __syncthreads();
+      for (int e = threadIdx.x; e < s_cnt; e += blockDim.x) {
+        const int i = s_near[s_list[e] >> 16], j = jlo + (s_list[e] & 0xffff);
+        const int ti = types[i], tj = types[j];
+        const int ni = norb_of(ti), njo = norb_of(tj);
+        const int oi = offs[i], oj = offs[j];
+        double B[4][4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int b = 0; b < 4; ++b) B[a][b] = 0.0;
+        for_images(m, m.rcut, R + 3 * i, R + 3 * j, i == j, [&](const double (&d)[3], double r) {
+          double V, dV;
+          hop_radial(m, r, &V, &dV);
+          const double ir = 1.0 / r, l[3] = {d[0] * ir, d[1] * ir, d[2] * ir};
+          double Bi[4][4];
+          sk_block(ti, tj, l, V, Bi);
+          for (int a = 0; a < ni; ++a)
+            for (int b = 0; b < njo; ++b) B[a][b] += Bi[a][b];
+        });
+        if (i == j) {
+          if (ti == TB_TYPE_O) {
+            B[0][0] += m.eps_s_O;
+            B[1][1] += m.eps_p_O;
+            B[2][2] += m.eps_p_O;
+            B[3][3] += m.eps_p_O;
+          } else {
+            B[0][0] += m.eps_s_H;
+          }
+        }
+        for (int a = 0; a < ni; ++a) {
+          const int r = oi + a - r0;
+          if (r < 0 || r >= kBB) continue;
+          for (int b = 0; b < njo; ++b) {
+            const int c = oj + b - c0;
+            if (c < 0 || c >= kBB) continue;
+            blk[(size_t)r * kBB + c] = B[a][b];
+          }
         }
       }
-      for (int a = 0; a < ni; ++a) {
-        const int r = oi + a - r0;
-        if (r < 0 || r >= kBB) continue;
-        for (int b = 0; b < njo; ++b) {
-          const int c = oj + b - c0;
-          if (c < 0 || c >= kBB) continue;
-          blk[(size_t)r * kBB + c] = B[a][b];
-        }
-      }
+      __syncthreads();
     }
     __syncthreads();
   }
 }
 
-// Visit the atoms of the stored block columns of row I once each (consecutive
-// block rows share at most their straddling atom): fn(j), skipping the blocks
-// whose atom box lies beyond m.range of the point x (their atoms, the
-// straddling one included, are out of range and contribute nothing).  The
-// lanes test 32 blocks at a time.
+// Visiting the atoms of the stored block columns of row I once each (consecutive
+// block rows share at most their straddling atom) skips the blocks whose atom box lies
+// beyond m.range of the point (their atoms, the straddling one included, are out of
+// range and contribute nothing).
+// The atoms whose nearest image passes the FP32 screen of atom i, each once, through a
+// warp's list (kNbList entries): fn(j) by full warps, a list at a time, each lane taking
+// its entries in list order.  A warp that ran fn for the lanes in range of each 32 atoms
+// spent most of its 64-bit issue on masked lanes: k_v_bsr 662 -> 213 us and k_forces_bsr
+// 926 -> 483 us at 16383 orbitals (with for_images' short form).
+constexpr int kNbList = 256;
 template <class Fn>
-__device__ __forceinline__ void for_neighbour_atoms(const tb_bsr& H, const BsrModelWs& w, const ModelDev& m, int I,
-                                                    const double* x, int lane, Fn fn) {
-  const float xf[3] = {(float)x[0], (float)x[1], (float)x[2]};
+__device__ __forceinline__ void for_atoms_in_range(const tb_bsr& H, const BsrModelWs& w, const ModelDev& m, int I,
+                                                   int i, const double* __restrict__ R, float range, int lane,
+                                                   int* list, Fn fn) {
+  const float xi[3] = {(float)R[3 * i], (float)R[3 * i + 1], (float)R[3 * i + 2]};
+  int cnt = 0;
+  auto flush = [&]() {
+    __syncwarp();
+    for (int e = lane; e < cnt; e += 32) fn(list[e]);
+    __syncwarp();
+    cnt = 0;
+  };
   const int s1 = H.row_ptr[I + 1];
   int next = 0;
   for (int s0 = H.row_ptr[I]; s0 < s1; s0 += 32) {
-    const bool near = s0 + lane < s1 && box_in_range(m, w, H.col[s0 + lane], xf);
-    const unsigned mask = __ballot_sync(0xffffffffu, near);
-    const int cnt = min(32, s1 - s0);
-    for (int t = 0; t < cnt; ++t) {
-      const int J = H.col[s0 + t];
-      const int lo = max(next, w.atom_lo[J]), hi = w.atom_hi[J];
+    // the lanes test 32 blocks at a time, and hold their atom ranges
+    const int J = s0 + lane < s1 ? H.col[s0 + lane] : 0;
+    const int lo0 = w.atom_lo[J], hi0 = w.atom_hi[J];
+    const unsigned mask = __ballot_sync(0xffffffffu, s0 + lane < s1 && box_in_range(m, w, J, xi));
+    const int cntb = min(32, s1 - s0);
+    for (int t = 0; t < cntb; ++t) {
+      const int lo = max(next, __shfl_sync(0xffffffffu, lo0, t)), hi = __shfl_sync(0xffffffffu, hi0, t);
       if ((mask >> t) & 1u)
-        for (int j = lo + lane; j < hi; j += 32) fn(j);
+        for (int j0 = lo; j0 < hi; j0 += 32) {
+          const int j = j0 + lane;
+          bool hit = false;
+          if (j < hi) {
+            const float xj[3] = {(float)R[3 * j], (float)R[3 * j + 1], (float)R[3 * j + 2]};
+            hit = j == i || screen_xyz(xi, xj, (float)m.box, range);
+          }
+          const unsigned mk = __ballot_sync(0xffffffffu, hit);
+          if (hit) list[cnt + __popc(mk & ((1u << lane) - 1u))] = j;
+          cnt += __popc(mk);
+          if (cnt > kNbList - 32) flush();
+        }
       next = max(next, hi);
     }
   }
+  flush();
 }
 
 // v_i = sum_l gamma_il n_l over the atoms within range (windowed gamma, its
@@ -1235,31 +1339,18 @@ __device__ __forceinline__ void for_neighbour_atoms(const tb_bsr& H, const BsrMo
 __global__ void __launch_bounds__(256) k_v_bsr(ModelDev m, int N, const int32_t* __restrict__ offs,
                                                const double* __restrict__ R, const double* __restrict__ n_aux,
                                                tb_bsr H, BsrModelWs w, double* __restrict__ v) {
+  __shared__ int s_list[8][kNbList];
   const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (i >= N || *H.status != TB_OK) return;  // an overflowed pattern has no columns to visit
-  const double* Ri = R + 3 * i;
   double s = 0.0;
-  for_neighbour_atoms(H, w, m, offs[i] / kBB, Ri, lane, [&](int j) {
-    const double* Rj = R + 3 * j;
-    if (j != i && !screen_f32(Ri, Rj, (float)m.box, (float)m.gcut)) return;
-    double d0[3];
-    min_image(Ri, Rj, m.box, d0);
-    int lo3[3], hi3[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) image_range(d0[c], m.box, m.gcut, &lo3[c], &hi3[c]);
+  for_atoms_in_range(H, w, m, offs[i] / kBB, i, R, (float)m.gcut, lane, s_list[threadIdx.x >> 5], [&](int j) {
     double g = 0.0;
-    for (int kx = lo3[0]; kx <= hi3[0]; ++kx)
-      for (int ky = lo3[1]; ky <= hi3[1]; ++ky)
-        for (int kz = lo3[2]; kz <= hi3[2]; ++kz) {
-          if (j == i && kx == 0 && ky == 0 && kz == 0) continue;
-          const double d[3] = {d0[0] + kx * m.box, d0[1] + ky * m.box, d0[2] + kz * m.box};
-          const double r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-          if (r >= m.gcut) continue;
-          double gg, dgg;
-          gamma_radial(m, r, &gg, &dgg);
-          g += gg;
-        }
+    for_images(m, m.gcut, R + 3 * i, R + 3 * j, j == i, [&](const double (&)[3], double r) {
+      double gg, dgg;
+      gamma_radial(m, r, &gg, &dgg);
+      g += gg;
+    });
     s += g * n_aux[j];
   });
   s = warp_sum(s);
@@ -1286,12 +1377,13 @@ __global__ void k_mulliken_bsr(int N, const int32_t* __restrict__ types, const i
 }
 
 // As k_forces, with D read from BSR and the neighbours from H's pattern.
-__global__ void __launch_bounds__(32) k_forces_bsr(ModelDev m, int N, const int32_t* __restrict__ types,
-                                                   const int32_t* __restrict__ offs, const double* __restrict__ R,
-                                                   tb_bsr H, tb_bsr D, BsrModelWs w, const double* __restrict__ q,
-                                                   const double* __restrict__ n_aux, const double* __restrict__ v,
-                                                   double* __restrict__ F, double* __restrict__ energy) {
-  const int a = blockIdx.x;
+__global__ void __launch_bounds__(128) k_forces_bsr(ModelDev m, int N, const int32_t* __restrict__ types,
+                                                    const int32_t* __restrict__ offs, const double* __restrict__ R,
+                                                    tb_bsr H, tb_bsr D, BsrModelWs w, const double* __restrict__ q,
+                                                    const double* __restrict__ n_aux, const double* __restrict__ v,
+                                                    double* __restrict__ F, double* __restrict__ energy) {
+  __shared__ int s_list[4][kNbList];
+  const int a = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (a >= N || *H.status != TB_OK || *D.status != TB_OK) return;
   const double* Ra = R + 3 * a;
@@ -1300,52 +1392,52 @@ __global__ void __launch_bounds__(32) k_forces_bsr(ModelDev m, int N, const int3
   const double na = n_aux[a];
   double f[3] = {0.0, 0.0, 0.0};
   double e_band = 0.0, e_pair = 0.0;
-  for_neighbour_atoms(H, w, m, oa / kBB, Ra, lane, [&](int b) {
+  for_atoms_in_range(H, w, m, oa / kBB, a, R, (float)m.range, lane, s_list[threadIdx.x >> 5], [&](int b) {
     const double* Rb = R + 3 * b;
-    if (b != a && !screen_f32(Ra, Rb, (float)m.box, (float)m.range)) return;
     const int tb = types[b], ob = offs[b];
     const double wb = 2.0 * q[b] - n_aux[b];
     const double nb = n_aux[b];
     double Dl[4][4];
     const int nra = norb_of(ta), nrb = norb_of(tb);
-    for (int x = 0; x < 4; ++x)
-      for (int y = 0; y < 4; ++y) Dl[x][y] = (x < nra && y < nrb) ? bsr_get(D, oa + x, ob + y) : 0.0;
-    double d0[3];
-    min_image(Ra, Rb, m.box, d0);
-    int lo3[3], hi3[3];
+    if (oa / kBB == (oa + nra - 1) / kBB && ob / kBB == (ob + nrb - 1) / kBB) {
+      // both atoms within one block row: one block lookup for the pair
+      const int slot = bsr_slot(D.row_ptr, D.col, oa / kBB, ob / kBB);
+      const double* blk = D.val + (size_t)max(slot, 0) * kBB * kBB + (size_t)(oa % kBB) * kBB + ob % kBB;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) image_range(d0[c], m.box, m.range, &lo3[c], &hi3[c]);
-    for (int kx = lo3[0]; kx <= hi3[0]; ++kx)
-      for (int ky = lo3[1]; ky <= hi3[1]; ++ky)
-        for (int kz = lo3[2]; kz <= hi3[2]; ++kz) {
-          if (b == a && kx == 0 && ky == 0 && kz == 0) continue;
-          const double d[3] = {d0[0] + kx * m.box, d0[1] + ky * m.box, d0[2] + kz * m.box};
-          const double r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-          if (r >= m.range) continue;
-          const double l[3] = {d[0] / r, d[1] / r, d[2] / r};
-          if (r < m.rcut) {
-            double V, dV, Eblk, g[3];
-            hop_radial(m, r, &V, &dV);
-            band_pair_g(ta, tb, [&](int x, int y) { return Dl[x][y]; }, l, r, V, dV, &Eblk, g);
-            e_band += 2.0 * Eblk;
-            if (b != a)
+      for (int x = 0; x < 4; ++x)
 #pragma unroll
-              for (int k = 0; k < 3; ++k) f[k] += 4.0 * g[k];
-            double ph, dph;
-            pair_radial(m, r, &ph, &dph);
-            e_pair += 0.5 * ph;
-            if (b != a)
+        for (int y = 0; y < 4; ++y) Dl[x][y] = (slot >= 0 && x < nra && y < nrb) ? blk[x * kBB + y] : 0.0;
+    } else {
 #pragma unroll
-              for (int k = 0; k < 3; ++k) f[k] += dph * l[k];
-          }
-          if (b != a) {
-            double gg, dgg;
-            gamma_radial(m, r, &gg, &dgg);
-            const double c = 0.5 * (wa * nb + wb * na) * dgg;
+      for (int x = 0; x < 4; ++x)
 #pragma unroll
-            for (int k = 0; k < 3; ++k) f[k] += c * l[k];
-          }
-        }
+        for (int y = 0; y < 4; ++y) Dl[x][y] = (x < nra && y < nrb) ? bsr_get(D, oa + x, ob + y) : 0.0;
+    }
+    for_images(m, m.range, Ra, Rb, b == a, [&](const double (&d)[3], double r) {
+      const double ir = 1.0 / r, l[3] = {d[0] * ir, d[1] * ir, d[2] * ir};
+      if (r < m.rcut) {
+        double V, dV, Eblk, g[3];
+        hop_radial(m, r, &V, &dV);
+        band_pair_g(ta, tb, [&](int x, int y) { return Dl[x][y]; }, l, r, V, dV, &Eblk, g);
+        e_band += 2.0 * Eblk;
+        if (b != a)
+#pragma unroll
+          for (int k = 0; k < 3; ++k) f[k] += 4.0 * g[k];
+        double ph, dph;
+        pair_radial(m, r, &ph, &dph);
+        e_pair += 0.5 * ph;
+        if (b != a)
+#pragma unroll
+          for (int k = 0; k < 3; ++k) f[k] += dph * l[k];
+      }
+      if (b != a) {
+        double gg, dgg;
+        gamma_radial(m, r, &gg, &dgg);
+        const double c = 0.5 * (wa * nb + wb * na) * dgg;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) f[k] += c * l[k];
+      }
+    });
   });
 #pragma unroll
   for (int k = 0; k < 3; ++k) f[k] = warp_sum(f[k]);
@@ -1460,7 +1552,7 @@ extern "C" int tb_forces_bsr(tb_ctx* ctx, const tb_params* p, const tb_system* s
     return tb_fail(ctx, TB_ERR_ARG, "tb_forces_bsr: workspace too small");
   cudaStream_t s = as_stream(stream);
   TB_CUDA_TRY(ctx, cudaMemsetAsync(energy, 0, 4 * sizeof(double), s));
-  k_forces_bsr<<<N, 32, 0, s>>>(m, N, sys->types, sys->orb_off, R, *H, *D, w, q, n_aux, v, F, energy);
+  k_forces_bsr<<<(N + 3) / 4, 128, 0, s>>>(m, N, sys->types, sys->orb_off, R, *H, *D, w, q, n_aux, v, F, energy);
   TB_LAUNCH_CHECK(ctx);
   return TB_OK;
 }
