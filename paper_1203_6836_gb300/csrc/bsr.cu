@@ -17,7 +17,7 @@
 //           (every CTA the same), build each row's bitmaps of stored and live
 //           (not all-zero) super-blocks;
 //   symbolic  candidates of row I = OR of the live bitmaps of its live
-//           columns; scans give the output slots; each upper output block
+//           columns; every block scans the rows' counts for the output slots; each upper output block
 //           (I <= J; X^2 and its pattern are symmetric) gets the list of common
 //           K (live in both rows I and J) as pairs of source slots; the upper
 //           blocks are listed in (band of 8 block rows, column, row) order;
@@ -86,16 +86,27 @@ struct Buf {
   void* lo;
 };
 
+// An upper output block of the numeric kernel: all that its warps need to know of it in two
+// loads, which they make a block ahead (a chain of six dependent loads before).
+struct __align__(16) Unit {
+  int o, p0, np, om;  // slot, first pair and pairs, slot of the mirror
+  int I, J, oi, pad;  // block row and column, slot in S (or -1)
+};
+__device__ __forceinline__ Unit load_unit(const Unit* u) {
+  const int4 a = reinterpret_cast<const int4*>(u)[0], b = reinterpret_cast<const int4*>(u)[1];
+  return Unit{a.x, a.y, a.z, a.w, b.x, b.y, b.z, 0};
+}
+
 struct Sym {
   uint32_t* cand;    // [nsb * MW]
   int* cnt;          // [nsb]
-  int* out_row;      // [cap]
+  int* rowp;         // [nsb] pairs of a row's upper blocks
+  int* ucnt;         // [nsb] upper blocks of a row
   int* old_idx;      // [cap]
-  int* pcnt;         // [cap]
-  int* pair_ptr;     // [cap + 1]
+  int2* pcnt;        // [cap] pairs of the earlier blocks of the block's row, of the block
   int2* pairs;       // [pcap]
   int* scal;         // [4]: blocks of the new pattern, pairs, upper blocks
-  int* order;        // [cap] upper output blocks in the numeric kernel's order
+  Unit* order;       // [cap] upper output blocks in the numeric kernel's order
   uint16_t* flags;   // [nsb * nsb] X0 sub-block keep masks
 };
 
@@ -173,80 +184,104 @@ __device__ __forceinline__ void x0_affine(const Args& a, double* e, double* s) {
   *s = 1.0 / w;
 }
 
-__device__ __forceinline__ double x0_val(const double* H, int n, int r, int c, double emax, double inv) {
-  if (r >= n || c >= n) return 0.0;
-  return ((r == c ? emax : 0.0) - H[(size_t)r * n + c]) * inv;
-}
-
 // Whether any lane's value is not zero (an integer test and a vote: a few cycles,
 // where an FP64 instruction of a warp takes 19).
-__device__ __forceinline__ bool any_nonzero(double x) {
-  return __any_sync(0xffffffffu, (__double_as_longlong(x) << 1) != 0);
+// The halves come from a move that the compiler does not see through: it turns the
+// test of a double's bits into a comparison in FP64.
+__device__ __forceinline__ bool nonzero_bits(double x) {
+  uint32_t lo, hi;
+  asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "d"(x));
+  return ((hi << 1) | lo) != 0u;
 }
+__device__ __forceinline__ bool any_nonzero(double x) { return __any_sync(0xffffffffu, nonzero_bits(x)); }
 
-// Per-lane partial sums of squares of the 16 32 x 32 sub-blocks of a 128 x 128
-// block x(r, c) (256 threads: warp w takes rows w + 8k, lane l the columns
-// 32 c + l, so every row segment is one coalesced load; row w + 8k lies in
-// sub-block row k / 4).
-template <class X>
-__device__ __forceinline__ void block_partials(X x, double (&acc)[16]) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int s = 0; s < 16; ++s) acc[s] = 0.0;
-#pragma unroll
-  for (int kb = 0; kb < 4; ++kb) {  // the rows of one sub-block row: 16 loads in flight
-    double v[4][4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-#pragma unroll
-      for (int cc = 0; cc < 4; ++cc) v[k][cc] = x(warp + 32 * kb + 8 * k, 32 * cc + lane);
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-#pragma unroll
-      for (int cc = 0; cc < 4; ++cc)
-        if (any_nonzero(v[k][cc])) acc[kb * 4 + cc] = fma(v[k][cc], v[k][cc], acc[kb * 4 + cc]);
+// Values to be added in FP64, gathered first: zeros add nothing, and where no lane holds a
+// value in both p and v the two are one value a lane.  flush(p) when some lane has two.  In
+// a molecular H a row of 32 elements holds one or two that are not zero, so that about five
+// rows share an FP64 instruction (at 76 cycles a warp and scheduler it costs more than the
+// test, the vote and the merge together).  The caller flushes the last p.
+template <class Fn>
+__device__ __forceinline__ void gather_add(double v, double& p, Fn flush) {
+  const bool nv = nonzero_bits(v);
+  if (__any_sync(0xffffffffu, nv && nonzero_bits(p))) {
+    flush(p);
+    p = v;
+  } else if (nv) {
+    p = v;
   }
 }
 
-// Keep mask of super-block (I, J) of X0 = s (e I - H) from the partial sums
-// (block_partials) of e I - H over its upper twin (min(I,J), max(I,J)): a
-// warp sum per sub-block, the eight warps combined in a fixed order, times
-// scale2 = s^2, kept where ||.||_F >= tau (one FMA per element: GB300's FP64
-// rate is low); below the
-// diagonal the twin's mask transposed, so that the pattern is exactly
-// symmetric (the products compute upper blocks and mirror them).  Called by
-// every thread of the block; the mask is valid in thread 0.
-__device__ uint16_t keep_mask(const Args& a, int I, int J, const double (&acc)[16], double scale2) {
-  __shared__ double wsum[8][16];
+// Keep mask of a super-block of X0 = s (e I - H) from the elements x(r, c) of e I - H: a
+// 32 x 32 sub-block is kept where s^2 sum x^2 >= tau^2 (scale2 = s^2; one FMA per element:
+// GB300's FP64 rate is low).  Each of the 8 warps takes two sub-blocks: its lanes the
+// columns, so that a row is one coalesced load, 16 in flight, and a sub-block's sum stays
+// in one warp, few FP64 instructions to a sub-block (gather_add).  Called by
+// every thread of the block, which all get the mask.  (Sums of each of the 16 sub-blocks in
+// every warp, combined through shared memory, took 80 FP64 additions a warp and a serial
+// sum of 128: 849 us at 16383 orbitals.)
+template <class X>
+__device__ __forceinline__ uint16_t block_keep(const Args& a, double scale2, X x) {
+  __shared__ unsigned s_mask;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) s_mask = 0u;
+  __syncthreads();
+#pragma unroll 1
+  for (int q = warp; q < 16; q += 8) {
+    const int r0 = 32 * (q >> 2), c = 32 * (q & 3) + lane;
+    double acc = 0.0, p = 0.0;
+    auto flush = [&](double y) { acc = fma(y, y, acc); };
 #pragma unroll
-  for (int s = 0; s < 16; ++s) {
-    const double v = warp_sum(acc[s]);
-    if (lane == 0) wsum[warp][s] = v;
+    for (int h = 0; h < 2; ++h) {
+      double v[16];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) v[k] = x(r0 + 16 * h + k, c);
+#pragma unroll
+      for (int k = 0; k < 16; ++k) gather_add(v[k], p, flush);
+    }
+    if (any_nonzero(p)) {
+      flush(p);
+      acc = warp_sum(acc) * scale2;
+      if (lane == 0 && acc >= a.tau2 && acc > 0.0) atomicOr(&s_mask, 1u << q);
+    }
   }
   __syncthreads();
-  uint16_t f = 0;
-  if (threadIdx.x == 0)
-    for (int s = 0; s < 16; ++s) {
-      double t = 0.0;
-      for (int w = 0; w < 8; ++w) t += wsum[w][s];
-      t *= scale2;
-      if (t >= a.tau2 && t > 0.0) f |= (uint16_t)(1u << (I <= J ? s : (s & 3) * 4 + (s >> 2)));
-    }
-  __syncthreads();  // wsum is reused by the next block of a grid-stride loop
+  const uint16_t f = (uint16_t)s_mask;
+  __syncthreads();  // s_mask is reused by the next block of a grid-stride loop
   return f;
 }
 
-// One block per super-block (I, J) of X0 = s (e I - H): its keep mask.
+// The same from H's super-block (I, J) at h (row stride ld; null: zero).
+__device__ uint16_t x0_keep(const Args& a, const double* h, size_t ld, int I, int J, double e, double scale2) {
+  const int ne = max(0, a.n - I * SB), nc = max(0, a.n - J * SB);  // rows and columns inside the matrix
+  if (h && I != J && ne >= SB && nc >= SB)
+    return block_keep(a, scale2, [&](int r, int c) { return h[r * ld + c]; });
+  return block_keep(a, scale2, [&](int r, int c) {
+    if (r >= ne || c >= nc) return 0.0;
+    const double x = h ? h[r * ld + c] : 0.0;
+    return I == J && r == c ? e - x : x;
+  });
+}
+
+__device__ __forceinline__ uint16_t mask_transposed(uint16_t f) {
+  uint16_t t = 0;
+  for (int q = 0; q < 16; ++q)
+    if ((f >> q) & 1) t |= (uint16_t)(1u << ((q & 3) * 4 + (q >> 2)));
+  return t;
+}
+
+// One block per upper super-block (I, J) of X0 = s (e I - H): its keep mask, and below the
+// diagonal the twin's mask transposed, so that the pattern is exactly symmetric (the
+// products compute upper blocks and mirror them).
 __global__ void __launch_bounds__(256) k_bsr_init_flags(const double* __restrict__ H, Args a, Sym sy) {
   const int I = blockIdx.y, J = blockIdx.x;
-  const int I0 = min(I, J), J0 = max(I, J);
+  if (I > J) return;
   double emax, inv;
   x0_affine(a, &emax, &inv);
-  double acc[16];
-  block_partials([&](int r, int c) { return x0_val(H, a.n, I0 * SB + r, J0 * SB + c, emax, 1.0); }, acc);
-  const uint16_t f = keep_mask(a, I, J, acc, inv * inv);
-  if (threadIdx.x == 0) sy.flags[(size_t)I * a.nsb + J] = f;
+  const uint16_t f = x0_keep(a, H + (size_t)I * SB * a.n + J * SB, a.n, I, J, emax, inv * inv);
+  if (threadIdx.x == 0) {
+    sy.flags[(size_t)I * a.nsb + J] = f;
+    if (I != J) sy.flags[(size_t)J * a.nsb + I] = mask_transposed(f);
+  }
 }
 
 // Row I of X0: live bitmap of its kept super-blocks; stored = live (and the
@@ -300,64 +335,118 @@ __global__ void k_bsr_scan_rows(Args a, Sym sy, int* row_ptr) {
   }
 }
 
-// Fill the X0 blocks of row I (one block per row): values with dropped
-// sub-blocks zeroed, operand splits, trace partials of the row.
-template <int P>
-__global__ void __launch_bounds__(256) k_bsr_init_fill(const double* __restrict__ H, Args a, Sym sy, Buf b) {
-  if (a.st->err) return;
-  const int I = blockIdx.x;
+// Fill the X0 blocks of row I, kFillSplit thread blocks sharing its stored blocks: values
+// with dropped sub-blocks zeroed, operand splits, trace partials of each thread block.
+// src(J, &ld): H's super-block (I, J) (null: zero).  A warp takes a sub-block at a time, its
+// lanes the columns: whole-row loads and stores; dropped sub-blocks and rows that are all
+// zero take no FP64 work.  (One thread block a row, 32 elements of a row to a thread: 325 us
+// at 16383 orbitals.)
+constexpr int kFillSplit = 4;
+template <int P, class Src>
+__device__ void x0_fill_row(const Args& a, const Sym& sy, const Buf& b, Src src) {
+  __shared__ uint16_t s_col[kMaxNsb];
+  __shared__ float s_t[8][32][33];  // stored splits: a sub-block to be read by rows
+  __shared__ double s1[8], s2[8];
+  const int I = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   double emax, inv;
   x0_affine(a, &emax, &inv);
+  const uint32_t* st = b.stored + I * MW;
+  for (int J = threadIdx.x; J < a.nsb; J += blockDim.x)
+    if ((st[J >> 5] >> (J & 31)) & 1u) s_col[popc_below(st, J)] = (uint16_t)J;
+  __syncthreads();
   double t1 = 0.0, t2 = 0.0;
-  int o = b.row_ptr[I];
-  for (int J = 0; J < a.nsb; ++J) {
+  const int o0 = b.row_ptr[I], cnt = b.row_ptr[I + 1] - o0;
+  const int ne = max(0, a.n - I * SB);
+  for (int k = blockIdx.y; k < cnt; k += kFillSplit) {
+    const int J = s_col[k], o = o0 + k;
     const uint16_t f = sy.flags[(size_t)I * a.nsb + J];
-    if (!f && !(a.keep_diag && J == I)) continue;
+    const int nc = max(0, a.n - J * SB);
+    size_t ld = 0;
+    const double* h = src(J, &ld);
     if (threadIdx.x == 0) {
       b.col[o] = J;
       b.nz[o] = f != 0;
     }
-    // 128 rows x 4 segments of 32: 512 segments over 256 threads
-    for (int seg = threadIdx.x; seg < SB * 4; seg += blockDim.x) {
-      const int r = seg >> 2, cs = seg & 3;
-      const bool keep = (f >> ((r >> 5) * 4 + cs)) & 1;
-      float y[32];
-      for (int j = 0; j < 32; ++j) {
-        const double x = keep ? x0_val(H, a.n, I * SB + r, J * SB + 32 * cs + j, emax, inv) : 0.0;
-        y[j] = (float)x;
-        const double xf = (double)y[j];
-        t2 += xf * xf;
-        if (I == J && r == 32 * cs + j) t1 += xf;
+#pragma unroll 1
+    for (int q = warp; q < 16; q += 8) {
+      const int r0 = 32 * (q >> 2), c0 = 32 * (q & 3), c = c0 + lane;
+      float* dst = b.val + (size_t)o * kTiles + (size_t)r0 * SB + c0;
+      if ((f >> q) & 1) {
+        const bool dsub = I == J && r0 == c0;
+        float yd = 0.0f;
+#pragma unroll
+        for (int rb = 0; rb < 32; rb += 16) {
+          double x[16];
+#pragma unroll
+          for (int r = 0; r < 16; ++r)
+            x[r] = h && r0 + rb + r < ne && c < nc ? h[(r0 + rb + r) * ld + c] : 0.0;
+#pragma unroll
+          for (int r = 0; r < 16; ++r) {
+            float y = 0.0f;
+            if (dsub) {
+              const bool on = rb + r == lane && r0 + lane < ne;
+              y = (float)(((on ? emax : 0.0) - x[r]) * inv);
+              if (on) yd = y;
+            } else if (any_nonzero(x[r])) {
+              y = (float)(-x[r] * inv) + 0.0f;  // + 0: the zeros of X0 are positive
+            }
+            if (__any_sync(0xffffffffu, y != 0.0f)) {
+              const double d = abs_to_f64(y);
+              t2 = fma(d, d, t2);
+            }
+            dst[(size_t)(rb + r) * SB + lane] = y;
+            if constexpr (!kStaged<P>) s_t[warp][rb + r][lane] = y;
+          }
+        }
+        if (dsub) t1 += (double)yd;
+      } else {
+#pragma unroll
+        for (int r = 0; r < 32; r += 4)
+          *reinterpret_cast<float4*>(dst + (size_t)(r + (lane >> 3)) * SB + 4 * (lane & 7)) =
+              make_float4(0.f, 0.f, 0.f, 0.f);
+        if constexpr (!kStaged<P>)
+          for (int r = 0; r < 32; ++r) s_t[warp][r][lane] = 0.0f;
       }
-      const size_t e0 = (size_t)o * kTiles + (size_t)r * SB + 32 * cs;
-      float* dst = b.val + e0;
-      for (int j = 0; j < 32; ++j) dst[j] = y[j];
       if constexpr (!kStaged<P>) {
-        char* h = static_cast<char*>(b.hi) + e0 * Prec<P>::eb;
-        char* l = b.lo ? static_cast<char*>(b.lo) + e0 * Prec<P>::eb : h;
-        store_operands<P>(y, h, l);
+        __syncwarp();
+        float y[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) y[j] = s_t[warp][lane][j];
+        __syncwarp();
+        const size_t e0 = (size_t)o * kTiles + (size_t)(r0 + lane) * SB + c0;
+        char* hp = static_cast<char*>(b.hi) + e0 * Prec<P>::eb;
+        char* lp = b.lo ? static_cast<char*>(b.lo) + e0 * Prec<P>::eb : hp;
+        store_operands<P>(y, hp, lp);
       }
     }
-    ++o;
   }
-  __shared__ double s1[8], s2[8];
   t1 = warp_sum(t1);
   t2 = warp_sum(t2);
-  if ((threadIdx.x & 31) == 0) {
-    s1[threadIdx.x >> 5] = t1;
-    s2[threadIdx.x >> 5] = t2;
+  if (lane == 0) {
+    s1[warp] = t1;
+    s2[warp] = t2;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
     double x = 0, y = 0;
-    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) {
+    for (int q = 0; q < 8; ++q) {
       x += s1[q];
       y += s2[q];
     }
-    a.parts_out[3 * I] = x;
-    a.parts_out[3 * I + 1] = y;
-    a.parts_out[3 * I + 2] = 0.0;
+    double* p = a.parts_out + 3 * (I * kFillSplit + blockIdx.y);
+    p[0] = x;
+    p[1] = y;
+    p[2] = 0.0;
   }
+}
+
+template <int P>
+__global__ void __launch_bounds__(256) k_bsr_init_fill(const double* __restrict__ H, Args a, Sym sy, Buf b) {
+  if (a.st->err) return;
+  x0_fill_row<P>(a, sy, b, [&](int J, size_t* ld) {
+    *ld = a.n;
+    return H + (size_t)blockIdx.x * SB * a.n + J * SB;
+  });
 }
 
 // ---- BSR input (dm_sp2_sparse): H given as 128 x 128 FP64 blocks
@@ -375,14 +464,14 @@ __device__ __forceinline__ int bsr_find(const int* __restrict__ row_ptr, const i
   return -1;
 }
 
-// Gershgorin partials of block row I (kBndSplit blocks of 256 threads, 32 rows
+// Gershgorin partials of block row I (kBndSplit blocks of 256 threads, 16 rows
 // each): warp w takes rows w + 8k, lane l the columns 32 c + l, so each block is read
-// as 16 independent coalesced loads a lane, and the row sums stay in registers until
+// as 8 independent coalesced loads a lane, two blocks at a time, and the row sums stay in registers until
 // one warp sum per row; min(H_ii - r_i) and max(H_ii + r_i) over the rows go into
 // bparts[2 (I kBndSplit + y)].  The FP64 pipe would bound this kernel (1.1 ms for the
 // 1.2 GB of a 16 383-atom H): pieces of rows that are all zero, most of a block of a
 // molecular H, are skipped.
-constexpr int kBndSplit = 4;
+constexpr int kBndSplit = 8;
 __global__ void __launch_bounds__(256) k_bsr_bounds_in(tb_bsr H, double* __restrict__ bparts) {
   __shared__ double smin[8], smax[8];
   constexpr int kRows = 16 / kBndSplit;  // rows per warp
@@ -393,26 +482,37 @@ __global__ void __launch_bounds__(256) k_bsr_bounds_in(tb_bsr H, double* __restr
     if (threadIdx.x == 0) bparts[0] = bparts[1] = 0.0;
     return;
   }
-  double rad[kRows], dia[kRows];
+  double rad[kRows], dia[kRows], pend[kRows];
 #pragma unroll
-  for (int k = 0; k < kRows; ++k) rad[k] = dia[k] = 0.0;
-  for (int o = H.row_ptr[I]; o < H.row_ptr[I + 1]; ++o) {
-    const double* blk = H.val + (size_t)o * kTiles;
-    const bool dblk = H.col[o] == I;
-    double x[kRows][4];
+  for (int k = 0; k < kRows; ++k) rad[k] = dia[k] = pend[k] = 0.0;
+  const int o1 = H.row_ptr[I + 1];
+  for (int o = H.row_ptr[I]; o < o1; o += 2) {
+    const bool two = o + 1 < o1;
+    const bool dblk[2] = {H.col[o] == I, two && H.col[o + 1] == I};
+    double x[2][kRows][4];
 #pragma unroll
-    for (int k = 0; k < kRows; ++k)
+    for (int t = 0; t < 2; ++t)
 #pragma unroll
-      for (int cc = 0; cc < 4; ++cc) x[k][cc] = blk[(size_t)(r0 + 8 * k) * SB + 32 * cc + lane];
+      for (int k = 0; k < kRows; ++k)
 #pragma unroll
-    for (int k = 0; k < kRows; ++k)
+        for (int cc = 0; cc < 4; ++cc)
+          x[t][k][cc] = t == 0 || two ? H.val[(size_t)(o + t) * kTiles + (r0 + 8 * k) * SB + 32 * cc + lane] : 0.0;
 #pragma unroll
-      for (int cc = 0; cc < 4; ++cc) {
-        if (!any_nonzero(x[k][cc])) continue;
-        if (dblk && 32 * cc + lane == r0 + 8 * k) dia[k] += x[k][cc];
-        else rad[k] += fabs(x[k][cc]);
-      }
+    for (int t = 0; t < 2; ++t)
+#pragma unroll
+      for (int k = 0; k < kRows; ++k)
+#pragma unroll
+        for (int cc = 0; cc < 4; ++cc) {
+          double v = x[t][k][cc];
+          if (dblk[t] && 32 * cc + lane == r0 + 8 * k) {
+            dia[k] = v;
+            v = 0.0;
+          }
+          gather_add(v, pend[k], [&](double y) { rad[k] += fabs(y); });
+        }
   }
+#pragma unroll
+  for (int k = 0; k < kRows; ++k) rad[k] += fabs(pend[k]);
   double lo = INFINITY, hi = -INFINITY;
 #pragma unroll
   for (int k = 0; k < kRows; ++k) {
@@ -436,22 +536,6 @@ __global__ void __launch_bounds__(256) k_bsr_bounds_in(tb_bsr H, double* __restr
     bparts[0] = a;
     bparts[1] = b;
   }
-}
-
-// e delta - h at element (r, c) of block (I, J) (zero outside the n x n matrix).
-__device__ __forceinline__ double x0_unscaled(const double* blk, int I, int J, int n, int r, int c, double e) {
-  const int gr = I * SB + r, gc = J * SB + c;
-  if (gr >= n || gc >= n) return 0.0;
-  const double h = blk ? blk[(size_t)r * SB + c] : 0.0;
-  return gr == gc ? e - h : -h;
-}
-
-__device__ __forceinline__ double x0_blk(const double* blk, int I, int J, int n, int r, int c, double emax,
-                                         double inv) {
-  const int gr = I * SB + r, gc = J * SB + c;
-  if (gr >= n || gc >= n) return 0.0;
-  const double h = blk ? blk[(size_t)r * SB + c] : 0.0;
-  return ((gr == gc ? emax : 0.0) - h) * inv;
 }
 
 // As k_bsr_init_flags, from the blocks of a BSR H (an absent block of H is
@@ -483,18 +567,11 @@ __global__ void __launch_bounds__(256) k_bsr_init_flags_in(tb_bsr H, Args a, Sym
   for (int o = blockIdx.x; o < nblk; o += gridDim.x) {
     const int I = bsr_row_of(H.row_ptr, H.nsb, o), J = H.col[o];
     if (I > J) continue;  // its mask is its twin's transposed (or 0: H stores none)
-    const double* blk = H.val + (size_t)o * kTiles;
-    double acc[16];
-    block_partials([&](int r, int c) { return x0_unscaled(blk, I, J, a.n, r, c, emax); }, acc);
-    const uint16_t f = keep_mask(a, I, J, acc, inv * inv);
+    const uint16_t f = x0_keep(a, H.val + (size_t)o * kTiles, SB, I, J, emax, inv * inv);
     if (threadIdx.x == 0) {
       sy.flags[(size_t)I * a.nsb + J] = f;
-      if (I != J && bsr_find(H.row_ptr, H.col, J, I) >= 0) {
-        uint16_t t = 0;
-        for (int q = 0; q < 16; ++q)
-          if ((f >> q) & 1) t |= (uint16_t)(1u << ((q & 3) * 4 + (q >> 2)));
-        sy.flags[(size_t)J * a.nsb + I] = t;
-      }
+      if (I != J && f && bsr_find(H.row_ptr, H.col, J, I) >= 0)
+        sy.flags[(size_t)J * a.nsb + I] = mask_transposed(f);
     }
   }
 }
@@ -504,9 +581,7 @@ __global__ void __launch_bounds__(256) k_bsr_init_flags_diag(tb_bsr H, Args a, S
   if (*H.status != TB_OK || bsr_find(H.row_ptr, H.col, I, I) >= 0) return;
   double emax, inv;
   x0_affine(a, &emax, &inv);
-  double acc[16];
-  block_partials([&](int r, int c) { return x0_unscaled(nullptr, I, I, a.n, r, c, emax); }, acc);
-  const uint16_t f = keep_mask(a, I, I, acc, inv * inv);
+  const uint16_t f = x0_keep(a, nullptr, 0, I, I, emax, inv * inv);
   if (threadIdx.x == 0) sy.flags[(size_t)I * a.nsb + I] = f;
 }
 
@@ -514,60 +589,11 @@ __global__ void __launch_bounds__(256) k_bsr_init_flags_diag(tb_bsr H, Args a, S
 template <int P>
 __global__ void __launch_bounds__(256) k_bsr_init_fill_in(tb_bsr H, Args a, Sym sy, Buf b) {
   if (a.st->err) return;
-  const int I = blockIdx.x;
-  double emax, inv;
-  x0_affine(a, &emax, &inv);
-  double t1 = 0.0, t2 = 0.0;
-  int o = b.row_ptr[I];
-  for (int J = 0; J < a.nsb; ++J) {
-    const uint16_t f = sy.flags[(size_t)I * a.nsb + J];
-    if (!f && !(a.keep_diag && J == I)) continue;
-    const int slot = bsr_find(H.row_ptr, H.col, I, J);
-    const double* blk = slot >= 0 ? H.val + (size_t)slot * kTiles : nullptr;
-    if (threadIdx.x == 0) {
-      b.col[o] = J;
-      b.nz[o] = f != 0;
-    }
-    for (int seg = threadIdx.x; seg < SB * 4; seg += blockDim.x) {
-      const int r = seg >> 2, cs = seg & 3;
-      const bool keep = (f >> ((r >> 5) * 4 + cs)) & 1;
-      float y[32];
-      for (int j = 0; j < 32; ++j) {
-        const double x = keep ? x0_blk(blk, I, J, a.n, r, 32 * cs + j, emax, inv) : 0.0;
-        y[j] = (float)x;
-        const double xf = (double)y[j];
-        t2 += xf * xf;
-        if (I == J && r == 32 * cs + j) t1 += xf;
-      }
-      const size_t e0 = (size_t)o * kTiles + (size_t)r * SB + 32 * cs;
-      float* dst = b.val + e0;
-      for (int j = 0; j < 32; ++j) dst[j] = y[j];
-      if constexpr (!kStaged<P>) {
-        char* hp = static_cast<char*>(b.hi) + e0 * Prec<P>::eb;
-        char* lp = b.lo ? static_cast<char*>(b.lo) + e0 * Prec<P>::eb : hp;
-        store_operands<P>(y, hp, lp);
-      }
-    }
-    ++o;
-  }
-  __shared__ double s1[8], s2[8];
-  t1 = warp_sum(t1);
-  t2 = warp_sum(t2);
-  if ((threadIdx.x & 31) == 0) {
-    s1[threadIdx.x >> 5] = t1;
-    s2[threadIdx.x >> 5] = t2;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double x = 0, y = 0;
-    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) {
-      x += s1[q];
-      y += s2[q];
-    }
-    a.parts_out[3 * I] = x;
-    a.parts_out[3 * I + 1] = y;
-    a.parts_out[3 * I + 2] = 0.0;
-  }
+  x0_fill_row<P>(a, sy, b, [&](int J, size_t* ld) {
+    *ld = SB;
+    const int slot = bsr_find(H.row_ptr, H.col, blockIdx.x, J);
+    return slot >= 0 ? H.val + (size_t)slot * kTiles : nullptr;
+  });
 }
 
 // ------------------------------------------------------- per projection
@@ -684,139 +710,221 @@ __global__ void k_bsr_cand(Args a, Buf A, Buf B, Buf S, Sym sy) {
   }
 }
 
-// Output blocks of row I: column, slot of S_IJ (or -1), pair count.
-__global__ void k_bsr_fill_out(Args a, Buf A, Buf B, Buf S, Buf bn, Sym sy) {
-  if (a.st->done || a.st->err) return;
-  const int I = blockIdx.x;
+// Sum of v over the rows before I, and over all nsb rows (256 threads; every thread gets
+// both): each block of a symbolic kernel scans the rows' counts for itself, instead of a
+// launch of one block before it.
+__device__ void rows_prefix(const int* __restrict__ v, int nsb, int I, long long* before, long long* total) {
+  __shared__ long long s_b[8], s_t[8];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  long long b = 0, t = 0;
+  for (int i = threadIdx.x; i < nsb; i += 256) {
+    const int x = v[i];
+    t += x;
+    if (i < I) b += x;
+  }
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) {
+    b += __shfl_xor_sync(0xffffffffu, b, d);
+    t += __shfl_xor_sync(0xffffffffu, t, d);
+  }
+  if (lane == 0) {
+    s_b[warp] = b;
+    s_t[warp] = t;
+  }
+  __syncthreads();
+  b = t = 0;
+  for (int w = 0; w < 8; ++w) {
+    b += s_b[w];
+    t += s_t[w];
+  }
+  *before = b;
+  *total = t;
+}
+
+// Whether the call is finished or failed, the same for every thread of the block also where
+// another block of this launch sets the error.
+__device__ __forceinline__ bool stopped(const SP2State* st) {
+  return __syncthreads_or(threadIdx.x == 0 && (st->done || st->err));
+}
+
+// Output blocks of row I: its start, and for each block the column, the slot of S_IJ (or
+// -1) and the pairs of the row's blocks before it; the row's pairs and upper blocks.
+__global__ void __launch_bounds__(256) k_bsr_fill_out(Args a, Buf A, Buf B, Buf S, Buf bn, Sym sy) {
+  __shared__ int s_w[8];
+  if (stopped(a.st)) return;
+  const int I = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  long long base, total;
+  rows_prefix(sy.cnt, a.nsb, I, &base, &total);
+  if (threadIdx.x == 0) {
+    bn.row_ptr[I] = (int)base;
+    if (I == 0) {
+      bn.row_ptr[a.nsb] = (int)total;
+      sy.scal[0] = (int)total;
+      if (total > a.cap) atomicExch(&a.st->err, TB_ERR_OOM);
+    }
+  }
+  if (total > a.cap) return;
   const uint32_t* ci = sy.cand + I * MW;
   const uint32_t* si = S.stored ? S.stored + I * MW : nullptr;
   const uint32_t* li = A.live + I * MW;
-  for (int J = threadIdx.x; J < a.nsb; J += blockDim.x) {
-    if (!((ci[J >> 5] >> (J & 31)) & 1u)) continue;
-    const int o = bn.row_ptr[I] + popc_below(ci, J);
-    bn.col[o] = J;
-    bn.nz[o] = 0;
-    sy.out_row[o] = I;
-    sy.old_idx[o] = (si && ((si[J >> 5] >> (J & 31)) & 1u)) ? S.row_ptr[I] + popc_below(si, J) : -1;
+  int run = 0, upper = 0;
+  long long prod = 0;  // a block above the diagonal has a mirror with as many products
+  for (int J0 = 0; J0 < a.nsb; J0 += 256) {
+    const int J = J0 + (int)threadIdx.x;
+    const bool has = J < a.nsb && ((ci[J >> 5] >> (J & 31)) & 1u);
     int pc = 0;
-    const uint32_t* lj = B.live + J * MW;
-    if (J >= I)  // the product is symmetric: blocks below the diagonal are written as mirrors
+    if (has && J >= I) {  // the product is symmetric: blocks below the diagonal are written as mirrors
+      const uint32_t* lj = B.live + J * MW;
       for (int w = 0; w < a.mw; ++w) pc += __popc(li[w] & lj[w]);
-    sy.pcnt[o] = pc;
-  }
-}
-
-// Exclusive scan of the pair counts of all output blocks (one block).
-__global__ void __launch_bounds__(1024) k_bsr_scan_pairs(Args a, Sym sy) {
-  __shared__ int part[1024];
-  if (a.st->done || a.st->err) return;
-  const int nb = sy.scal[0];
-  const int per = (nb + blockDim.x - 1) / blockDim.x;
-  const int lo = threadIdx.x * per, hi = min(nb, lo + per);
-  int s = 0;
-  for (int i = lo; i < hi; ++i) s += sy.pcnt[i];
-  part[threadIdx.x] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int acc = 0;
-    for (int t = 0; t < (int)blockDim.x; ++t) {
-      const int v = part[t];
-      part[t] = acc;
-      acc += v;
+      ++upper;
+      prod += J > I ? 2 * pc : pc;
     }
-    sy.scal[1] = acc;
-    sy.pair_ptr[nb] = acc;
-    a.st->block_products += (unsigned long long)acc;
-    if (acc > a.pcap) atomicExch(&a.st->err, TB_ERR_OOM);
-  }
-  __syncthreads();
-  int run = part[threadIdx.x];
-  for (int i = lo; i < hi; ++i) {
-    sy.pair_ptr[i] = run;
-    run += sy.pcnt[i];
-  }
-}
-
-// Pairs (slot of A_IK, slot of B_JK) of every upper output block (I, J):
-// (A B)_IJ = sum_K A_IK B_JK^T for a symmetric B.
-__global__ void k_bsr_pairs(Args a, Buf A, Buf B, Buf bn, Sym sy) {
-  if (a.st->done || a.st->err) return;
-  const int nb = sy.scal[0];
-  for (int o = blockIdx.x * blockDim.x + threadIdx.x; o < nb; o += gridDim.x * blockDim.x) {
-    const int I = sy.out_row[o], J = bn.col[o];
-    if (J < I) continue;
-    const uint32_t* li = A.live + I * MW;
-    const uint32_t* lj = B.live + J * MW;
-    const uint32_t* si = A.stored + I * MW;
-    const uint32_t* sj = B.stored + J * MW;
-    int p = sy.pair_ptr[o];
-    // the mirrored block (J, I) of the full product has as many block products
-    if (J > I) atomicAdd(&a.st->block_products, (unsigned long long)sy.pcnt[o]);
-    for (int w = 0; w < a.mw; ++w) {
-      uint32_t m = li[w] & lj[w];
-      while (m) {
-        const int K = 32 * w + __ffs(m) - 1;
-        m &= m - 1u;
-        sy.pairs[p++] = make_int2(A.row_ptr[I] + popc_below(si, K), B.row_ptr[J] + popc_below(sj, K));
-      }
+    int incl = pc;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= d) incl += t;
+    }
+    if (lane == 31) s_w[warp] = incl;
+    __syncthreads();
+    int before = run;
+    for (int w = 0; w < 8; ++w) {
+      if (w < warp) before += s_w[w];
+      run += s_w[w];
+    }
+    __syncthreads();
+    if (has) {
+      const int o = (int)base + popc_below(ci, J);
+      bn.col[o] = J;
+      bn.nz[o] = 0;
+      sy.old_idx[o] = (si && ((si[J >> 5] >> (J & 31)) & 1u)) ? S.row_ptr[I] + popc_below(si, J) : -1;
+      sy.pcnt[o] = make_int2(before + incl - pc, pc);
     }
   }
-}
-
-// Upper output blocks (I <= J) in (band of kBand block rows, column J, row I)
-// order.  The persistent numeric kernel takes them in this order, so the CTAs
-// working at the same time cover a few columns of one band: they share the
-// (I, K) tiles of the band's rows and the (J, K) tiles of those columns in L2
-// instead of each streaming its own.  One block; one warp per band.
-__global__ void __launch_bounds__(1024) k_bsr_order(Args a, Buf bn, Sym sy) {
-  __shared__ int s_off[kMaxNsb / kBand + 1];
-  if (a.st->done || a.st->err) return;
-  const int nbands = (a.nsb + kBand - 1) / kBand;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int b = warp; b < nbands; b += nw) {
-    int c = 0;
-    for (int I = b * kBand; I < min(a.nsb, (b + 1) * kBand); ++I) {
-      if (lane < MW) {
-        uint32_t m = sy.cand[I * MW + lane];
-        const int lo = I - 32 * lane;  // keep bits J >= I
-        if (lo >= 32) m = 0u;
-        else if (lo > 0) m &= ~((1u << lo) - 1u);
-        c += __popc(m);
-      }
-    }
-    c = __reduce_add_sync(0xffffffffu, c);
-    if (lane == 0) s_off[b] = c;
+  upper = __reduce_add_sync(0xffffffffu, upper);
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) prod += __shfl_xor_sync(0xffffffffu, prod, d);
+  if (lane == 0) {
+    s_w[warp] = upper;
+    if (prod) atomicAdd(&a.st->block_products, (unsigned long long)prod);
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    int acc = 0;
-    for (int b = 0; b < nbands; ++b) {
-      const int v = s_off[b];
-      s_off[b] = acc;
-      acc += v;
-    }
-    sy.scal[2] = acc;
+    int u = 0;
+    for (int w = 0; w < 8; ++w) u += s_w[w];
+    sy.rowp[I] = run;
+    sy.ucnt[I] = u;
   }
-  __syncthreads();
-  for (int b = warp; b < nbands; b += nw) {
-    int pos = s_off[b];
-    const int I0 = b * kBand;
-    const int I = I0 + lane;
-    // only the columns J >= I0 that some row of the band holds (the OR of the
-    // band's candidate words), in increasing order
-    for (int w = I0 >> 5; w < a.mw; ++w) {
-      uint32_t any = 0u;
-      for (int r = 0; r < kBand && I0 + r < a.nsb; ++r) any |= sy.cand[(I0 + r) * MW + w];
-      if (w == (I0 >> 5)) any &= ~((1u << (I0 & 31)) - 1u);
-      while (any) {
-        const int J = 32 * w + __ffs(any) - 1;
-        any &= any - 1u;
-        const bool has = lane < kBand && I < a.nsb && I <= J && ((sy.cand[I * MW + w] >> (J & 31)) & 1u);
-        const unsigned m = __ballot_sync(0xffffffffu, has);
-        if (has) sy.order[pos + __popc(m & ((1u << lane) - 1u))] = bn.row_ptr[I] + popc_below(sy.cand + I * MW, J);
-        pos += __popc(m);
+}
+
+// The numeric kernel's lists, in one launch:
+// - blocks below nsb * kPairSplit: the pairs (slot of A_IK, slot of B_JK) of every upper
+//   output block (I, J), (A B)_IJ = sum_K A_IK B_JK^T for a symmetric B: a warp per output
+//   block, its lanes the columns K of a bitmap word, so that the pairs are written
+//   coalesced (a thread per output block: 11 us a projection at 128 block rows, and the
+//   scan of the pair counts before it another 11);
+// - the others: the upper output blocks (I <= J) in (band of kBand block rows, column J,
+//   row I) order.  The persistent numeric kernel takes them in this order, so the CTAs
+//   working at the same time cover a few columns of one band: they share the (I, K) tiles
+//   of the band's rows and the (J, K) tiles of those columns in L2 instead of each
+//   streaming its own.  A warp per band and bitmap word, its lanes the columns (a warp per
+//   band walking the columns: 22 us a projection).
+constexpr int kPairSplit = 4;
+__global__ void __launch_bounds__(256) k_bsr_pairs(Args a, Buf A, Buf B, Buf bn, Sym sy) {
+  if (stopped(a.st)) return;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1u;
+  const int npb = a.nsb * kPairSplit;
+  const bool listing = (int)blockIdx.x >= npb;
+  const int I = listing ? 0 : blockIdx.x / kPairSplit;
+  long long before, total;
+  rows_prefix(sy.rowp, a.nsb, I, &before, &total);
+  if (blockIdx.x == 0 && threadIdx.x == 0 && total > a.pcap) atomicExch(&a.st->err, TB_ERR_OOM);
+  if (total > a.pcap) return;
+  if (!listing) {
+    const int part = blockIdx.x % kPairSplit;
+    const uint32_t al = A.live[I * MW + lane], as = A.stored[I * MW + lane];
+    const int ra0 = A.row_ptr[I], o1 = bn.row_ptr[I + 1];
+    for (int o = bn.row_ptr[I] + part * 8 + warp; o < o1; o += kPairSplit * 8) {
+      const int J = bn.col[o];
+      if (J < I) continue;
+      int p = (int)before + sy.pcnt[o].x;
+      const uint32_t m_l = al & B.live[J * MW + lane], bs = B.stored[J * MW + lane];
+      int ra = ra0, rb = B.row_ptr[J];
+      for (int w = 0; w < a.mw; ++w) {
+        const uint32_t m = __shfl_sync(0xffffffffu, m_l, w), sa = __shfl_sync(0xffffffffu, as, w),
+                       sb = __shfl_sync(0xffffffffu, bs, w);
+        if ((m >> lane) & 1u)
+          sy.pairs[p + __popc(m & below)] = make_int2(ra + __popc(sa & below), rb + __popc(sb & below));
+        p += __popc(m);
+        ra += __popc(sa);
+        rb += __popc(sb);
       }
     }
+    return;
+  }
+  const int id = ((int)blockIdx.x - npb) * 8 + warp, band = id / a.mw, w = id % a.mw, I0 = band * kBand;
+  if (id == 0) {
+    int u = 0;
+    for (int i = lane; i < a.nsb; i += 32) u += sy.ucnt[i];
+    u = __reduce_add_sync(0xffffffffu, u);
+    if (lane == 0) sy.scal[2] = u;
+  }
+  if (I0 >= a.nsb) return;
+  int pos = 0, pairs0 = 0;  // entries and pairs before the band
+  for (int i = lane; i < I0; i += 32) {
+    pos += sy.ucnt[i];
+    pairs0 += sy.rowp[i];
+  }
+  pairs0 = __reduce_add_sync(0xffffffffu, pairs0);
+  uint32_t word[kBand];  // word w of the band's rows, columns J >= I only
+  int slot[kBand];       // slot of the first block of that word
+  const int J = 32 * w + lane;
+  int mine = 0;
+#pragma unroll
+  for (int r = 0; r < kBand; ++r) {
+    const int Ir = I0 + r;
+    const uint32_t c = Ir < a.nsb ? sy.cand[Ir * MW + lane] : 0u;  // lane: the word
+    const int lo = Ir - 32 * lane;                                 // keep bits J >= I
+    const uint32_t up = lo >= 32 ? 0u : lo > 0 ? c & ~((1u << lo) - 1u) : c;
+    if (lane < w) pos += __popc(up);
+    slot[r] = __reduce_add_sync(0xffffffffu, lane < w ? __popc(c) : 0);
+    if (Ir < a.nsb) slot[r] += bn.row_ptr[Ir];
+    const uint32_t cw = __shfl_sync(0xffffffffu, c, w);
+    slot[r] += __popc(cw & below);
+    word[r] = __shfl_sync(0xffffffffu, up, w);
+    mine += (word[r] >> lane) & 1u;
+  }
+  pos = __reduce_add_sync(0xffffffffu, pos);
+  int incl = mine;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, incl, d);
+    if (lane >= d) incl += t;
+  }
+  pos += incl - mine;
+  if (!mine) return;
+  // slot of the mirror (J, I): the band's rows lie in one word of row J
+  const uint32_t* cj = sy.cand + J * MW;
+  const int mir = bn.row_ptr[J] + popc_below(cj, I0);
+  const uint32_t wj = cj[I0 >> 5] >> (I0 & 31);
+  int2 pc[kBand];
+  int oi[kBand], rp[kBand];
+#pragma unroll
+  for (int r = 0; r < kBand; ++r) {  // loads of all rows in flight together
+    const int o = (word[r] >> lane) & 1u ? slot[r] : 0;
+    pc[r] = sy.pcnt[o];
+    oi[r] = sy.old_idx[o];
+    rp[r] = I0 + r < a.nsb ? sy.rowp[I0 + r] : 0;
+  }
+#pragma unroll
+  for (int r = 0; r < kBand; ++r) {
+    if ((word[r] >> lane) & 1u) {
+      int4* u = reinterpret_cast<int4*>(sy.order + pos++);
+      u[0] = make_int4(slot[r], pairs0 + pc[r].x, pc[r].y, J > I0 + r ? mir + __popc(wj & ((1u << r) - 1u)) : slot[r]);
+      u[1] = make_int4(I0 + r, J, oi[r], 0);
+    }
+    pairs0 += rp[r];
   }
 }
 
@@ -840,6 +948,9 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
   const int br = ep.branch ? (int)((st->branch[a.k >> 6] >> (a.k & 63)) & 1ull) : 0;
   const float alpha = br ? ep.a1 : ep.a0, gamma = br ? ep.g1 : ep.g0;
   const int nu = sy.scal[2];  // upper output blocks, walked in sy.order
+  // an FP32 sum of squares below this is below tau^2 (thresholds whose squares could
+  // underflow take the FP64 sum)
+  const float drop32 = a.tau2 > 1e-24 ? (float)(0.9999 * a.tau2) : -1.0f;
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   if (threadIdx.x == 0) {
@@ -871,11 +982,14 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
       prefetch_map(&bl);
     }
     int g = 0, issued = 0;
+    int4 next = blockIdx.x < nu ? *reinterpret_cast<const int4*>(sy.order + blockIdx.x) : make_int4(0, 0, 0, 0);
     for (int u = blockIdx.x; u < nu && !s_abort; u += gridDim.x) {
-      const int o = sy.order[u];
-      const int p0 = sy.pair_ptr[o], p1 = sy.pair_ptr[o + 1];
+      const int p0 = next.y, p1 = next.y + next.z;
+      if (u + (int)gridDim.x < nu) next = *reinterpret_cast<const int4*>(sy.order + u + gridDim.x);
+      int2 pr1 = p0 < p1 ? sy.pairs[p0] : make_int2(0, 0);
       for (int p = p0; p < p1 && !s_abort; ++p) {
-        const int2 pr = sy.pairs[p];
+        const int2 pr = pr1;
+        if (p + 1 < p1) pr1 = sy.pairs[p + 1];
         for (int c = 0; c < chunks; ++c, ++g) {
           const int s = g % NS;
           if (g >= NS && !mbar_wait(&empty[s], ((g / NS) - 1) & 1, &s_abort)) break;
@@ -904,15 +1018,16 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
       const uint32_t lo0 = sdesc_lo(smem_u32(smem));
       constexpr uint32_t id = idesc(C::tf32 ? 2u : 1u);
       int g = 0, it = 0;
+      int next = blockIdx.x < nu ? sy.order[blockIdx.x].np : 0;
       for (int u = blockIdx.x; u < nu && !s_abort; u += gridDim.x) {
-        const int o = sy.order[u];
+        const int np = next;
+        if (u + (int)gridDim.x < nu) next = sy.order[u + gridDim.x].np;
         const int buf = it & 1;
         if (it >= 2 && !mbar_wait(&tempty[buf], ((it >> 1) - 1) & 1, &s_abort)) break;
         tc_fence_after();
         const uint32_t d = tmem + buf * SB;
-        const int p0 = sy.pair_ptr[o], p1 = sy.pair_ptr[o + 1];
         bool first = true;
-        for (int p = p0; p < p1 && !s_abort; ++p) {
+        for (int p = 0; p < np && !s_abort; ++p) {
           for (int c = 0; c < chunks; ++c, ++g) {
             const int s = g % NS;
             if (!mbar_wait(kStaged<P> ? &conv[s] : &full[s], (g / NS) & 1, &s_abort)) break;
@@ -949,10 +1064,10 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
     __syncwarp();
   } else if (kStaged<P> && warp >= 6) {
     // converters: warps 6-9 A, 10-13 B
-    int g = 0;
+    int g = 0, next = blockIdx.x < nu ? sy.order[blockIdx.x].np : 0;
     for (int u = blockIdx.x; u < nu && !s_abort; u += gridDim.x) {
-      const int o = sy.order[u];
-      const int npc = (sy.pair_ptr[o + 1] - sy.pair_ptr[o]) * chunks;
+      const int npc = next * chunks;
+      if (u + (int)gridDim.x < nu) next = sy.order[u + gridDim.x].np;
       for (int i = 0; i < npc && !s_abort; ++i, ++g) {
         const int s = g % NS;
         if (!mbar_wait_warp(&full[s], (g / NS) & 1, &s_abort)) break;
@@ -968,34 +1083,34 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
     const int row = 32 * q + lane;
     double t1 = 0.0, t2 = 0.0;
     int it = 0;
+    Unit next{};
+    if (blockIdx.x < nu) next = load_unit(sy.order + blockIdx.x);
     for (int u = blockIdx.x; u < nu; u += gridDim.x) {
-      const int o = sy.order[u];
+      const Unit un = next;
+      if (u + (int)gridDim.x < nu) next = load_unit(sy.order + u + gridDim.x);
       const int buf = it & 1;
       ++it;
+      const int o = un.o, om = un.om, I = un.I, J = un.J, oi = un.oi;
+      const bool has = un.np > 0, mirror = J > I;
+      // a diagonal block of a product of two matrices is not exactly symmetric
+      // in rounding (A B against B A): its upper triangle is kept and mirrored
+      const bool symd = I == J && !a.same_ab;
+      float* xmir = bn.val + (size_t)om * kTiles;
+      // this warp's 32 rows of S_IJ and of the new block; the sub-tile of S that a step needs
+      // is fetched a step (the first one, the products) ahead
+      const float* xold = S.val + (size_t)(oi >= 0 ? oi : 0) * kTiles + (size_t)(32 * q) * SB;
+      const int c_first = symd ? q : 0;  // sub-blocks before it are written as mirrors
+      float4 xg[8];
+      if (oi >= 0) tile_fetch(xold + 32 * c_first, SB, lane, xg);
       if (!mbar_wait_warp(&tfull[buf], ((it - 1) >> 1) & 1, &s_abort)) break;
       tc_fence_after();
-      const bool has = sy.pair_ptr[o + 1] > sy.pair_ptr[o];
-      const int I = sy.out_row[o], J = bn.col[o];
-      const bool mirror = J > I;
-      // slot of the transposed block (J, I) in the new pattern
-      const int om = mirror ? bn.row_ptr[J] + popc_below(sy.cand + J * MW, I) : o;
-      float* xmir = bn.val + (size_t)om * kTiles;
-      const int oi = sy.old_idx[o];
-      // this warp's 32 rows of S_IJ and of the new block
-      const float* xold = S.val + (size_t)(oi >= 0 ? oi : 0) * kTiles + (size_t)(32 * q) * SB;
       float* xnew = bn.val + (size_t)o * kTiles + (size_t)(32 * q) * SB;
       // stored splits (not with kStaged)
       char* hrow = kStaged<P> ? nullptr : static_cast<char*>(bn.hi) + ((size_t)o * kTiles + (size_t)row * SB) * C::eb;
       char* lrow = bn.lo ? static_cast<char*>(bn.lo) + ((size_t)o * kTiles + (size_t)row * SB) * C::eb : hrow;
       int kept = 0;
-      // a diagonal block of a product of two matrices is not exactly symmetric
-      // in rounding (A B against B A): its upper triangle is kept and mirrored
-      const bool symd = I == J && !a.same_ab;
 #pragma unroll 1
-      for (int c = 0; c < 4; ++c) {
-        if (symd && c < q) continue;  // written as the mirror of sub-block (c, q)
-        float4 xg[8];
-        if (oi >= 0) tile_fetch(xold + 32 * c, SB, lane, xg);
+      for (int c = c_first; c < 4; ++c) {
         uint32_t v[32];
         if (has) {
           tmem_ld32(tmem + (static_cast<uint32_t>(32 * q) << 16) + buf * SB + 32 * c, v);
@@ -1007,6 +1122,7 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
         float xs[32];
         if (oi >= 0) {
           tile_turn_in(reinterpret_cast<uint8_t*>(s_sym[q]), lane, xg, xs);
+          if (c < 3) tile_fetch(xold + 32 * (c + 1), SB, lane, xg);
         } else {
 #pragma unroll
           for (int j = 0; j < 32; ++j) xs[j] = 0.0f;
@@ -1029,18 +1145,28 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
             if (j < lane) y[j] = s_sym[q][j][lane];
           __syncwarp();
         }
+        // The FP32 sum of the squares decides the sub-blocks that are clearly dropped (its
+        // rounding, 37 steps of 2^-24, is a fortieth of drop32's margin): only the others take FP64 work.
+        float s32 = 0.0f;
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          const double d = abs_to_f64(y[j]);
-          ss = fma(d, d, ss);
+        for (int j = 0; j < 32; ++j) s32 = fmaf(y[j], y[j], s32);
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) s32 += __shfl_xor_sync(0xffffffffu, s32, d);
+        const bool open = !(s32 < drop32);
+        if (open) {
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {
+            const double d = abs_to_f64(y[j]);
+            ss = fma(d, d, ss);
+          }
         }
         // squared Frobenius norm of sub-block (q, c); this lane's share of it is also its
         // share of ||X||_F^2 when the sub-block is kept.  (The FP64 pipe, at 1.7 results per
         // clock and SM, bounds the blocks of few products: one FMA per element and no
         // conversion leaves 5 us of the 19 us that two of each took.)
         const double mine = ss;
-        ss = warp_sum(ss);
-        const bool keep = ss >= a.tau2 && ss > 0.0;
+        if (open) ss = warp_sum(ss);
+        const bool keep = open && ss >= a.tau2 && ss > 0.0;
         if (!keep) {
 #pragma unroll
           for (int j = 0; j < 32; ++j) y[j] = 0.0f;
@@ -1246,8 +1372,8 @@ constexpr int kMaxBufs = 7;  // matrices of the Fermi expansion (SP2: two)
 struct BsrLayout {
   int n, ld, nsb, cap, pcap, nbuf;
   bool staged;  // tf32x3: FP32 masters only, no stored operand splits
-  size_t off_state, off_bparts, off_parts, off_scal, off_flags, off_cand, off_cnt, off_outrow, off_oldidx,
-      off_pcnt, off_pptr, off_pairs, off_order;
+  size_t off_state, off_bparts, off_parts, off_scal, off_flags, off_cand, off_cnt, off_oldidx,
+      off_rowp, off_ucnt, off_pcnt, off_pairs, off_order;
   size_t off_rp[kMaxBufs], off_col[kMaxBufs], off_nz[kMaxBufs], off_st[kMaxBufs], off_lv[kMaxBufs],
       off_val[kMaxBufs], off_hi[kMaxBufs], off_lo[kMaxBufs];
   size_t total;
@@ -1265,7 +1391,7 @@ BsrLayout bsr_layout(int n, int prec, int bpr, int nbuf) {
   const int per_row = (bpr <= 0 || bpr > L.nsb) ? L.nsb : bpr;
   L.cap = L.nsb * per_row;
   L.pcap = L.cap * per_row;
-  L.nparts = std::max(L.nsb, kMaxGrid);
+  L.nparts = std::max(kFillSplit * L.nsb, kMaxGrid);
   size_t o = 0;
   auto take = [&](size_t bytes) {
     size_t r = o;
@@ -1282,12 +1408,12 @@ BsrLayout bsr_layout(int n, int prec, int bpr, int nbuf) {
   L.off_flags = take(sizeof(uint16_t) * (size_t)L.nsb * L.nsb);
   L.off_cand = take(sizeof(uint32_t) * MW * L.nsb);
   L.off_cnt = take(sizeof(int) * L.nsb);
-  L.off_outrow = take(sizeof(int) * L.cap);
+  L.off_rowp = take(sizeof(int) * L.nsb);
+  L.off_ucnt = take(sizeof(int) * L.nsb);
   L.off_oldidx = take(sizeof(int) * L.cap);
-  L.off_pcnt = take(sizeof(int) * L.cap);
-  L.off_pptr = take(sizeof(int) * (L.cap + 1));
+  L.off_pcnt = take(sizeof(int2) * L.cap);
   L.off_pairs = take(sizeof(int2) * (size_t)L.pcap);
-  L.off_order = take(sizeof(int) * L.cap);
+  L.off_order = take(sizeof(Unit) * L.cap);
   for (int b = 0; b < nbuf; ++b) {
     L.off_rp[b] = take(sizeof(int) * (L.nsb + 1));
     L.off_col[b] = take(sizeof(int) * L.cap);
@@ -1342,13 +1468,13 @@ int bind_engine(tb_ctx* ctx, int prec, const BsrLayout& L, void* ws, Engine* e) 
   Sym& sy = e->sy;
   sy.cand = reinterpret_cast<uint32_t*>(base + L.off_cand);
   sy.cnt = reinterpret_cast<int*>(base + L.off_cnt);
-  sy.out_row = reinterpret_cast<int*>(base + L.off_outrow);
+  sy.rowp = reinterpret_cast<int*>(base + L.off_rowp);
+  sy.ucnt = reinterpret_cast<int*>(base + L.off_ucnt);
   sy.old_idx = reinterpret_cast<int*>(base + L.off_oldidx);
-  sy.pcnt = reinterpret_cast<int*>(base + L.off_pcnt);
-  sy.pair_ptr = reinterpret_cast<int*>(base + L.off_pptr);
+  sy.pcnt = reinterpret_cast<int2*>(base + L.off_pcnt);
   sy.pairs = reinterpret_cast<int2*>(base + L.off_pairs);
   sy.scal = reinterpret_cast<int*>(base + L.off_scal);
-  sy.order = reinterpret_cast<int*>(base + L.off_order);
+  sy.order = reinterpret_cast<Unit*>(base + L.off_order);
   sy.flags = reinterpret_cast<uint16_t*>(base + L.off_flags);
   for (int i = 0; i < L.nbuf; ++i) {
     Buf& b = e->m[i].b;
@@ -1404,8 +1530,8 @@ int launch_start(tb_ctx* ctx, Engine& e, const Args& a, const double* H, const t
   TB_LAUNCH_CHECK(ctx);
   k_bsr_scan_rows<<<1, 32, 0, s>>>(a, e.sy, out.b.row_ptr);
   TB_LAUNCH_CHECK(ctx);
-  if (Hb) k_bsr_init_fill_in<P><<<nsb, 256, 0, s>>>(*Hb, a, e.sy, out.b);
-  else k_bsr_init_fill<P><<<nsb, 256, 0, s>>>(H, a, e.sy, out.b);
+  if (Hb) k_bsr_init_fill_in<P><<<dim3(nsb, kFillSplit), 256, 0, s>>>(*Hb, a, e.sy, out.b);
+  else k_bsr_init_fill<P><<<dim3(nsb, kFillSplit), 256, 0, s>>>(H, a, e.sy, out.b);
   TB_LAUNCH_CHECK(ctx);
   return TB_OK;
 }
@@ -1422,11 +1548,9 @@ int launch_product(tb_ctx* ctx, Engine& e, Args a, const Mat& A, const Mat& B, c
   const Buf& Sb = S ? S->b : none;
   const int nsb = e.L.nsb;
   k_bsr_cand<<<nsb, 256, 0, s>>>(a, A.b, B.b, Sb, e.sy);
-  k_bsr_scan_rows<<<1, 32, 0, s>>>(a, e.sy, out.b.row_ptr);
   k_bsr_fill_out<<<nsb, 256, 0, s>>>(a, A.b, B.b, Sb, out.b, e.sy);
-  k_bsr_scan_pairs<<<1, 1024, 0, s>>>(a, e.sy);
-  k_bsr_pairs<<<std::max(1, std::min(e.L.cap, 4096) / 128 + 1), 128, 0, s>>>(a, A.b, B.b, out.b, e.sy);
-  k_bsr_order<<<1, 1024, 0, s>>>(a, out.b, e.sy);
+  const int nlist = (nsb + kBand - 1) / kBand * a.mw;  // a warp each
+  k_bsr_pairs<<<nsb * kPairSplit + (nlist + 7) / 8, 256, 0, s>>>(a, A.b, B.b, out.b, e.sy);
   TB_LAUNCH_CHECK(ctx);
   if (prof_k >= 0) tb_prof_mark(ctx, 1, 2 * prof_k, s);
   k_bsr_step_tc<P><<<grid, kNumThreads<P>, kNumSmem<P>, s>>>(a, A.mh, A.ml, B.mh, B.ml, Sb, out.b, e.sy, ep);
@@ -1490,7 +1614,7 @@ int run_bsr(tb_ctx* ctx, const double* H, const tb_bsr* Hb, int n, double nocc, 
   for (int k = 0; k <= o->max_iter; ++k) {
     a.k = k;
     a.parts_in = slot[k & 1];
-    a.nparts_in = k == 0 ? L.nsb : grid;
+    a.nparts_in = k == 0 ? kFillSplit * L.nsb : grid;
     a.parts_out = slot[(k + 1) & 1];
     Mat& bo = e.m[k & 1];
     Mat& bn = e.m[(k + 1) & 1];
