@@ -13,10 +13,10 @@
 // at most 1024 super-rows and each row's pattern is a 1024-bit bitmap.
 //
 // Per projection (all on the device, no host synchronisation):
-//   decide  reduce the trace partials of X_k, take the stop/branch decision
-//           (every CTA the same), build each row's bitmaps of stored and live
-//           (not all-zero) super-blocks;
-//   symbolic  candidates of row I = OR of the live bitmaps of its live
+//   symbolic  reduce the trace partials of X_k and take the stop/branch decision
+//           (every CTA the same); each row has bitmaps of its stored and its live
+//           (not all-zero) super-blocks, written with the pattern and by the numeric
+//           kernel; candidates of row I = OR of the live bitmaps of its live
 //           columns; every block scans the rows' counts for the output slots; each upper output block
 //           (I <= J; X^2 and its pattern are symmetric) gets the list of common
 //           K (live in both rows I and J) as pairs of source slots; the upper
@@ -78,7 +78,6 @@ inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 struct Buf {
   int* row_ptr;      // [nsb + 1]
   int* col;          // [cap]
-  int* nz;           // [cap] live flag (some sub-block kept)
   uint32_t* stored;  // [nsb * MW]
   uint32_t* live;    // [nsb * MW]
   float* val;        // [cap * kTiles] FP32 master
@@ -365,10 +364,7 @@ __device__ void x0_fill_row(const Args& a, const Sym& sy, const Buf& b, Src src)
     const int nc = max(0, a.n - J * SB);
     size_t ld = 0;
     const double* h = src(J, &ld);
-    if (threadIdx.x == 0) {
-      b.col[o] = J;
-      b.nz[o] = f != 0;
-    }
+    if (threadIdx.x == 0) b.col[o] = J;
 #pragma unroll 1
     for (int q = warp; q < 16; q += 8) {
       const int r0 = 32 * (q >> 2), c0 = 32 * (q & 3), c = c0 + lane;
@@ -600,28 +596,16 @@ __global__ void __launch_bounds__(256) k_bsr_init_fill_in(tb_bsr H, Args a, Sym 
 
 // ------------------------------------------------------- per projection
 
-// Bitmaps of row I of b: stored blocks and live (not all-zero) blocks; ms and
-// ml are zeroed shared arrays of the calling block.
-__device__ void row_bitmaps(const Buf& b, int I, uint32_t* ms, uint32_t* ml) {
-  for (int o = b.row_ptr[I] + threadIdx.x; o < b.row_ptr[I + 1]; o += blockDim.x) {
-    const int J = b.col[o];
-    atomicOr(&ms[J >> 5], 1u << (J & 31));
-    if (b.nz[o]) atomicOr(&ml[J >> 5], 1u << (J & 31));
-  }
-  __syncthreads();
-  if (threadIdx.x < MW) {
-    b.stored[I * MW + threadIdx.x] = ms[threadIdx.x];
-    b.live[I * MW + threadIdx.x] = ml[threadIdx.x];
-  }
+// Whether the call is finished or failed, the same for every thread of the block also where
+// another block of this launch sets the error.
+__device__ __forceinline__ bool stopped(const SP2State* st) {
+  return __syncthreads_or(threadIdx.x == 0 && (st->done || st->err));
 }
 
-// Decision for projection k (every block the same) and the bitmaps of row I
-// of X_k: stored blocks and live (not all-zero) blocks.
-__global__ void k_bsr_decide(Args a, Buf b) {
+// Decision for projection k, the same in every block (256 threads): whether the phase stops.
+__device__ bool bsr_decide(const Args& a) {
   __shared__ int s_stop;
-  __shared__ uint32_t ms[MW], ml[MW];
   SP2State* st = a.st;
-  if (st->done || st->err) return;
   if (threadIdx.x < 32) {
     double x = 0, y = 0;
     for (int i = threadIdx.x; i < a.nparts_in; i += 32) {
@@ -654,35 +638,19 @@ __global__ void k_bsr_decide(Args a, Buf b) {
       }
     }
   }
-  if (threadIdx.x < MW) {
-    ms[threadIdx.x] = 0u;
-    ml[threadIdx.x] = 0u;
-  }
   __syncthreads();
-  if (s_stop) return;
-  row_bitmaps(b, blockIdx.x, ms, ml);
-}
-
-// Bitmaps of stored and live blocks of every row of a product's output.
-__global__ void k_bsr_bitmaps(Args a, Buf b) {
-  __shared__ uint32_t ms[MW], ml[MW];
-  if (a.st->done || a.st->err) return;
-  if (threadIdx.x < MW) {
-    ms[threadIdx.x] = 0u;
-    ml[threadIdx.x] = 0u;
-  }
-  __syncthreads();
-  row_bitmaps(b, blockIdx.x, ms, ml);
+  return s_stop;
 }
 
 // Candidate columns of row I of A B: the OR of B's live rows over A's live
 // columns of row I; unless A and B are one matrix also the same with A and B
 // exchanged (the pattern of B A = (A B)^T), so that the pattern is symmetric
 // as the upper-block computation with mirrors needs; S's live blocks; the
-// diagonal block with keep_diag.  A and B are symmetric (rows = columns).
-__global__ void k_bsr_cand(Args a, Buf A, Buf B, Buf S, Sym sy) {
+// diagonal block with keep_diag.  With `decide` the projection's decision first.  A and B are symmetric (rows = columns).
+__global__ void __launch_bounds__(256) k_bsr_cand(Args a, Buf A, Buf B, Buf S, Sym sy, bool decide) {
   __shared__ uint32_t c[MW];
-  if (a.st->done || a.st->err) return;
+  if (stopped(a.st)) return;
+  if (decide && bsr_decide(a)) return;
   const int I = blockIdx.x;
   if (threadIdx.x < MW) c[threadIdx.x] = 0u;
   __syncthreads();
@@ -743,12 +711,6 @@ __device__ void rows_prefix(const int* __restrict__ v, int nsb, int I, long long
   *total = t;
 }
 
-// Whether the call is finished or failed, the same for every thread of the block also where
-// another block of this launch sets the error.
-__device__ __forceinline__ bool stopped(const SP2State* st) {
-  return __syncthreads_or(threadIdx.x == 0 && (st->done || st->err));
-}
-
 // Output blocks of row I: its start, and for each block the column, the slot of S_IJ (or
 // -1) and the pairs of the row's blocks before it; the row's pairs and upper blocks.
 __global__ void __launch_bounds__(256) k_bsr_fill_out(Args a, Buf A, Buf B, Buf S, Buf bn, Sym sy) {
@@ -769,6 +731,10 @@ __global__ void __launch_bounds__(256) k_bsr_fill_out(Args a, Buf A, Buf B, Buf 
   const uint32_t* ci = sy.cand + I * MW;
   const uint32_t* si = S.stored ? S.stored + I * MW : nullptr;
   const uint32_t* li = A.live + I * MW;
+  if (threadIdx.x < MW) {  // the numeric kernel adds the live ones
+    bn.stored[I * MW + threadIdx.x] = ci[threadIdx.x];
+    bn.live[I * MW + threadIdx.x] = 0u;
+  }
   int run = 0, upper = 0;
   long long prod = 0;  // a block above the diagonal has a mirror with as many products
   for (int J0 = 0; J0 < a.nsb; J0 += 256) {
@@ -798,7 +764,6 @@ __global__ void __launch_bounds__(256) k_bsr_fill_out(Args a, Buf A, Buf B, Buf 
     if (has) {
       const int o = (int)base + popc_below(ci, J);
       bn.col[o] = J;
-      bn.nz[o] = 0;
       sy.old_idx[o] = (si && ((si[J >> 5] >> (J & 31)) & 1u)) ? S.row_ptr[I] + popc_below(si, J) : -1;
       sy.pcnt[o] = make_int2(before + incl - pc, pc);
     }
@@ -1256,10 +1221,9 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
       tc_fence_before();
       if (lane == 0) {
         // the block is live when any of its 32-row bands kept a sub-block
-        // (nz[o] was zeroed when the output pattern was built)
         if (kept) {
-          atomicOr(&bn.nz[o], 1);
-          if (mirror) atomicOr(&bn.nz[om], 1);
+          atomicOr(&bn.live[I * MW + (J >> 5)], 1u << (J & 31));
+          if (mirror) atomicOr(&bn.live[J * MW + (I >> 5)], 1u << (I & 31));
         }
         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tempty[buf])) : "memory");
       }
@@ -1307,7 +1271,7 @@ __global__ void k_bsr_to_dense(const SP2State* st, Args a, Buf b0, Buf b1, Sym s
 }
 
 // out = alpha X + delta I on X's pattern (X stores every diagonal block when
-// delta != 0): values, operand splits, live flags and bitmaps.  Exact up to
+// delta != 0): values, operand splits and bitmaps.  Exact up to
 // the FP32 rounding of the values; nothing is dropped.
 template <int P>
 __global__ void __launch_bounds__(256) k_bsr_affine(Args a, Buf X, Buf out, float alpha, float delta) {
@@ -1323,10 +1287,7 @@ __global__ void __launch_bounds__(256) k_bsr_affine(Args a, Buf X, Buf out, floa
   for (int o = blockIdx.x; o < nblk; o += gridDim.x) {
     const int I = slot_row(X, a.nsb, o), J = X.col[o];
     const bool diag = I == J && delta != 0.0f;
-    if (threadIdx.x == 0) {
-      out.col[o] = J;
-      out.nz[o] = X.nz[o] | (diag ? 1 : 0);
-    }
+    if (threadIdx.x == 0) out.col[o] = J;
     if constexpr (kStaged<P>) {
       // 16 bytes a lane, consecutive across the block, several loads in flight (a thread
       // per 32-value segment took 0.31 ms for what memory moves in 0.05)
@@ -1432,7 +1393,7 @@ struct BsrLayout {
   bool staged;  // tf32x3: FP32 masters only, no stored operand splits
   size_t off_state, off_bparts, off_parts, off_scal, off_flags, off_cand, off_cnt, off_oldidx,
       off_rowp, off_ucnt, off_pcnt, off_pairs, off_list, off_npl, off_order;
-  size_t off_rp[kMaxBufs], off_col[kMaxBufs], off_nz[kMaxBufs], off_st[kMaxBufs], off_lv[kMaxBufs],
+  size_t off_rp[kMaxBufs], off_col[kMaxBufs], off_st[kMaxBufs], off_lv[kMaxBufs],
       off_val[kMaxBufs], off_hi[kMaxBufs], off_lo[kMaxBufs];
   size_t total;
   int nparts;
@@ -1477,7 +1438,6 @@ BsrLayout bsr_layout(int n, int prec, int bpr, int nbuf) {
   for (int b = 0; b < nbuf; ++b) {
     L.off_rp[b] = take(sizeof(int) * (L.nsb + 1));
     L.off_col[b] = take(sizeof(int) * L.cap);
-    L.off_nz[b] = take(sizeof(int) * L.cap);
     L.off_st[b] = take(sizeof(uint32_t) * MW * L.nsb);
     L.off_lv[b] = take(sizeof(uint32_t) * MW * L.nsb);
     L.off_val[b] = take(sizeof(float) * (size_t)L.cap * kTiles);
@@ -1542,7 +1502,6 @@ int bind_engine(tb_ctx* ctx, int prec, const BsrLayout& L, void* ws, Engine* e) 
     Buf& b = e->m[i].b;
     b.row_ptr = reinterpret_cast<int*>(base + L.off_rp[i]);
     b.col = reinterpret_cast<int*>(base + L.off_col[i]);
-    b.nz = reinterpret_cast<int*>(base + L.off_nz[i]);
     b.stored = reinterpret_cast<uint32_t*>(base + L.off_st[i]);
     b.live = reinterpret_cast<uint32_t*>(base + L.off_lv[i]);
     b.val = reinterpret_cast<float*>(base + L.off_val[i]);
@@ -1604,12 +1563,12 @@ int launch_start(tb_ctx* ctx, Engine& e, const Args& a, const double* H, const t
 // is none of A, B, S.  prof_k >= 0 marks the numeric launch for profiling.
 template <int P>
 int launch_product(tb_ctx* ctx, Engine& e, Args a, const Mat& A, const Mat& B, const Mat* S, Mat& out, Epi ep,
-                   int grid, cudaStream_t s, int prof_k = -1) {
+                   int grid, cudaStream_t s, bool decide = false, int prof_k = -1) {
   a.same_ab = &A == &B;
   const Buf none{};
   const Buf& Sb = S ? S->b : none;
   const int nsb = e.L.nsb;
-  k_bsr_cand<<<nsb, 256, 0, s>>>(a, A.b, B.b, Sb, e.sy);
+  k_bsr_cand<<<nsb, 256, 0, s>>>(a, A.b, B.b, Sb, e.sy, decide);
   k_bsr_fill_out<<<nsb, 256, 0, s>>>(a, A.b, B.b, Sb, out.b, e.sy);
   const int nlist = (nsb + kBand - 1) / kBand * a.mw;  // a warp each
   k_bsr_pairs<<<nsb * kPairSplit + (nlist + 7) / 8, 256, 0, s>>>(a, A.b, B.b, out.b, e.sy);
@@ -1681,8 +1640,7 @@ int run_bsr(tb_ctx* ctx, const double* H, const tb_bsr* Hb, int n, double nocc, 
     a.parts_out = slot[(k + 1) & 1];
     Mat& bo = e.m[k & 1];
     Mat& bn = e.m[(k + 1) & 1];
-    k_bsr_decide<<<L.nsb, 128, 0, s>>>(a, bo.b);
-    if ((rc = launch_product<P>(ctx, e, a, bo, bo, &bo, bn, sp2_epi, grid, s, k))) return rc;
+    if ((rc = launch_product<P>(ctx, e, a, bo, bo, &bo, bn, sp2_epi, grid, s, true, k))) return rc;
     tb_prof_mark(ctx, 0, k + 1, s);
   }
   if (Db) {
@@ -1775,7 +1733,6 @@ int run_bsr_fermi(tb_ctx* ctx, const tb_bsr* Hb, int n, double nocc, double kT, 
   auto product = [&](const Mat& X1, const Mat& X2, const Mat* S, Mat& out, Epi ep) -> int {
     int r = launch_product<P>(ctx, e, a, X1, X2, S, out, ep, grid, s);
     if (r) return r;
-    k_bsr_bitmaps<<<L.nsb, 128, 0, s>>>(a, out.b);
     TB_LAUNCH_CHECK(ctx);
     return TB_OK;
   };

@@ -299,20 +299,6 @@ __device__ __forceinline__ double abs_to_f64(float x) {
   return __hiloint2double((int)hi, (int)lo);
 }
 
-// Deterministic sum of `np` partial pairs by one warp (fixed order): lane l
-// adds partials l, l+32, ..., then a fixed butterfly.  Same result in every CTA.
-__device__ __forceinline__ void warp_reduce_partials(const double* parts, int np, double* s0,
-                                                     double* s1) {
-  const int lane = threadIdx.x & 31;
-  double a = 0.0, b = 0.0;
-  for (int i = lane; i < np; i += 32) {
-    a += parts[2 * i];
-    b += parts[2 * i + 1];
-  }
-  *s0 = warp_sum(a);
-  *s1 = warp_sum(b);
-}
-
 // Decision of SP2 projection k from the traces of X_k (t1 = Tr X, t2 = Tr X^2).
 // Returns 1 when the phase stops before projection k (setting *capped when
 // the iteration cap was the reason), else 0 and sets *branch.

@@ -23,7 +23,8 @@
 // dropped one, (5, 5), biases by ~K 2^-62.  22 bf16 products replace one FP64
 // GEMM (6-bit slices would need 7 slices and 28 products for the same bounds).
 
-// Kernel layout: one CTA per 128 x 128 tile of the upper triangle (X^2 is
+// Kernel layout: one CTA per 128 x 128 tile of the upper triangle, or per 32 or 64
+// columns of one where the matrix has few tiles (oz_unit) (X^2 is
 // symmetric; the epilogue also writes each off-diagonal tile transposed,
 // one coalesced 32-lane store per column); warp 0 issues TMA loads
 // of (slice s, row block m) and (slice t, row block n) tiles, warp 1 issues

@@ -6,13 +6,15 @@
 // Tr X and Tr X^2 = ||X||_F^2 (look-ahead rule: the projection whose trace
 // lands closer to N_occ); stop when Tr X - Tr X^2 <= tol.
 //
-// Device-side control: step kernel k first reduces, in a fixed order, the
-// trace partials written by the epilogue of kernel k-1, takes the
-// stop/branch decision (identical in every CTA) and either returns at once
-// or computes X_{k+1}.  Launched eagerly, the host enqueues max_iter + 1 step
-// kernels; captured into a CUDA graph, the projections after the first are
-// a while node that stops with the decision.  No host synchronisation
-// happens inside dm_sp2.
+// Device-side control: the projections run in one launch (sp2_run.cu, sp2_run64.cu: a grid
+// barrier between them, nothing after the stop) where that is the faster form: FP64 up to
+// n = 512, tf32 and tf32x3 below ld = 4096 or where CTA pairs do not pay.  Otherwise (and while
+// projections are being timed) step kernel k first reduces, in a fixed order, the trace
+// partials written by the epilogue of kernel k-1, takes the stop/branch decision
+// (identical in every CTA) and either returns at once or computes X_{k+1}: launched
+// eagerly, the host enqueues max_iter + 1 step kernels; captured into a CUDA graph, the
+// projections after the first are a while node that stops with the decision.  No host
+// synchronisation happens inside dm_sp2.
 //
 // Precision paths: TB_PREC_FP64 runs every projection as an FP64 GEMM (16 x 16
 // output tiles for ld <= 512, 64 x 64 above); the tensor-core paths

@@ -100,17 +100,6 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
   d |= static_cast<uint64_t>(2) << 61;
   return d;
 }
-// The same for a 64-byte swizzle (layout type 4): 8-row groups of 64-byte
-// rows, 512 bytes apart.
-__device__ __forceinline__ uint64_t sdesc64(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);
-  d |= static_cast<uint64_t>(1) << 16;
-  d |= static_cast<uint64_t>(512 >> 4) << 32;
-  d |= static_cast<uint64_t>(1) << 46;
-  d |= static_cast<uint64_t>(4) << 61;
-  return d;
-}
 // One thread of a warp, picked the way the compiler knows to be one (so that what it
 // computes for tcgen05 instructions can stay in uniform registers).
 __device__ __forceinline__ bool elect_one() {
