@@ -186,7 +186,7 @@ __device__ __forceinline__ void x0_affine(const Args& a, double* e, double* s) {
 }
 
 // Whether any lane's value is not zero (an integer test and a vote: a few cycles,
-// where an FP64 instruction of a warp takes 19).
+// where an FP64 instruction of a warp takes 76 of its scheduler).
 // The halves come from a move that the compiler does not see through: it turns the
 // test of a double's bits into a comparison in FP64.
 __device__ __forceinline__ bool nonzero_bits(double x) {
@@ -219,7 +219,7 @@ __device__ __forceinline__ void gather_add(double v, double& p, Fn flush) {
 // in one warp, few FP64 instructions to a sub-block (gather_add).  Called by
 // every thread of the block, which all get the mask.  (Sums of each of the 16 sub-blocks in
 // every warp, combined through shared memory, took 80 FP64 additions a warp and a serial
-// sum of 128: 849 us at 16383 orbitals.)
+// sum of 128: 849 us for the 16383 atoms of a vapour, 194 us now.)
 template <class X>
 __device__ __forceinline__ uint16_t block_keep(const Args& a, double scale2, X x) {
   __shared__ unsigned s_mask;
@@ -341,7 +341,7 @@ __global__ void k_bsr_scan_rows(Args a, Sym sy, int* row_ptr) {
 // src(J, &ld): H's super-block (I, J) (null: zero).  A warp takes a sub-block at a time, its
 // lanes the columns: whole-row loads and stores; dropped sub-blocks and rows that are all
 // zero take no FP64 work.  (One thread block a row, 32 elements of a row to a thread: 325 us
-// at 16383 orbitals.)
+// for 16383 atoms, 51 us now.)
 constexpr int kFillSplit = 4;
 template <int P, class Src>
 __device__ void x0_fill_row(const Args& a, const Sym& sy, const Buf& b, Src src) {
@@ -462,13 +462,13 @@ __device__ __forceinline__ int bsr_find(const int* __restrict__ row_ptr, const i
   return -1;
 }
 
-// Gershgorin partials of block row I (kBndSplit blocks of 256 threads, 16 rows
-// each): warp w takes rows w + 8k, lane l the columns 32 c + l, so each block is read
-// as 8 independent coalesced loads a lane, two blocks at a time, and the row sums stay in registers until
-// one warp sum per row; min(H_ii - r_i) and max(H_ii + r_i) over the rows go into
-// bparts[2 (I kBndSplit + y)].  The FP64 pipe would bound this kernel (1.1 ms for the
-// 1.2 GB of a 16 383-atom H): pieces of rows that are all zero, most of a block of a
-// molecular H, are skipped.
+// Gershgorin partials of block row I (kBndSplit blocks of 256 threads, 16 rows each): warp w
+// takes rows w + 8k, lane l the columns 32 c + l, so each block is read as 8 independent
+// coalesced loads a lane, two blocks at a time, and the row sums stay in registers until one
+// warp sum per row; min(H_ii - r_i) and max(H_ii + r_i) over the rows go into
+// bparts[2 (I kBndSplit + y)].  One addition an element would make the FP64 pipe the bound
+// (1.1 ms for the 1.2 GB of a 16383-atom H); the elements are gathered (gather_add) first:
+// 0.40 ms, against 0.18 ms for the bytes.
 constexpr int kBndSplit = 8;
 __global__ void __launch_bounds__(256) k_bsr_bounds_in(tb_bsr H, double* __restrict__ bparts) {
   __shared__ double smin[8], smax[8];
@@ -788,7 +788,7 @@ __global__ void __launch_bounds__(256) k_bsr_fill_out(Args a, Buf A, Buf B, Buf 
 // - blocks below nsb * kPairSplit: the pairs (slot of A_IK, slot of B_JK) of every upper
 //   output block (I, J), (A B)_IJ = sum_K A_IK B_JK^T for a symmetric B: a warp per output
 //   block, its lanes the columns K of a bitmap word, so that the pairs are written
-//   coalesced (a thread per output block: 11 us a projection at 128 block rows, and the
+//   coalesced (a thread per output block: 11 us a projection at 256 block rows, and the
 //   scan of the pair counts before it another 11);
 // - the others: the upper output blocks (I <= J) in (band of kBand block rows, column J,
 //   row I) order.  The persistent numeric kernel takes them in this order, so the CTAs
@@ -899,7 +899,7 @@ __global__ void __launch_bounds__(256) k_bsr_pairs(Args a, Buf A, Buf B, Buf bn,
 // The numeric kernel's order: the band list sorted (stably) into classes of falling pair
 // counts (four to an octave), which its thread blocks take in rounds of alternating
 // direction: no two of them differ by more than about one block's work, where the band list
-// in rounds left the mean one a quarter of the time idle (16383 orbitals: 154 -> 126 us a
+// in rounds left the mean one a quarter of the time idle (16383 atoms: 154 -> 126 us a
 // projection; a liquid of 4096 atoms 39.0 -> 35.6 ms in all).  Within a class the bands stay
 // together.  A thread block per class.
 constexpr int kClasses = 44;  // up to 1024 pairs: ten octaves and one

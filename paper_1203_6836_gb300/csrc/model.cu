@@ -1167,7 +1167,7 @@ constexpr int kPairList = 4096;
 // Bound by the 64-bit work of the pairs in range (few of a block's pairs) and by the stores
 // of the zeroed blocks: 959 us with every warp running the pairs' branch for whichever of
 // its lanes were in range and the six divisions of the image bounds, 363 us with the list
-// (16383 orbitals, 0.1 g/cc).
+// (16383 atoms, 0.1 g/cc).
 // The h elements of stored block o (one CTA per block, grid-stride): every
 // ordered atom pair (i, j) of the two rows, summed over the images within the
 // cut-off, onsite energies for i == j; each element belongs to one pair.
@@ -1291,7 +1291,7 @@ __global__ void __launch_bounds__(256) k_h_blocks(ModelDev m, int N, const int32
 // warp's list (kNbList entries): fn(j) by full warps, a list at a time, each lane taking
 // its entries in list order.  A warp that ran fn for the lanes in range of each 32 atoms
 // spent most of its 64-bit issue on masked lanes: k_v_bsr 662 -> 213 us and k_forces_bsr
-// 926 -> 483 us at 16383 orbitals (with for_images' short form).
+// 926 -> 483 us at 16383 atoms (with for_images' short form).
 constexpr int kNbList = 256;
 template <class Fn>
 __device__ __forceinline__ void for_atoms_in_range(const tb_bsr& H, const BsrModelWs& w, const ModelDev& m, int I,
