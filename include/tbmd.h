@@ -195,8 +195,8 @@ int tb_ctx_set_wait_limit(tb_ctx* ctx, unsigned long long ns);
  * tcgen05.mma.cta_group::2, which halves the operand bytes each SM loads per
  * flop; otherwise (and for every other tensor-core product) one CTA computes
  * a 128 x 128 tile.  TB_SP2_FORM_AUTO (the default) takes the pair form
- * where its tile schedule is predicted to finish first (on GB300: ld = 4096
- * and up), TB_SP2_FORM_SINGLE never, TB_SP2_FORM_PAIRS wherever ld allows.
+ * where its tile schedule is predicted to finish first (on GB300: ld = 2304
+ * to 2816 and from 3328), TB_SP2_FORM_SINGLE never, TB_SP2_FORM_PAIRS wherever ld allows.
  * Both forms compute the same products in the same order; results agree to
  * the order of the FP64 trace sums.  A grid limit (tb_ctx_set_grid_limit)
  * caps the pair form at max_ctas / 2 clusters.  TB_ERR_ARG for an unknown

@@ -11,8 +11,8 @@
 // k_sp2_step_tc: X is bitwise the same.  The FP64 trace partials have a slot per 128 x
 // 32 chunk, so the sums do not depend on the grid.
 //
-// From ld = 4096 on dm_sp2 takes the launched CTA-pair form, which halves the operand
-// bytes per flop and where a launch is 1% of a projection.
+// Where CTA pairs are the faster form (sp2_tc_pairs in gemm_tc.cu) dm_sp2 takes that one,
+// launched: it halves the operand bytes per flop, and a launch is 1% of its projection.
 
 #include "persist.cuh"
 #include "sp2_run.cuh"
