@@ -14,7 +14,8 @@
 //     multiplied further has no FP32 master;
 //   - a unit (128 x BN of the upper triangle) always belongs to the same CTA,
 //     so the FP32 values an epilogue adds (E, W, L) are its own earlier stores,
-//     and only the TMA producer waits at the barriers.
+//     and only the TMA producer waits at the barriers (the stores are another warp's, so
+//     a value of the product just before is read behind that wait all the same).
 // Same operand values, products and order of accumulation per element as the
 // launched form (k_gemm_tc): the matrices are bitwise the same.
 //
@@ -285,8 +286,11 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_foe_run(const FoeRunArgs a, 
           const RunUnit un = run_unit<BN>(wu, u);
           const int r0 = un.I * 128, gr = r0 + 32 * q + lane;
           const bool diag = un.I == un.J;
-          // the FP32 values added: this CTA's own earlier stores, past L1 (TMA wrote
-          // them), fetched while the MMAs run
+          // The FP32 values added: this CTA's own earlier stores, past L1 (TMA wrote them).
+          // E and L are at least one grid barrier old here, so they are fetched while the
+          // MMAs run.  W (kZ1) is the product just before, whose stores another warp may
+          // still be issuing: it is fetched behind tfull, which comes after the barrier that
+          // this CTA's store warp arrives at when its stores are written.
           float ev[16];
           auto load_e = [&](int row, int col) {
             const float4* e4 = reinterpret_cast<const float4*>(a.m[r.e] + (size_t)row * a.ld + col);
@@ -299,8 +303,9 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_foe_run(const FoeRunArgs a, 
               ev[4 * j + 3] = t.w;
             }
           };
-          if (r.e >= 0) load_e(gr, un.J * 128 + un.c0 + 16 * half);
+          if (r.e >= 0 && r.kind != kZ1) load_e(gr, un.J * 128 + un.c0 + 16 * half);
           if (!mbar_wait_warp(&tfull[buf], (t_epi >> 1) & 1, &s_abort, wl)) break;
+          if (r.kind == kZ1) load_e(gr, un.J * 128 + un.c0 + 16 * half);
           tc_fence_after();
 #pragma unroll 1
           for (int c = 0; c < un.nc; c += 32) {
