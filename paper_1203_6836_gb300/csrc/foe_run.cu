@@ -93,9 +93,8 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_foe_run(const FoeRunArgs a, 
   const StageRing ring{smem + Q::stages * Q::stage_bytes, sfull, sfree};
   const unsigned G = gridDim.x;
   const RunUnits wu = run_units<BN>(a.ld, (int)G);
-  // the CTAs that have units arrive at the barriers (a cluster may have a few more)
-  const unsigned Gw = min(G, (unsigned)wu.U);
-  const bool works = blockIdx.x < Gw;
+  const unsigned Gw = min(G, (unsigned)wu.U);  // the CTAs that arrive at the barriers
+  if (blockIdx.x >= Gw) return;                // no units
   const unsigned long long wl = a.wait_ns ? a.wait_ns : kWaitNs;  // pipeline wait limit
   const int nk = a.ld / 32;
   unsigned* bar = &a.st->bar;
@@ -133,7 +132,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_foe_run(const FoeRunArgs a, 
   int g = 0, t_mma = 0, t_epi = 0, issued = 0;  // g: stages gone through by this role
   int used = 0;                                 // arrays put through the staging ring
   uint32_t cpar = 0, gopar = 0;                 // parities of the next conv (a bit per stage) and go phase
-  const int mine = (int)blockIdx.x < wu.U ? (wu.U - 1 - (int)blockIdx.x) / (int)G + 1 : 0;  // units of this CTA
+  const int mine = (wu.U - 1 - (int)blockIdx.x) / (int)G + 1;  // units of this CTA
   unsigned phase = 0;                           // barrier phases completed before this expansion
   while (s_go) {
     if (warp == 0 && lane == 0) {
@@ -205,7 +204,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_foe_run(const FoeRunArgs a, 
                 break;
         }
         tma_store_wait();
-        if (works && !s_abort) run_arrive(bar);
+        if (!s_abort) run_arrive(bar);
       }
     } else if (warp == 10) {
       // ------------------------------------------------------------ diagonal patches
@@ -271,7 +270,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_foe_run(const FoeRunArgs a, 
         }
         fence_async_all();
         epi_sync();
-        if (eid == 0 && works) run_arrive(bar);
+        if (eid == 0) run_arrive(bar);
       }
       const int q = warp & 3, half = (warp - 2) >> 2;
       for (int p = 0; p < np && !s_abort; ++p) {

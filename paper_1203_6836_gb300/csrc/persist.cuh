@@ -93,10 +93,11 @@ __device__ __forceinline__ void fence_async_shared() {
 
 // Grid barrier: every CTA that has units adds one per phase to a counter that
 // is zero at the start of the call; phase p is over when it reaches p times
-// their number.  (A CTA without units has nothing that paces its arrivals, so
-// it only waits.)  The CTAs must be co-resident (a cooperative launch, or a
-// grid of one cluster).  A wait gives up after kWaitNs, or once another CTA has
-// recorded an error.
+// their number.  (A cluster, a power of two, may hold CTAs without units.  Nothing would
+// pace them: the others could be two phases ahead, rewriting the buffers from which an
+// idle one still takes its decision.  They leave at once.)  The CTAs must be co-resident
+// (a cooperative launch, or a grid of one cluster).  A wait gives up after kWaitNs, or
+// once another CTA has recorded an error.
 __device__ __forceinline__ void run_arrive(unsigned* bar) {
   asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
 }
@@ -346,7 +347,7 @@ inline bool tb_run_shape(const tb_ctx* ctx, int ld, int captured, RunShape* r) {
   r->grid = U < most ? U : most;
   r->cluster = r->grid <= 16;
   if (r->cluster) {
-    int c = 1;  // a power of two: at most one round more, or CTAs that only wait at the barrier
+    int c = 1;  // a power of two: at most one round more, or CTAs that leave at once
     while (c < r->grid && 2 * c <= most) c *= 2;
     r->grid = c;
   }

@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_sp2_run(const Sp2RunArgs g0,
   const unsigned G = gridDim.x;
   const RunUnits wu = run_units<BN>(a.ld, (int)G);
   const unsigned Gw = min(G, (unsigned)wu.U);  // the CTAs that arrive at the barriers
-  const bool works = blockIdx.x < Gw;
+  if (blockIdx.x >= Gw) return;                // no units
   const unsigned long long wl = a.wait_ns ? a.wait_ns : kWaitNs;  // pipeline wait limit
   const int nk = a.ld / 32;
   const int slots = 4 * wu.tiles;
@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_sp2_run(const Sp2RunArgs g0,
         }
         tma_store_wait();
         if (s_abort) break;
-        if (works) run_arrive(g0.bar);
+        run_arrive(g0.bar);
       }
       tma_store_wait();
     }
@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_sp2_run(const Sp2RunArgs g0,
       }
       fence_async_all();
       epi_sync();
-      if (eid == 0 && works) {
+      if (eid == 0) {
         run_arrive(g0.bar);
         run_arrive(g0.bar_tr);
       }
@@ -396,13 +396,9 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_sp2_run(const Sp2RunArgs g0,
         __syncwarp();
         if (lane == 0) arrive(&tempty[buf]);
       }
-      if (!asked) {  // a CTA without units
-        if (lane == 0) d = decision(k);
-        d = __shfl_sync(0xffffffffu, d, 0);
-      }
       if (d < 0 || (d & 1)) break;
       __syncwarp();  // the slots are the first warp's stores
-      if (eid == 0 && works) run_arrive(g0.bar_tr);
+      if (eid == 0) run_arrive(g0.bar_tr);
     }
   }
   __syncthreads();

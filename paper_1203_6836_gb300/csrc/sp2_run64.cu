@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(kThr) k_sp2_run64(const Sp2Run64Args g) {
   const unsigned G = gridDim.x;
   const int nt = (a.n + T - 1) / T, U = nt * (nt + 1) / 2;
   const unsigned Gw = min(G, (unsigned)U);
-  const bool works = blockIdx.x < Gw;
+  if (blockIdx.x >= Gw) return;  // no units (persist.cuh, grid barrier)
   const int kn = nt * T;  // columns in use; the padding up to it is zero
   auto tile = [&](int u, int* I, int* J) {
     int i = 0;
@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(kThr) k_sp2_run64(const Sp2Run64Args g) {
       }
       put_parts(g.parts[0], u, t1, t2);
     }
-    if (threadIdx.x == 0 && works) run_arrive(g.bar);
+    if (threadIdx.x == 0) run_arrive(g.bar);
   }
   for (int k = 0;; ++k) {
     const double* X = g.F[k & 1];
@@ -131,11 +131,9 @@ __global__ void __launch_bounds__(kThr) k_sp2_run64(const Sp2Run64Args g) {
       }
     };
     const int oi = (threadIdx.x % (T * T)) / T, oj = threadIdx.x % T, kg = threadIdx.x / (T * T);
-    if (works) {
-      tile(blockIdx.x, &I, &J);
-      fetch(0);
-      xrc = __ldcg(X + (size_t)(I * T + oi) * a.ld + J * T + oj);
-    }
+    tile(blockIdx.x, &I, &J);
+    fetch(0);
+    xrc = __ldcg(X + (size_t)(I * T + oi) * a.ld + J * T + oj);
     if (warp == 0) {
       double x = 0.0, y = 0.0;
       for (int i = lane; i < U; i += 32) {
@@ -221,7 +219,7 @@ __global__ void __launch_bounds__(kThr) k_sp2_run64(const Sp2Run64Args g) {
       }
       put_parts(g.parts[(k & 1) ^ 1], u, t1, t2);
     }
-    if (threadIdx.x == 0 && works) run_arrive(g.bar);
+    if (threadIdx.x == 0) run_arrive(g.bar);
   }
   if (threadIdx.x == 0) {
     if (s_abort) atomicExch(&st->err, TB_ERR_TIMEOUT);
