@@ -93,7 +93,9 @@ __global__ void __launch_bounds__(256) k_kick_energy(int N, double* __restrict__
     s_ke[w] = ke;
     s_dq[w] = dq;
   }
-  __syncthreads();
+  // (the cluster's: another block's shared memory may be written once that block has started)
+  if constexpr (CS > 1) cooperative_groups::this_cluster().sync();
+  else __syncthreads();
   if (threadIdx.x == 0) {
     double a = 0.0, b = 0.0;
     for (int k = 0; k < (int)(blockDim.x >> 5); ++k) {
