@@ -1160,6 +1160,7 @@ __global__ void __launch_bounds__(kNumThreads<P>, 1)
         }
         if (symd && c == q) {
           // the 32 x 32 diagonal sub-block: element (l, j) with j < l from lane j
+          __syncwarp();  // every lane is done with what tile_turn_in or tile_store left there
 #pragma unroll
           for (int j = 0; j < 32; ++j) s_sym[q][lane][j] = y[j];
           __syncwarp();
