@@ -71,7 +71,9 @@ Layout make_layout(int n, size_t inner) {
 }
 
 // C = alpha A B + beta E + gamma I (E may be null), n x n row-major; skipped
-// when *skip is set; sym: C is symmetric (its upper tiles, mirrored).  T x T tile per CTA, 256 threads with (T/16)^2 outputs.
+// when *skip is set; sym: C is symmetric (its upper triangle, mirrored: inside a diagonal
+// tile too, where the two halves differ in rounding).  T x T tile per CTA, 256 threads with
+// (T/16)^2 outputs.
 template <int T>
 __global__ void __launch_bounds__(256) k_gemm64(int n, double alpha, const double* __restrict__ A,
                                                 const double* __restrict__ B, double beta,
@@ -118,13 +120,13 @@ __global__ void __launch_bounds__(256) k_gemm64(int n, double alpha, const doubl
 #pragma unroll
     for (int j = 0; j < R; ++j) {
       const int r = row0 + ty + 16 * i, c = col0 + tx + 16 * j;
-      if (r >= n || c >= n) continue;
+      if (r >= n || c >= n || (sym && c < r)) continue;
       const size_t e = (size_t)r * n + c;
       double v = alpha * acc[i][j];
       if (E) v += beta * E[e];
       if (r == c) v += gamma;
       C[e] = v;
-      if (sym && blockIdx.x != blockIdx.y) C[(size_t)c * n + r] = v;
+      if (sym) C[(size_t)c * n + r] = v;
     }
 }
 
@@ -245,9 +247,9 @@ __global__ void __launch_bounds__(kNsThr) k_ns_run(const NsArgs g) {
   };
   auto put = [&](double* C, int I, int J, double v) {
     const int r = I * 16 + oi, c = J * 16 + oj;
-    if (r >= n || c >= n) return;
+    if (r >= n || c >= n || c < r) return;
     C[(size_t)r * n + c] = v;
-    if (I != J) C[(size_t)c * n + r] = v;
+    C[(size_t)c * n + r] = v;
   };
   for (int row = blockIdx.x * (kNsThr / 32) + warp; row < n; row += G * (kNsThr / 32)) row_bound(g.S, n, row, lane, st);
   bool ok = meet();
@@ -278,7 +280,7 @@ __global__ void __launch_bounds__(kNsThr) k_ns_run(const NsArgs g) {
       const bool dg = I == J && oi == oj;
       if (dg) t += 1.5;
       put(g.T, I, J, t);
-      if (I * 16 + oi < n && J * 16 + oj < n) {
+      if (J * 16 + oj < n && I * 16 + oi <= J * 16 + oj) {  // the elements that put() stores
         const unsigned long long b = dev_bits(t, dg);
         m = b > m ? b : m;
       }
