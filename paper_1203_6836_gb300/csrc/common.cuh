@@ -161,6 +161,7 @@ struct SP2State {
   unsigned long long block_products;  // block-sparse path: executed 128^3 block products
   int kc[2];                     // main-phase projection index inside a while graph node
   unsigned bar, pad_[31], bar_tr;  // arrivals at the grid barriers of the single-launch forms (own lines)
+  unsigned left;                   // CTAs of a single-launch form that have finished
 };
 
 // Parameters of a purification step shared by the FP64 and tensor-core kernels.

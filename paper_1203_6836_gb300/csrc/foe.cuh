@@ -34,6 +34,7 @@ struct FoeState {
   int skipd[kFoeMaxM];  // 1: doubling step k returns at once (k < m_max - meff, or done)
   double tr[kFoeMaxMu + 1], trdd[kFoeMaxMu + 1], mus[kFoeMaxMu + 1];
   unsigned bar;  // arrivals at the grid barriers of the single-launch form
+  unsigned left; // its CTAs that have finished
 };
 
 // After an expansion, from Tr E, Tr W and Tr E W: Tr D = n/2 + Tr E,

@@ -415,8 +415,8 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_foe_run(const FoeRunArgs a, 
       }
     }
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0)
-    foe_report(&fs, s_abort ? TB_ERR_TIMEOUT : fs.err, a.n, a.nocc, a.tol, a.mu_out, a.rep);
+  if (threadIdx.x == 0 && run_last(&a.st->left, Gw))
+    foe_report(&fs, *reinterpret_cast<const volatile int*>(err), a.n, a.nocc, a.tol, a.mu_out, a.rep);
   tc_fence_before();
   if (warp == 1) {
     if (elect_one()) {

@@ -42,6 +42,7 @@ struct NonorthState {
   int iters;
   int err;
   unsigned bar;    // grid barrier of k_ns_run
+  unsigned left;   // its CTAs that have finished
   unsigned long long cmax;               // largest row sum of |S|, as bits (which order alike)
   unsigned long long tmax[kMaxNS];       // max |I - T_k| of each iteration, as bits
 };
@@ -315,15 +316,15 @@ __global__ void __launch_bounds__(kNsThr) k_ns_run(const NsArgs g) {
     const int r = I * 16 + oi, q = J * 16 + oj;
     if (r < n && q < n) put(g.T, I, J, f * __ldcg(g.Z[cur] + (size_t)r * n + q));
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    st->done = done;
-    if (g.rep) {
-      g.rep->status = !ok ? TB_ERR_TIMEOUT : done ? TB_OK : TB_ERR_NOT_CONVERGED;
+  if (threadIdx.x == 0) {
+    if (!ok) atomicExch(&st->err, TB_ERR_TIMEOUT);
+    if (run_last(&st->left, G) && g.rep) {
+      const int err = *reinterpret_cast<volatile int*>(&st->err);
+      g.rep->status = err ? err : done ? TB_OK : TB_ERR_NOT_CONVERGED;
       g.rep->ns_iters = it;
       g.rep->ns_residual = res;
     }
   }
-  if (!ok && threadIdx.x == 0) atomicExch(&st->err, TB_ERR_TIMEOUT);
 }
 
 // Y = S / c, Z = I.

@@ -116,6 +116,13 @@ __device__ __forceinline__ bool run_wait(const unsigned* bar, unsigned target, c
     }
   }
 }
+// Whether this CTA is the last of n to leave (one thread, after it has recorded the CTA's
+// error, if any).  It writes the report: whether one of them gave up is known only then.
+__device__ __forceinline__ bool run_last(unsigned* left, unsigned n) {
+  unsigned v;
+  asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(v) : "l"(left) : "memory");
+  return v + 1 == n;
+}
 // Barrier of the 256 epilogue threads; epi_any: the same, true in all of them
 // when `v` is in any.
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }

@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(kThr) k_sp2_run64(const Sp2Run64Args g) {
   }
   if (threadIdx.x == 0) {
     if (s_abort) atomicExch(&st->err, TB_ERR_TIMEOUT);
-    if (blockIdx.x == 0 && g.rep) sp2_fill_report(st, 0, a.n, a.nocc, g.rep);
+    if (run_last(&st->left, Gw) && g.rep) sp2_fill_report(st, 0, a.n, a.nocc, g.rep);
   }
 }
 
