@@ -181,7 +181,9 @@ int tb_ctx_sp2_launch_times(tb_ctx* ctx, int phase, float* ms, int cap, int* cou
  * same up to the order of the FP64 trace sums.  TB_ERR_ARG for max_ctas < 0.
  * tb_ctx_set_wait_limit sets the time limit, in ns of the device's global
  * timer (1 .. 2e9; default 2e9), of the pipeline waits (data and accumulator
- * barriers) of the dense-projection and Fermi-product kernels.  A wait that
+ * barriers) of the dense-projection and Fermi-product kernels.  Where several
+ * products run in one launch, the waits between them (for the other thread
+ * blocks) keep the 2 s.  A wait that
  * runs out makes the kernel stop its pipeline, wait (at the full 2 s limit)
  * for its own copies and MMAs in flight, free its TMEM and return; the call's
  * report then says TB_ERR_TIMEOUT and the context stays usable.  Both apply

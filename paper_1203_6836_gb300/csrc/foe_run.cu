@@ -95,7 +95,9 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_foe_run(const FoeRunArgs a, 
   const RunUnits wu = run_units<BN>(a.ld, (int)G);
   const unsigned Gw = min(G, (unsigned)wu.U);  // the CTAs that arrive at the barriers
   if (blockIdx.x >= Gw) return;                // no units
-  const unsigned long long wl = a.wait_ns ? a.wait_ns : kWaitNs;  // pipeline wait limit
+  // Pipeline wait limit.  A wait that spans the grid barrier (a product's first stage and first
+  // accumulator, what the stores and the patches wait for) is not the pipeline's: kWaitNs.
+  const unsigned long long wl = a.wait_ns ? a.wait_ns : kWaitNs;
   const int nk = a.ld / 32;
   unsigned* bar = &a.st->bar;
   const int* err = &a.st->err;
@@ -174,10 +176,11 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_foe_run(const FoeRunArgs a, 
             tc_fence_after();
             for (int kb = 0; kb < nk; ++kb, ++g) {
               const int s = g % Q::stages;
+              const unsigned long long lim = kb == 0 && u == (int)blockIdx.x ? kWaitNs : wl;
               if (r.patch) {
-                if (!mbar_wait(&conv[s], (cpar >> s) & 1, &s_abort, wl)) break;
+                if (!mbar_wait(&conv[s], (cpar >> s) & 1, &s_abort, lim)) break;
                 cpar ^= 1u << s;
-              } else if (!mbar_wait(&full[s], (g / Q::stages) & 1, &s_abort, wl)) {
+              } else if (!mbar_wait(&full[s], (g / Q::stages) & 1, &s_abort, lim)) {
                 break;
               }
               tc_fence_after();
@@ -200,7 +203,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_foe_run(const FoeRunArgs a, 
           for (int c = 0; c < un.nc; c += 32)
             for (int h = h0; h < h1; ++h)
               if (!ring_store<P, BN>(ring, used, &mp.a[r.out][h], &mp.s[r.out][h], un.I * 128, un.J * 128 + un.c0 + c,
-                                     un.I == un.J ? (un.c0 + c) >> 5 : kOff, &s_abort, wl))
+                                     un.I == un.J ? (un.c0 + c) >> 5 : kOff, &s_abort, kWaitNs))
                 break;
         }
         tma_store_wait();
@@ -221,7 +224,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_foe_run(const FoeRunArgs a, 
           g += mine * nk;
           continue;
         }
-        if (!mbar_wait_warp(&go, gopar, &s_abort, wl)) break;
+        if (!mbar_wait_warp(&go, gopar, &s_abort, kWaitNs)) break;
         gopar ^= 1u;
         for (int u = blockIdx.x; u < wu.U && !s_abort; u += G) {
           const RunUnit un = run_unit<BN>(wu, u);
@@ -303,7 +306,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_foe_run(const FoeRunArgs a, 
             }
           };
           if (r.e >= 0 && r.kind != kZ1) load_e(gr, un.J * 128 + un.c0 + 16 * half);
-          if (!mbar_wait_warp(&tfull[buf], (t_epi >> 1) & 1, &s_abort, wl)) break;
+          if (!mbar_wait_warp(&tfull[buf], (t_epi >> 1) & 1, &s_abort, u == (int)blockIdx.x ? kWaitNs : wl)) break;
           if (r.kind == kZ1) load_e(gr, un.J * 128 + un.c0 + 16 * half);
           tc_fence_after();
 #pragma unroll 1

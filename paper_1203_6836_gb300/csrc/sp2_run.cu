@@ -54,7 +54,9 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_sp2_run(const Sp2RunArgs g0,
   const RunUnits wu = run_units<BN>(a.ld, (int)G);
   const unsigned Gw = min(G, (unsigned)wu.U);  // the CTAs that arrive at the barriers
   if (blockIdx.x >= Gw) return;                // no units
-  const unsigned long long wl = a.wait_ns ? a.wait_ns : kWaitNs;  // pipeline wait limit
+  // Pipeline wait limit.  A wait that spans a grid barrier (a projection's first stage and first
+  // accumulator, the decisions, what the stores wait for) is not the pipeline's: kWaitNs.
+  const unsigned long long wl = a.wait_ns ? a.wait_ns : kWaitNs;
   const int nk = a.ld / 32;
   const int slots = 4 * wu.tiles;
   if (threadIdx.x == 0) {
@@ -105,7 +107,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_sp2_run(const Sp2RunArgs g0,
   };
   // The decision of projection k, by one thread; -1 when the wait gave up.
   auto decision = [&](int k) -> int {
-    if (!mbar_wait(&dec[k & 1], (k >> 1) & 1, &s_abort, wl)) return -1;
+    if (!mbar_wait(&dec[k & 1], (k >> 1) & 1, &s_abort, kWaitNs)) return -1;
     const int d = *reinterpret_cast<volatile int*>(&s_dec[k & 1]);
     arrive(&decfree[k & 1]);
     return d;
@@ -176,7 +178,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_sp2_run(const Sp2RunArgs g0,
           tc_fence_after();
           for (int kb = 0; kb < nk; ++kb, ++g) {
             const int s = g % Q::stages;
-            if (!mbar_wait(&full[s], (g / Q::stages) & 1, &s_abort, wl)) break;
+            if (!mbar_wait(&full[s], (g / Q::stages) & 1, &s_abort, kb == 0 && i == 0 ? kWaitNs : wl)) break;
             tc_fence_after();
             stage_mma<P, BN>(lo0 + s * (Q::stage_bytes >> 4), tmem + buf * BN, id, kb == 0, false);
             umma_commit(&empty[s]);
@@ -205,7 +207,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_sp2_run(const Sp2RunArgs g0,
       int stop = 1;
       if (lane == 0) {
         // the slot of two projections ago has been read by everyone
-        if (k >= 2 && !mbar_wait(&decfree[k & 1], ((k >> 1) - 1) & 1, &s_abort, wl)) ok = false;
+        if (k >= 2 && !mbar_wait(&decfree[k & 1], ((k >> 1) - 1) & 1, &s_abort, kWaitNs)) ok = false;
         int br = 0, capped = 0;
         if (ok && !s_abort) {
           b.k = k;
@@ -248,7 +250,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_sp2_run(const Sp2RunArgs g0,
           for (int c = 0; c < un.nc; c += 32)
             for (int h = 0; h < (Q::C::split ? 3 : 2); ++h)
               if (!ring_store<P, BN>(ring, used, &mp.a[ob][h], &mp.s[ob][h], un.I * 128, un.J * 128 + un.c0 + c,
-                                     un.I == un.J ? kAsIs : kOff, &s_abort, wl))
+                                     un.I == un.J ? kAsIs : kOff, &s_abort, kWaitNs))
                 break;
         }
         tma_store_wait();
@@ -328,7 +330,7 @@ __global__ void __launch_bounds__(kRunThreads, 1) k_sp2_run(const Sp2RunArgs g0,
         const int buf = t & 1;
         const int r0 = un.I * 128, gr = r0 + 32 * q + lane;
         const bool diag = un.I == un.J;
-        const bool ok = mbar_wait_warp(&tfull[buf], (t >> 1) & 1, &s_abort, wl);
+        const bool ok = mbar_wait_warp(&tfull[buf], (t >> 1) & 1, &s_abort, asked ? wl : kWaitNs);
         // X_k (this CTA's own earlier stores, past L1: TMA wrote them), fetched before the
         // branch that may not take it is known
         float xv[16];

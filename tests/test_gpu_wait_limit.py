@@ -47,3 +47,25 @@ def test_a_call_that_says_ok_is_complete(ctx, kind, n):
         tbmd.tb_ctx_set_wait_limit(ctx, 2_000_000_000)
     D, status = call()
     assert status == tbmd.TB_OK and torch.equal(D, D0)
+
+
+def test_the_limit_does_not_count_other_products(ctx):
+    """n = 1500: a product takes about 50 us, its pipeline waits a few.  Warps that take part in
+    some products only wait for several in between; a limit of 100 us is not theirs."""
+    n = 1500
+    H, _ = random_gapped_matrix(n, n // 2, gap=2.0, width=20.0, seed=n)
+    Ht = torch.as_tensor(H, device="cuda")
+    s = FermiSolver(ctx, n, fermi_opts())
+    out = []
+    for limit in (2_000_000_000, 100_000):
+        D = torch.full_like(Ht, float("nan"))
+        s.mu.fill_(float("nan"))
+        tbmd.tb_ctx_set_wait_limit(ctx, limit)
+        try:
+            s(Ht, float(n // 2), 0.3, D)
+            torch.cuda.synchronize()
+        finally:
+            tbmd.tb_ctx_set_wait_limit(ctx, 2_000_000_000)
+        assert fermi_report_to_dict(s.report)["status"] == tbmd.TB_OK, limit
+        out.append(D)
+    assert torch.equal(out[0], out[1])
