@@ -549,7 +549,7 @@ extern "C" int dm_sp2(tb_ctx* ctx, const double* H, int n, double nocc, const tb
     g.bar = &st->bar;
     g.D = D;
     g.rep = rep;
-    return sp2_run64(ctx, g, captured, s);
+    return sp2_run64(ctx, g, s);
   }
   if (!tc) {
     k_init_x<<<g_init, 256, 0, s>>>(H, n, ld, bparts, nb, st, F0, nullptr, slot[0]);

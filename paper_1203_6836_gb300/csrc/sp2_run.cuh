@@ -32,7 +32,7 @@ struct Sp2Run64Args {
   tb_sp2_report* rep;   // device or NULL
 };
 // n <= kSp2Run64Max: the whole FP64 path on `s`.
-int sp2_run64(tb_ctx* ctx, const Sp2Run64Args& g, int captured, cudaStream_t s);
+int sp2_run64(tb_ctx* ctx, const Sp2Run64Args& g, cudaStream_t s);
 
 // The report of a call from its state (one thread); mode 0: FP64 main phase, 1: FP64
 // refinement, 2: FP32 master without refinement.

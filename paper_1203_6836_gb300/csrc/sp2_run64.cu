@@ -228,10 +228,14 @@ __global__ void __launch_bounds__(kThr) k_sp2_run64(const Sp2Run64Args g) {
 }
 
 template <int T>
-int launch(tb_ctx* ctx, const Sp2Run64Args& g, int captured, cudaStream_t s) {
+int launch(tb_ctx* ctx, const Sp2Run64Args& g, cudaStream_t s) {
   const int nt = (g.a.n + T - 1) / T, U = nt * (nt + 1) / 2;
-  // captured steps run beside those of other trajectories: half the chip at most
-  const int G = std::min(U, tb_persistent_grid(ctx, captured ? ctx->sm_count / 2 : 1 << 30));
+  // The whole chip, also under capture: three of these blocks fit an SM, so chains of several
+  // captured steps run side by side.  (Held to half the chip, as the chains that fill an SM's
+  // shared memory are, a captured call of n = 192 took 460 us for its 78 units on 76 blocks,
+  // 258 on the whole chip, 326 launched; n = 512 4.10 ms, 2.38, 4.03.  Four such calls at once,
+  // us a call: n = 192 197 / 144 / 206, n = 512 1913 / 2189 / 3765.)
+  const int G = std::min(U, tb_persistent_grid(ctx, 1 << 30));
   static RunFits fits;
   int ran = 0, c = 1;
   if (G <= 16) {
@@ -245,6 +249,6 @@ int launch(tb_ctx* ctx, const Sp2Run64Args& g, int captured, cudaStream_t s) {
 
 }  // namespace
 
-int sp2_run64(tb_ctx* ctx, const Sp2Run64Args& g, int captured, cudaStream_t s) {
-  return g.a.n <= 136 ? launch<8>(ctx, g, captured, s) : launch<16>(ctx, g, captured, s);
+int sp2_run64(tb_ctx* ctx, const Sp2Run64Args& g, cudaStream_t s) {
+  return g.a.n <= 136 ? launch<8>(ctx, g, s) : launch<16>(ctx, g, s);
 }
