@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(256) k_init_x(const double* __restrict__ H, in
 // T x T output tile per CTA, 16 x 16 threads, (T/16)^2 outputs per thread.
 template <int T>
 __global__ void __launch_bounds__(256) k_sp2_step_f64(const SP2StepArgs a_in, const double* __restrict__ X,
-                                                      double* __restrict__ Y) {
+                                                      double* __restrict__ Y, int half) {
   constexpr int R = T / 16;
   __shared__ double As[kF64K][T + 1];
   __shared__ double Bs[kF64K][T + 1];
@@ -279,14 +279,13 @@ __global__ void __launch_bounds__(256) k_sp2_step_f64(const SP2StepArgs a_in, co
   if (stop) return;
 
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  // upper-triangle tiles only, mirrored: X is symmetric (the FP64 pipe bounds this
-  // kernel, so the half that is left out is half its time)
+  // half: upper-triangle tiles only, mirrored (X is symmetric)
   double* const part = a.parts_out + 3 * (blockIdx.y * gridDim.x + blockIdx.x);
-  if (blockIdx.x < blockIdx.y) {
+  if (half && blockIdx.x < blockIdx.y) {
     if (threadIdx.x < 3) part[threadIdx.x] = 0.0;
     return;
   }
-  const bool mirror = blockIdx.x != blockIdx.y;
+  const bool mirror = half && blockIdx.x != blockIdx.y;
   const double w = mirror ? 2.0 : 1.0;  // the transposed tile counts too
   const int row0 = blockIdx.y * T, col0 = blockIdx.x * T;
   const int ld = a.ld;
@@ -336,9 +335,13 @@ __global__ void __launch_bounds__(256) k_sp2_step_f64(const SP2StepArgs a_in, co
   block_sum3(t1, w * t2, w * t3, part);
 }
 
-void launch_f64(dim3 g, const SP2StepArgs& a, const double* X, double* Y, cudaStream_t s) {
-  if (f64_tile(a.ld) == 16) k_sp2_step_f64<16><<<g, 256, 0, s>>>(a, X, Y);
-  else k_sp2_step_f64<kF64Tile><<<g, 256, 0, s>>>(a, X, Y);
+// The FP64 pipe bounds a product of many tiles, so the lower ones are left out and mirrored:
+// n = 2048 259 -> 149 ms.  Tiles that all run at once take one tile's time either way, and
+// the mirrored stores would only add to it (n = 513 10.36 -> 10.56 ms, 700 12.62 -> 12.80).
+void launch_f64(const tb_ctx* ctx, dim3 g, const SP2StepArgs& a, const double* X, double* Y, cudaStream_t s) {
+  const int half = (int)(g.x * g.y) > ctx->sm_count;
+  if (f64_tile(a.ld) == 16) k_sp2_step_f64<16><<<g, 256, 0, s>>>(a, X, Y, half);
+  else k_sp2_step_f64<kF64Tile><<<g, 256, 0, s>>>(a, X, Y, half);
 }
 
 // FP32 master (buffer chosen by the main phase's iteration count) -> FP64: the
@@ -557,7 +560,7 @@ extern "C" int dm_sp2(tb_ctx* ctx, const double* H, int n, double nocc, const tb
     const dim3 g(ld / f64_tile(ld), ld / f64_tile(ld));
     const int npf = (int)(g.x * g.y);
     const int rc = main_phase(ctx, a, np_init, npf, slot, s, [&](const SP2StepArgs& b, int k, cudaStream_t q) {
-      launch_f64(g, b, (k & 1) ? F1 : F0, (k & 1) ? F0 : F1, q);
+      launch_f64(ctx, g, b, (k & 1) ? F1 : F0, (k & 1) ? F0 : F1, q);
       TB_LAUNCH_CHECK(ctx);
       return TB_OK;
     });
@@ -653,7 +656,7 @@ extern "C" int dm_sp2(tb_ctx* ctx, const double* H, int n, double nocc, const tb
       if (rc) return rc;
     } else {
       // FP64 FMA projection (or, at k = refine, only the final decision)
-      launch_f64(g, r, Fin, Fout, s);
+      launch_f64(ctx, g, r, Fin, Fout, s);
       TB_LAUNCH_CHECK(ctx);
     }
     tb_prof_mark(ctx, 1, k + 1, s);
