@@ -81,3 +81,28 @@ def test_repeated_calls_agree(ctx, n, prec):
         assert torch.equal(_call(ctx, s, H, 0.3 * n)[0], D0)
     for _ in range(3):
         assert torch.equal(_call(ctx, s, H, 0.3 * n, captured=True)[0], D0)
+
+
+def test_two_chains_share_the_chip(ctx):
+    """Two cooperative grids of 36 CTAs (one tile each), which run at the same time: each call's D
+    is the one it has alone."""
+    sizes = (900, 1000)
+    Hs = [_gapless(n, n + 2) for n in sizes]
+    sol = [FermiSolver(ctx, n, fermi_opts()) for n in sizes]
+    D0 = [_call(ctx, s, H, 0.3 * n, 60)[0] for s, H, n in zip(sol, Hs, sizes)]
+    Ds = [torch.full_like(H, float("nan")) for H in Hs]
+    streams = [torch.cuda.Stream() for _ in sizes]
+    torch.cuda.synchronize()
+    tbmd.tb_ctx_set_grid_limit(ctx, 60)
+    try:
+        for _ in range(10):
+            for s, H, D, n, st in zip(sol, Hs, Ds, sizes, streams):
+                with torch.cuda.stream(st):
+                    s.mu.fill_(float("nan"))
+                s(H, 0.3 * n, KT, D, stream=st)
+        torch.cuda.synchronize()
+    finally:
+        tbmd.tb_ctx_set_grid_limit(ctx, 0)
+    for s, D, R in zip(sol, Ds, D0):
+        assert fermi_report_to_dict(s.report)["status"] == tbmd.TB_OK
+        assert torch.equal(D, R)
