@@ -158,7 +158,8 @@ const char* tb_status_string(int status);
 const char* tb_ctx_last_error(const tb_ctx* ctx);
 
 /* Launch timing (measurement support, no counterpart in the paper).  With
- * profiling on, dm_sp2 records CUDA events on its stream between the
+ * profiling on, dm_sp2 runs a launch per projection also where it otherwise
+ * runs them in one, and records CUDA events on its stream between the
  * purification launches of its main phase (phase 0) and of its FP64
  * refinement (phase 1).  tb_ctx_sp2_launch_times waits for the last event
  * and writes the duration (ms) of each launch of the last dm_sp2 call into
@@ -208,9 +209,10 @@ int tb_ctx_set_wait_limit(tb_ctx* ctx, unsigned long long ns);
 #define TB_SP2_FORM_PAIRS 2
 int tb_ctx_set_sp2_form(tb_ctx* ctx, int form);
 /* The form (TB_SP2_FORM_SINGLE or TB_SP2_FORM_PAIRS) and the CTAs of the
- * persistent grid of the dense tensor-core projection dm_sp2 launches for
- * size n under the context's current settings (host only; queries the
- * device's cluster occupancy once).  TB_ERR_ARG for n < 1 or a null pointer. */
+ * persistent grid of the dense tensor-core projection kernel for size n under
+ * the context's current settings (host only; queries the device's cluster
+ * occupancy once).  Where the single form runs all projections in one launch
+ * (tf32, tf32x3), that launch has a grid of its own.  TB_ERR_ARG for n < 1 or a null pointer. */
 int tb_ctx_sp2_form_of(tb_ctx* ctx, int n, int* form, int* ctas);
 
 /* ----------------------------------------------------------- a1: H[n] build */

@@ -23,8 +23,8 @@
 //           blocks are listed in (band of 8 block rows, column, row) order;
 //   numeric  a persistent tcgen05 kernel walks that list: TMA loads the (I,K)
 //           and (J,K) tiles of every pair into shared memory (tf32x3: the FP32
-//           blocks, split into hi and lo there by four converter warps; other
-//           precisions: their stored splits), the MMA accumulates in TMEM
+//           blocks, split into hi and lo by eight converter warps, A into TMEM and B in
+//           place; other precisions: their stored splits), the MMA accumulates in TMEM
 //           (double-buffered between blocks), the epilogue applies the branch
 //           (X^2 or 2X - X^2), zeroes every 32 x 32 sub-block with ||.||_F <
 //           tau (one warp owns a 32-row band, so a sub-block norm is a warp

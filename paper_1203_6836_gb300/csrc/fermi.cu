@@ -123,8 +123,8 @@ __global__ void __launch_bounds__(256) k_foe_x0(const double* __restrict__ H, in
   }
 }
 
-// After an expansion: Tr E and ||E||_F^2 from the last product's partials
-// give Tr D = n/2 + Tr E and Tr D(I - D) = n/4 - ||E||_F^2; then the stop
+// After an expansion: Tr E, Tr W and Tr E W from the products' partials give
+// Tr D = n/2 + Tr E, Tr D(I - D) and Tr D(I - D)(I - 2D) (foe_mu_step); then the stop
 // test and the next mu (one block, every quantity FP64).  The expansion index
 // is the device count st->iters.  Inside a while graph node (cond != 0) the
 // condition is cleared on every stop: converged, capped, or an error flag
@@ -312,8 +312,8 @@ extern "C" int dm_fermi(tb_ctx* ctx, const double* H, int n, double nocc, double
   k_foe_bounds<<<1, 32, 0, s>>>(bparts, (n + 7) / 8, st, mu, kT, m);
   TB_LAUNCH_CHECK(ctx);
 
-  // tf32 and tf32x3: the whole expansion loop in one launch; a captured call whose matrix is too
-  // large for one cluster instead takes the launched form below, whose
+  // tf32 and tf32x3: the whole expansion loop in one launch; a captured call whose tiles are
+  // more than half the chip's SMs instead takes the launched form below, whose
   // chemical-potential loop is a while graph node
   {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;

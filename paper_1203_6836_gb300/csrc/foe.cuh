@@ -123,5 +123,5 @@ struct FoeRunArgs {
   unsigned long long wait_ns;
 };
 // Launches it on `s` and sets *ran, or leaves *ran 0 where the launched form
-// is to be used (a captured call of a size that one cluster does not hold).
+// is to be used (other precisions, a captured call of more tiles than half the SMs).
 int foe_run(tb_ctx* ctx, int precision, const FoeRunArgs& a, int captured, int* ran, cudaStream_t s);

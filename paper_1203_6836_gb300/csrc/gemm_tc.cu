@@ -724,9 +724,9 @@ int pair_capacity(tb_ctx* ctx) {
 // Per-SM throughput of the pair form relative to the single-CTA form, used to choose between
 // them.  tf32x3 projections, single CTAs (sp2_run.cu) against pairs, us: n = 2048 53 / 90,
 // 2816 127 / 114, 3072 138 / 167, 3328 191 / 178, 3584 222 / 192, 4096 305 / 262, 6144 934 / 752:
-// the rule takes the faster at each.  It does not know that sp2_run.cu cuts its last round into
-// quarters: at 2304 (78 / 97) and 2560 (103 / 107) it takes pairs, which the launched and the
-// captured forms are better served by.
+// the rule takes the faster of these.  At 2304 (78 / 97) and 2560 (103 / 107) it takes the slower
+// one: it counts the launched kernel's last round, cut into halves, where sp2_run.cu cuts its
+// own into quarters.
 constexpr double kPairGain = 1.45;
 
 int sp2_tc_pairs(tb_ctx* ctx, int ld) {

@@ -8,8 +8,9 @@
 // in arrival order while the sum of the admitted footprints stays within the
 // budget; the rest wait and are admitted when a retired trajectory frees its
 // memory.  Admission runs the initial SCF (xlbomd_init) and captures one step
-// into a CUDA graph (the chemical-potential loop of dm_fermi becomes a while
-// node), so a step request costs one graph launch.
+// into a CUDA graph (the chemical-potential loop of dm_fermi is inside its one
+// kernel, or a while node where that kernel would take more than half the chip),
+// so a step request costs one graph launch.
 //
 // Requests are served in submission order, at most one step in flight per
 // trajectory (its next step needs the previous one), on up to max_slots

@@ -8,8 +8,8 @@
 //
 // Device-side control: the projections run in one launch (sp2_run.cu, sp2_run64.cu: a grid
 // barrier between them, nothing after the stop) where that is the faster form: FP64 up to
-// n = 512, tf32 and tf32x3 below ld = 4096 or where CTA pairs do not pay.  Otherwise (and while
-// projections are being timed) step kernel k first reduces, in a fixed order, the trace
+// n = 512, tf32 and tf32x3 where CTA pairs are not taken (sp2_tc_pairs) and a captured call fits
+// half the chip.  Otherwise (and while projections are being timed) step kernel k first reduces, in a fixed order, the trace
 // partials written by the epilogue of kernel k-1, takes the stop/branch decision
 // (identical in every CTA) and either returns at once or computes X_{k+1}: launched
 // eagerly, the host enqueues max_iter + 1 step kernels; captured into a CUDA graph, the

@@ -2,7 +2,7 @@
 // projection and the stop/branch decisions run in one persistent grid, the
 // projections separated by a grid barrier (persist.cuh).
 //
-// What bounds the launched form below n = 4096: a projection of a 600 x 600 matrix is
+// What bounds the launched form of small matrices: a projection of a 600 x 600 matrix is
 // a few microseconds of work on 15 CTAs, each launch costs about as much again, and
 // the host enqueues max_iter + 1 (100) launches, most of which return at once: 1.3 ms
 // for 16 projections.  Here nothing runs after the stop, a small matrix is spread
