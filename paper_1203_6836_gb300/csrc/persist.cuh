@@ -338,7 +338,10 @@ __device__ __forceinline__ bool ring_store(const StageRing& r, int& used, const 
 // launch.  Captured steps run beside those of other trajectories, where a grid
 // that waits for the whole chip would hold them up: they take one cluster, a
 // cooperative grid of at most half the chip (one CTA a tile), or (false) the
-// launched form.
+// launched form.  So do products of more than kRunSteps 128 x 128 x 32 steps a CTA (0.2 s
+// at 0.8 us each: from ld = 33 000 on the whole chip): the waits between products last a whole
+// one and give up after 2 s, and a launch is nothing beside it.
+constexpr long long kRunSteps = 250000;
 struct RunShape {
   int bn, grid, cluster;
 };
@@ -358,7 +361,7 @@ inline bool tb_run_shape(const tb_ctx* ctx, int ld, int captured, RunShape* r) {
     while (c < r->grid && 2 * c <= most) c *= 2;
     r->grid = c;
   }
-  return true;
+  return (long long)((T + r->grid - 1) / r->grid) * (ld / 32) <= kRunSteps;
 }
 
 // Whether a cluster of 1, 2, .. 16 CTAs of one kernel fits a device: 0 not asked
